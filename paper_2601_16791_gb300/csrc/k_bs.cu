@@ -2032,7 +2032,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_step_persist(Dev d, long long s
   __syncwarp();
   if (!grid_sync(d.gbar, spin, d.status)) return;
   for (int t = next_tile(ctr + 2); t < d.ntiles; t = next_tile(ctr + 2))
-    jump_kick_tile<2, true>(d, 0.5, 0.5, t, reinterpret_cast<double*>(dsm_p));
+    jump_kick_tile<2, true, true>(d, 0.5, 0.5, t, reinterpret_cast<double*>(dsm_p));
 }
 
 static size_t persist_smem_bytes(const Dev& d) {

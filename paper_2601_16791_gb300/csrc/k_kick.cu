@@ -20,11 +20,11 @@ __global__ void __launch_bounds__(kThreads) k_prep(Dev d, double jump_frac, int 
 
 // One block per tile (register use capped at 80: three resident blocks of
 // 256 threads; see jump_kick_tile).
-template <int NKICK, bool FUSED>
-__global__ void __launch_bounds__(kThreads, 3) k_jump_kick(Dev d, double jump_frac,
-                                                          double kick_frac) {
-  extern __shared__ double dsm[];
-  jump_kick_tile<NKICK, FUSED>(d, jump_frac, kick_frac, blockIdx.x, dsm);
+template <int NKICK, bool FUSED, bool SPLIT>
+__global__ void __launch_bounds__(kThreads, SPLIT ? 2 : 3) k_jump_kick(Dev d, double jump_frac,
+                                                                      double kick_frac) {
+  extern __shared__ __align__(16) double dsm[];
+  jump_kick_tile<NKICK, FUSED, SPLIT>(d, jump_frac, kick_frac, blockIdx.x, dsm);
 }
 
 // Kick acceleration (gravity + drag) without changing the state: 3 x N.
@@ -80,20 +80,23 @@ void launch_prep(const Dev& d, double jump_frac, int nkick, cudaStream_t st) {
 void launch_jump_kick(const Dev& d, double jump_frac, double kick_frac, int nkick,
                       cudaStream_t st) {
   const size_t sm = kick_smem_bytes(d, false);
-  if (nkick == 2) k_jump_kick<2, false><<<d.ntiles, d.tile, sm, st>>>(d, jump_frac, kick_frac);
-  else k_jump_kick<1, false><<<d.ntiles, d.tile, sm, st>>>(d, jump_frac, kick_frac);
+  const bool split = split_gravity(d.big_max);
+  auto* k = nkick == 2 ? (split ? k_jump_kick<2, false, true> : k_jump_kick<2, false, false>)
+                       : (split ? k_jump_kick<1, false, true> : k_jump_kick<1, false, false>);
+  k<<<d.ntiles, d.tile, sm, st>>>(d, jump_frac, kick_frac);
 }
 
 // The interior steps' kick with its own prep (no k_prep launch before it):
 // jump 1/2, two half kicks; for forward runs without growth tracks or k
 // branches recorded or replayed.
 void launch_jump_kick_fused(const Dev& d, cudaStream_t st) {
-  k_jump_kick<2, true><<<d.ntiles, d.tile, kick_smem_bytes(d, true), st>>>(d, 0.5, 0.5);
+  auto* k = split_gravity(d.big_max) ? k_jump_kick<2, true, true> : k_jump_kick<2, true, false>;
+  k<<<d.ntiles, d.tile, kick_smem_bytes(d, true), st>>>(d, 0.5, 0.5);
 }
 
 void launch_accel(const Dev& d, double* acc, int drag_only, int acc_stride, int acc_base,
                   cudaStream_t st) {
-  k_accel<<<d.ntiles, d.tile, kick_smem_bytes(d, false), st>>>(d, acc, drag_only, acc_stride,
+  k_accel<<<d.ntiles, d.tile, stage_bytes(d.big_max), st>>>(d, acc, drag_only, acc_stride,
                                                               acc_base);
 }
 
@@ -103,9 +106,10 @@ void launch_accel(const Dev& d, double* acc, int drag_only, int acc_stride, int 
 void configure_kick() {
   const int c = cudaSharedmemCarveoutMaxShared;
   cudaFuncSetAttribute(k_prep, cudaFuncAttributePreferredSharedMemoryCarveout, c);
-  cudaFuncSetAttribute(k_jump_kick<1, false>, cudaFuncAttributePreferredSharedMemoryCarveout, c);
-  cudaFuncSetAttribute(k_jump_kick<2, false>, cudaFuncAttributePreferredSharedMemoryCarveout, c);
-  cudaFuncSetAttribute(k_jump_kick<2, true>, cudaFuncAttributePreferredSharedMemoryCarveout, c);
+  for (auto* k : {k_jump_kick<1, false, false>, k_jump_kick<2, false, false>,
+                  k_jump_kick<2, true, false>, k_jump_kick<1, false, true>,
+                  k_jump_kick<2, false, true>, k_jump_kick<2, true, true>})
+    cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, c);
 }
 
 }  // namespace mx

@@ -578,6 +578,7 @@ mx_status set_tiling(mx_system* s, int tile, int order) {
 // the same order and the pair keys are sorted).  Choices are kept in a
 // small JSON file ($MX_AUTOTUNE_CACHE, else ~/.cache/mx/autotune.json);
 // MX_AUTOTUNE=0 keeps the defaults.
+constexpr const char* kTuneTag = "split";
 std::string tune_key(const mx_system* s) {
   cudaDeviceProp prop;
   cudaGetDeviceProperties(&prop, s->device);
@@ -585,7 +586,8 @@ std::string tune_key(const mx_system* s) {
   bool gas = false;
   for (auto& p : s->params) gas |= (p.gas.enabled != 0);
   char buf[256];
-  std::snprintf(buf, sizeof(buf), "%s/%d|nsys%d|N%d|NB%d|gas%d", prop.name, prop.multiProcessorCount,
+  // kTuneTag: the kernels the choice was timed on (a cache file outlives a build)
+  std::snprintf(buf, sizeof(buf), "%s|%s/%d|nsys%d|N%d|NB%d|gas%d", kTuneTag, prop.name, prop.multiProcessorCount,
                 bucket(s->params.size()), bucket(s->N), bucket(s->NB), gas ? 1 : 0);
   return buf;
 }

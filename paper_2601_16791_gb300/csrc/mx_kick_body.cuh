@@ -5,6 +5,7 @@
 #include "mx_common.cuh"
 #include "mx_growth.cuh"
 #include "mx_physics.cuh"
+#include "mx_split.cuh"
 
 namespace mx {
 
@@ -65,6 +66,93 @@ __device__ __forceinline__ void gravity_all(const Dev& d, const SysDev& S, BigSm
         pair_acc(x - sb.x[k], y - sb.y[k], z - sb.z[k], sb.mu[k], rc * rc, 0.01 * (rc * rc),
                  0.1 * rc, 1.0 / (0.9 * rc), ax, ay, az);
       }
+    }
+  }
+}
+
+// Systems with more big bodies than can defer planetesimals sum the kick's
+// gravity in FP32 pairs (mx_split.cuh).  With few big bodies the pair sum is a
+// small part of the kick, and the catch-up of deferred planetesimals repeats
+// it term by term.
+__host__ __device__ __forceinline__ bool split_gravity(int nbig) { return nbig > kDeferMaxBig; }
+
+// Bytes of the FP64 staging (nine arrays of doubles), rounded up for the
+// SplitBig records behind it.
+__host__ __device__ __forceinline__ size_t stage_bytes(int big_max) {
+  return (9 * sizeof(double) * (size_t)big_chunk(big_max) + 15) & ~(size_t)15;
+}
+
+// gravity_all with far pairs in FP32 pairs; pairs inside the changeover shell
+// and targets off the positions' grid go through the FP64 pair_acc.  Every
+// thread of the block must call it.
+__device__ __forceinline__ void gravity_split(const Dev& d, const SysDev& S, BigSmem& sb,
+                                              bool act, int jl, double rcj, double x, double y,
+                                              double z, double& ax, double& ay, double& az,
+                                              const double* dj) {
+  __shared__ int s_hi;
+  SplitBig* sp = reinterpret_cast<SplitBig*>(reinterpret_cast<unsigned char*>(sb.x) +
+                                             stage_bytes(d.big_max));
+  const bool jbig = jl < S.nbig;
+  const float near_own = jbig ? near2_of(rcj * rcj) : 0.0f;
+  SplitPos t{};
+  int kt = INT_MIN;   // the grid t was cut on
+  for (int c0 = 0; c0 < S.nbig; c0 += sb.chunk) {
+    const int cn = min(sb.chunk, S.nbig - c0);
+    __syncthreads();
+    stage_bigs(d, S, c0, cn, sb, dj);
+    if (threadIdx.x == 0) s_hi = 0;
+    __syncthreads();
+    int hi = 0;
+    for (int k = threadIdx.x; k < cn; k += blockDim.x)
+      hi = max(hi, max(abs_hi(sb.x[k]), max(abs_hi(sb.y[k]), abs_hi(sb.z[k]))));
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    if ((threadIdx.x & 31) == 0) atomicMax(&s_hi, hi);
+    __syncthreads();
+    const int kg = split_k(s_hi);
+    const bool grid = kg <= kSplitMaxK;
+    if (grid)
+      for (int k = threadIdx.x; k < cn; k += blockDim.x) {
+        SplitBig b;
+        split3(sb.x[k], kg, b.x0, b.x1, b.x2);
+        split3(sb.y[k], kg, b.y0, b.y1, b.y2);
+        split3(sb.z[k], kg, b.z0, b.z1, b.z2);
+        b.muh = (float)sb.mu[k];
+        b.mul = (float)(sb.mu[k] - (double)b.muh);
+        b.near2 = near2_of(sb.rc2[k]);
+        sp[k] = b;
+      }
+    __syncthreads();
+    if (!act) continue;
+    auto pair64 = [&](int k) {
+      if (jbig) {
+        if (c0 + k == jl) return;
+        const double rc = fmax(sb.rc[k], rcj);
+        pair_acc(x - sb.x[k], y - sb.y[k], z - sb.z[k], sb.mu[k], rc * rc, 0.01 * (rc * rc),
+                 0.1 * rc, 1.0 / (0.9 * rc), ax, ay, az);
+      } else {
+        pair_acc(x - sb.x[k], y - sb.y[k], z - sb.z[k], sb.mu[k], sb.rc2[k], sb.rc2lo[k],
+                 sb.rc01[k], sb.i09rc[k], ax, ay, az);
+      }
+    };
+    if (!grid || !split_in_range(x, y, z, kg)) {
+#pragma unroll 1
+      for (int k = 0; k < cn; ++k) pair64(k);
+      continue;
+    }
+    if (kt != kg) {
+      kt = kg;
+      split3(x, kg, t.x0, t.x1, t.x2);
+      split3(y, kg, t.y0, t.y1, t.y2);
+      split3(z, kg, t.z0, t.z1, t.z2);
+    }
+#pragma unroll 1
+    for (int k0 = 0; k0 < cn; k0 += kSplitRun) {
+      const int kn = min(cn, k0 + kSplitRun);
+      SplitAcc acc{};
+#pragma unroll 2
+      for (int k = k0; k < kn; ++k)
+        if (!split_pair(t, sp[k], fmaxf(sp[k].near2, near_own), acc)) pair64(k);
+      split_flush(acc, ax, ay, az);
     }
   }
 }
@@ -308,7 +396,8 @@ __device__ __forceinline__ FusedPrep fused_prep(const Dev& d, const SysDev& S, c
 // registers set residency, and the extra warps outweigh the few spills
 // (measured on the gas disk and the semi-active disk).  `bid` is the tile,
 // `dsm` the block's dynamic shared memory (kick_smem_bytes).
-template <int NKICK, bool FUSED>
+// SPLIT: the gravity of systems that split_gravity names in FP32 pairs.
+template <int NKICK, bool FUSED, bool SPLIT>
 __device__ __forceinline__ void jump_kick_tile(const Dev& d, double jump_frac, double kick_frac,
                                                int bid, double* dsm) {
   BigSmem sb(dsm, big_chunk(d.big_max));
@@ -347,7 +436,10 @@ __device__ __forceinline__ void jump_kick_tile(const Dev& d, double jump_frac, d
     if (jl < S.nbig) rcj = d.brc[S.boff + jl];
   }
   double ax = 0, ay = 0, az = 0;
-  gravity_all(d, S, sb, act, jl, rcj, x, y, z, ax, ay, az, FUSED ? dj : nullptr);
+  if (SPLIT && split_gravity(S.nbig))
+    gravity_split(d, S, sb, act, jl, rcj, x, y, z, ax, ay, az, FUSED ? dj : nullptr);
+  else
+    gravity_all(d, S, sb, act, jl, rcj, x, y, z, ax, ay, az, FUSED ? dj : nullptr);
   if (!act) return;
   const bool big = jl < S.nbig;
   if (__double_as_longlong(jump_frac) != 0 && !(FUSED && big)) {   // jump_frac is +0 or 1/2
@@ -404,13 +496,15 @@ __device__ __forceinline__ void jump_kick_tile(const Dev& d, double jump_frac, d
     atomicOr(d.status, ST_NONFINITE);
 }
 
-// Dynamic shared memory of a kick: the big bodies' staging, and for a fused
+// Dynamic shared memory of a kick: the big bodies' staging (and their FP32
+// parts behind it, where a system's gravity takes them), and for a fused
 // kick with more than 32 big bodies the momentum tree (in the same space,
 // before the staging).
 __host__ __device__ __forceinline__ size_t kick_smem_bytes(const Dev& d, bool fused) {
-  size_t n = 9 * (size_t)big_chunk(d.big_max);
-  if (fused && d.big_max > 32 && n < 3 * (size_t)kThreads) n = 3 * (size_t)kThreads;
-  return n * sizeof(double);
+  size_t n = stage_bytes(d.big_max);
+  if (split_gravity(d.big_max)) n += sizeof(SplitBig) * (size_t)big_chunk(d.big_max);
+  if (fused && d.big_max > 32) n = n < 3 * kThreads * sizeof(double) ? 3 * kThreads * sizeof(double) : n;
+  return n;
 }
 
 }  // namespace mx

@@ -1,0 +1,82 @@
+"""The kick's gravity in FP32 pairs (systems with more than 64 big bodies)
+against the FP64 pair sum of mx_accel, at the same positions.
+
+With every velocity zero, the pre-drift velocity of a step is (h/2) a, a the
+acceleration of the first half kick (the momentum is zero, so nothing jumps).
+Bound: a pair's acceleration in FP32 pairs is a chain of about twenty
+roundings of 2^-48 and smaller, 20 x 2^-48 = 7e-14, times 1.5 for the power
+-3/2 and twice for their spread: 2e-13 of the sum of the pairs' magnitudes.
+"""
+import numpy as np
+import pytest
+
+from paper_2601_16791_gb300 import mx, workloads as W
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+TOL = 2e-13
+
+
+def place(w, far, shell):
+    """Positions of the workload at rest: every 7th planetesimal moved
+    off the positions' grid, every 5th close to a big body."""
+    x = w.xv_helio.copy()
+    x[3:] = 0.0
+    nb = w.nbig
+    rng = np.random.default_rng(11)
+    if shell:
+        for j in range(nb, w.n, 5):
+            b = rng.integers(nb)
+            d = rng.normal(size=3)
+            r = np.linalg.norm(x[:3, b])
+            rc = 3.0 * r * (w.m_big[b] / 3.0) ** (1 / 3)
+            x[:3, j] = x[:3, b] + d / np.linalg.norm(d) * rc * rng.uniform(0.05, 1.3)
+    if far:
+        x[:3, nb + 3::7] *= 50.0
+    return x
+
+
+@pytest.mark.parametrize("nbig,nsmall,scale,far,shell", [
+    (64, 300, 1.0, False, False),      # the FP64 rule
+    (65, 1, 1.0, False, False),
+    (65, 1000, 1.0, True, True),
+    (96, 333, 0.01, False, True),
+    (256, 500, 1.0, False, True),
+    (257, 1023, 1.0, True, False),     # a second, one-body chunk
+    (300, 2000, 30.0, False, True),
+    (550, 700, 1.0, True, True),
+    (70, 200, 3000.0, False, False),   # beyond the grid: FP64 throughout
+])
+def test_split_kick_against_fp64(nbig, nsmall, scale, far, shell):
+    w = W.semiactive_2000big_200k(seed=3, nbig=nbig, nsmall=nsmall)
+    w.xv_helio[:3] *= scale            # the disk at another size: orbits and Hill radii follow
+    w.xv_helio[3:] /= np.sqrt(scale)
+    x = place(w, far, shell)
+    w.params["dt"] = 1e-3   # the step itself is not under test: bodies at rest fall together
+    g = mx.System(w)
+    xd = torch.as_tensor(x, dtype=torch.float64, device="cuda").contiguous()
+    mx.mx_set_defer_window(g.h, 0)
+    mx.mx_set_state_device(g.h, xd)
+    acc = torch.empty((3, w.n), dtype=torch.float64, device="cuda")
+    mx.mx_accel(g.h, acc)
+    pre = torch.empty((6, w.n), dtype=torch.float64, device="cuda")
+    mx.mx_step(g.h, 1)
+    mx.mx_predrift_state(g.h, pre)
+    g.close()
+    want = 0.5 * w.params["dt"] * acc.cpu().numpy()
+    got = pre[3:].cpu().numpy()
+    # magnitude of the pairs (their changeover weight left out below 1)
+    d = x[:3, :, None] - x[:3, None, :nbig]
+    s2 = (d * d).sum(0)
+    s2[s2 == 0] = np.inf
+    size = 0.5 * w.params["dt"] * (W.G * w.m_big / s2).sum(1)
+    err = np.linalg.norm(got - want, axis=0) / size
+    assert err.max() <= TOL, err.max()
+    if nbig <= 64 or scale > 1000:
+        assert err.max() <= 4e-16
+    else:
+        assert err.max() > 0.0     # the split path ran
