@@ -1713,54 +1713,123 @@ __device__ void catch_back(const Dev& d, const SysDev& S, int sys, int j, int t,
   const double* BX = d.h_bx + (size_t)t * 3 * d.NB + S.boff;
   const double* hmu = d.h_mu + (size_t)t * d.NB + S.boff;
   const double* hrc = d.h_rc + (size_t)t * d.NB + S.boff;
-  // the pairs' weights on the lanes (lane l: big body c0 + l), then the sum
-  // in ascending order, as the kick's loop makes it (the same bits)
   double ax = 0, ay = 0, az = 0;
   const int lane = threadIdx.x & 31;
-  for (int c0 = 0; c0 < S.nbig; c0 += 32) {
-    const int l = c0 + lane;
-    double f = 0.0, ex = 0.0, ey = 0.0, ez = 0.0;
-    if (l < S.nbig) {
-      const double rc = hrc[l];
-      ex = x - BX[l];
-      ey = y - BX[d.NB + l];
-      ez = z - BX[2 * (size_t)d.NB + l];
-      f = pair_weight(ex, ey, ez, fmax(hmu[l], 0.0), rc * rc, 0.01 * (rc * rc), 0.1 * rc,
-                      (rc > 0.0) ? 1.0 / (0.9 * rc) : 0.0);
-    }
-    const int cn = min(32, S.nbig - c0);
-    for (int k = 0; k < cn; ++k) {
-      const double fk = __shfl_sync(0xffffffffu, f, k);
-      ax = fma(-fk, __shfl_sync(0xffffffffu, ex, k), ax);
-      ay = fma(-fk, __shfl_sync(0xffffffffu, ey, k), ay);
-      az = fma(-fk, __shfl_sync(0xffffffffu, ez, k), az);
-    }
-  }
   const int nk = head ? -hk : hk;
   if (lead) atomicAdd(ops + 1, (unsigned long long)nk);
   const double kick_h = 0.5 * S.h;
   const double hp0 = P2[0] * S.inv_mu0, hp1 = P2[1] * S.inv_mu0, hp2 = P2[2] * S.inv_mu0;
   const double rp = S.gas_on ? d.rp_cm[j] : 0.0, kd = S.gas_on ? d.kdrag[j] : 0.0;
-  GasAt gq = S.gas_on ? gas_at(S, x, y) : GasAt{false, 0.0, 0.0, 0.0};
-  if (S.gas_on && S.grow_on) {   // the slot's gaps, as in k_jump_kick
-    const double* hg = d.h_gap + (size_t)t * 3 * d.NB + S.boff;
-    gq.rho *= gap_factor(hg, hg + d.NB, hg + 2 * (size_t)d.NB, S.nbig, x, y);
-  }
-  if (S.gas_on && S.dg_on) {   // as in k_jump_kick
-    ax += gq.adg[0];
-    ay += gq.adg[1];
-  }
-  const DragConst dc = S.gas_on ? drag_const(S, gq, x, y, hp0, hp1, hp2, rp, kd) : DragConst{};
-  for (int kk = 0; kk < nk; ++kk) {   // as in k_jump_kick
+  if (S.split) {
+    // the pairs' terms on the lanes (lane l: big body c0 + l), then the sum in
+    // ascending order, as the kick's loop makes it (the same bits)
+    SplitAcc acc{};
+    int hi = 0;
+    for (int l = lane; l < S.nbig; l += 32)
+      hi = max(hi, max(abs_hi(BX[l]), max(abs_hi(BX[d.NB + l]), abs_hi(BX[2 * (size_t)d.NB + l]))));
+    const int kg = split_k(__reduce_max_sync(0xffffffffu, hi));
+    const bool far_ok = kg <= kSplitMaxK && split_in_range(x, y, z, kg);
+    SplitPos tp{};
+    if (far_ok) {
+      split3(x, kg, tp.x0, tp.x1, tp.x2);
+      split3(y, kg, tp.y0, tp.y1, tp.y2);
+      split3(z, kg, tp.z0, tp.z1, tp.z2);
+    }
+    for (int c0 = 0; c0 < S.nbig; c0 += 32) {
+      const int l = c0 + lane;
+      double f = 0.0, ex = 0.0, ey = 0.0, ez = 0.0;
+      SplitTerm ft{};
+      bool near = false;
+      if (l < S.nbig) {
+        const double rc = hrc[l];
+        const double bx = BX[l], by = BX[d.NB + l], bz = BX[2 * (size_t)d.NB + l];
+        const double mu = fmax(hmu[l], 0.0);
+        if (far_ok) {
+          const SplitBig b = split_big(bx, by, bz, mu, rc * rc, kg);
+          near = !split_term(tp, b, b.near2, ft);
+        } else {
+          near = true;
+        }
+        if (near) {
+          ex = x - bx;
+          ey = y - by;
+          ez = z - bz;
+          f = pair_weight(ex, ey, ez, mu, rc * rc, 0.01 * (rc * rc), 0.1 * rc,
+                          (rc > 0.0) ? 1.0 / (0.9 * rc) : 0.0);
+        }
+      }
+      const int cn = min(32, S.nbig - c0);
+      const unsigned nearm = __ballot_sync(0xffffffffu, near);
+      for (int k = 0; k < cn; ++k) {
+        if ((nearm >> k) & 1u) {
+          const double fk = __shfl_sync(0xffffffffu, f, k);
+          ax = fma(-fk, __shfl_sync(0xffffffffu, ex, k), ax);
+          ay = fma(-fk, __shfl_sync(0xffffffffu, ey, k), ay);
+          az = fma(-fk, __shfl_sync(0xffffffffu, ez, k), az);
+        } else {
+          SplitTerm fk;
+          fk.xh = __shfl_sync(0xffffffffu, ft.xh, k);
+          fk.xl = __shfl_sync(0xffffffffu, ft.xl, k);
+          fk.yh = __shfl_sync(0xffffffffu, ft.yh, k);
+          fk.yl = __shfl_sync(0xffffffffu, ft.yl, k);
+          fk.zh = __shfl_sync(0xffffffffu, ft.zh, k);
+          fk.zl = __shfl_sync(0xffffffffu, ft.zl, k);
+          split_sum(acc, fk);
+        }
+      }
+      if (far_ok) split_renorm(acc);
+    }
+    DragSplit dc{};
     if (S.gas_on) {
-      int kout = 0;
-      double dvec[3];
-      const double coef = gas_drag_coef(S, dc, u, v, w, dvec, -1, &kout);
-      kick_with_drag(kick_h, ax, ay, az, coef, dvec, u, v, w);
-    } else {
-      u = fma(kick_h, ax, u);
-      v = fma(kick_h, ay, v);
-      w = fma(kick_h, az, w);
+      dc = drag_split(S, x, y, hp0, hp1, hp2, rp, kd);
+      ax += dc.adg[0];
+      ay += dc.adg[1];
+    }
+    split_kicks(S, kick_h, nk, split_gravity(acc, ax, ay, az), S.gas_on != 0, dc, x, y, hp0, hp1, hp2,
+                rp, kd, u, v, w, [](int) { return -1; }, [](int, int) {});
+  } else {
+    // the pairs' weights on the lanes (lane l: big body c0 + l), then the sum
+    // in ascending order, as the kick's loop makes it (the same bits)
+    for (int c0 = 0; c0 < S.nbig; c0 += 32) {
+      const int l = c0 + lane;
+      double f = 0.0, ex = 0.0, ey = 0.0, ez = 0.0;
+      if (l < S.nbig) {
+        const double rc = hrc[l];
+        ex = x - BX[l];
+        ey = y - BX[d.NB + l];
+        ez = z - BX[2 * (size_t)d.NB + l];
+        f = pair_weight(ex, ey, ez, fmax(hmu[l], 0.0), rc * rc, 0.01 * (rc * rc), 0.1 * rc,
+                        (rc > 0.0) ? 1.0 / (0.9 * rc) : 0.0);
+      }
+      const int cn = min(32, S.nbig - c0);
+      for (int k = 0; k < cn; ++k) {
+        const double fk = __shfl_sync(0xffffffffu, f, k);
+        ax = fma(-fk, __shfl_sync(0xffffffffu, ex, k), ax);
+        ay = fma(-fk, __shfl_sync(0xffffffffu, ey, k), ay);
+        az = fma(-fk, __shfl_sync(0xffffffffu, ez, k), az);
+      }
+    }
+    GasAt gq = S.gas_on ? gas_at(S, x, y) : GasAt{false, 0.0, 0.0, 0.0};
+    if (S.gas_on && S.grow_on) {   // the slot's gaps, as in k_jump_kick
+      const double* hg = d.h_gap + (size_t)t * 3 * d.NB + S.boff;
+      gq.rho *= gap_factor(hg, hg + d.NB, hg + 2 * (size_t)d.NB, S.nbig, x, y);
+    }
+    if (S.gas_on && S.dg_on) {   // as in k_jump_kick
+      ax += gq.adg[0];
+      ay += gq.adg[1];
+    }
+    const DragConst dc = S.gas_on ? drag_const(S, gq, x, y, hp0, hp1, hp2, rp, kd) : DragConst{};
+    for (int kk = 0; kk < nk; ++kk) {   // as in k_jump_kick
+      if (S.gas_on) {
+        int kout = 0;
+        double dvec[3];
+        const double coef = gas_drag_coef(S, dc, u, v, w, dvec, -1, &kout);
+        kick_with_drag(kick_h, ax, ay, az, coef, dvec, u, v, w);
+      } else {
+        u = fma(kick_h, ax, u);
+        v = fma(kick_h, ay, v);
+        w = fma(kick_h, az, w);
+      }
     }
   }
   if (!(finite_d(x) && finite_d(y) && finite_d(z) && finite_d(u) && finite_d(v) && finite_d(w)) &&
@@ -2032,7 +2101,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_step_persist(Dev d, long long s
   __syncwarp();
   if (!grid_sync(d.gbar, spin, d.status)) return;
   for (int t = next_tile(ctr + 2); t < d.ntiles; t = next_tile(ctr + 2))
-    jump_kick_tile<2, true, true>(d, 0.5, 0.5, t, reinterpret_cast<double*>(dsm_p));
+    jump_kick_tile<2, true, kSplitAny>(d, 0.5, 0.5, t, reinterpret_cast<double*>(dsm_p));
 }
 
 static size_t persist_smem_bytes(const Dev& d) {

@@ -18,13 +18,24 @@ __global__ void __launch_bounds__(kThreads) k_prep(Dev d, double jump_frac, int 
   prep_system(d, jump_frac, nkick, blockIdx.x);
 }
 
-// One block per tile (register use capped at 80: three resident blocks of
-// 256 threads; see jump_kick_tile).
-template <int NKICK, bool FUSED, bool SPLIT>
-__global__ void __launch_bounds__(kThreads, SPLIT ? 2 : 3) k_jump_kick(Dev d, double jump_frac,
-                                                                      double kick_frac) {
+// One block per tile.  Register use is capped at 80 (three resident blocks of
+// 256 threads; see jump_kick_tile), where the pair loop is long (kSplitAny) at
+// 128: with few big bodies the FP32-pair kick is bound by the FP64 left in it
+// and gains from the third block in spite of its spills (4 cores + 100,000
+// bodies: 27 us against 32); with 2,000, the loop is bound by FP32 issue.
+template <int NKICK, bool FUSED, int MODE>
+__global__ void __launch_bounds__(kThreads, MODE == kSplitAny ? 2 : 3)
+    k_jump_kick(Dev d, double jump_frac, double kick_frac) {
   extern __shared__ __align__(16) double dsm[];
-  jump_kick_tile<NKICK, FUSED, SPLIT>(d, jump_frac, kick_frac, blockIdx.x, dsm);
+  jump_kick_tile<NKICK, FUSED, MODE>(d, jump_frac, kick_frac, blockIdx.x, dsm);
+}
+
+using KickKernel = void (*)(Dev, double, double);
+template <int NKICK, bool FUSED>
+KickKernel kick_kernel(int mode) {
+  return mode == kSplitNone  ? k_jump_kick<NKICK, FUSED, kSplitNone>
+         : mode == kSplitFew ? k_jump_kick<NKICK, FUSED, kSplitFew>
+                             : k_jump_kick<NKICK, FUSED, kSplitAny>;
 }
 
 // Kick acceleration (gravity + drag) without changing the state: 3 x N.
@@ -80,9 +91,8 @@ void launch_prep(const Dev& d, double jump_frac, int nkick, cudaStream_t st) {
 void launch_jump_kick(const Dev& d, double jump_frac, double kick_frac, int nkick,
                       cudaStream_t st) {
   const size_t sm = kick_smem_bytes(d, false);
-  const bool split = split_gravity(d.big_max);
-  auto* k = nkick == 2 ? (split ? k_jump_kick<2, false, true> : k_jump_kick<2, false, false>)
-                       : (split ? k_jump_kick<1, false, true> : k_jump_kick<1, false, false>);
+  const KickKernel k =
+      nkick == 2 ? kick_kernel<2, false>(d.split_mode) : kick_kernel<1, false>(d.split_mode);
   k<<<d.ntiles, d.tile, sm, st>>>(d, jump_frac, kick_frac);
 }
 
@@ -90,8 +100,7 @@ void launch_jump_kick(const Dev& d, double jump_frac, double kick_frac, int nkic
 // jump 1/2, two half kicks; for forward runs without growth tracks or k
 // branches recorded or replayed.
 void launch_jump_kick_fused(const Dev& d, cudaStream_t st) {
-  auto* k = split_gravity(d.big_max) ? k_jump_kick<2, true, true> : k_jump_kick<2, true, false>;
-  k<<<d.ntiles, d.tile, kick_smem_bytes(d, true), st>>>(d, 0.5, 0.5);
+  kick_kernel<2, true>(d.split_mode)<<<d.ntiles, d.tile, kick_smem_bytes(d, true), st>>>(d, 0.5, 0.5);
 }
 
 void launch_accel(const Dev& d, double* acc, int drag_only, int acc_stride, int acc_base,
@@ -106,10 +115,9 @@ void launch_accel(const Dev& d, double* acc, int drag_only, int acc_stride, int 
 void configure_kick() {
   const int c = cudaSharedmemCarveoutMaxShared;
   cudaFuncSetAttribute(k_prep, cudaFuncAttributePreferredSharedMemoryCarveout, c);
-  for (auto* k : {k_jump_kick<1, false, false>, k_jump_kick<2, false, false>,
-                  k_jump_kick<2, true, false>, k_jump_kick<1, false, true>,
-                  k_jump_kick<2, false, true>, k_jump_kick<2, true, true>})
-    cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, c);
+  for (int m : {kSplitNone, kSplitFew, kSplitAny})
+    for (KickKernel k : {kick_kernel<1, false>(m), kick_kernel<2, false>(m), kick_kernel<2, true>(m)})
+      cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, c);
 }
 
 }  // namespace mx

@@ -114,6 +114,25 @@ bool valid_params(const mx_params* p) {
          p->pair_cap > 0 && p->pair_cap <= (1 << 26) && p->eject_every >= 0;
 }
 
+// The kick in FP32 pairs (mx_split.cuh) is for systems whose big bodies are at
+// most this fraction of the star: lunar- to Mars-mass embryos (0.04 to 0.3e-6).
+// A planetesimal caught by a core of ten Earth masses passes it many times in a
+// few steps and multiplies last-place differences of its state by up to 1e9
+// (20 steps of the gas disk), so there every rounding of the FP64 kick is kept.
+constexpr double kSplitMaxMass = 1e-6;
+
+int split_mode(const std::vector<mx::SysDev>& sys) {
+  bool all = true, any = false;
+  int big_max = 0;
+  for (auto& y : sys) {
+    all = all && y.split;
+    any = any || y.split;
+    big_max = std::max(big_max, y.nbig);
+  }
+  if (!any) return mx::kSplitNone;
+  return all && big_max <= mx::kDeferMaxBig ? mx::kSplitFew : mx::kSplitAny;
+}
+
 // Per-system constants folded from the parameters.
 mx::SysDev make_sysdev(const mx_params& p, int off, int nbig, int n, int boff) {
   mx::SysDev s;
@@ -187,6 +206,7 @@ struct mx_system {
   cudaEvent_t mk_head[3] = {nullptr, nullptr, nullptr};
   cudaEvent_t mk_step[7] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
   long long step = 0;
+  bool stepped = false;           // a step-taking call was made
   int eject_every = 0;            // ejection test schedule (Sec. 3.5), 0: none
   bool removed_any = false;       // a test outside the schedule removed bodies
   bool grow_any = false;          // some system follows growth tracks (mx_set_growth)
@@ -578,7 +598,7 @@ mx_status set_tiling(mx_system* s, int tile, int order) {
 // the same order and the pair keys are sorted).  Choices are kept in a
 // small JSON file ($MX_AUTOTUNE_CACHE, else ~/.cache/mx/autotune.json);
 // MX_AUTOTUNE=0 keeps the defaults.
-constexpr const char* kTuneTag = "split";
+constexpr const char* kTuneTag = "split2";
 std::string tune_key(const mx_system* s) {
   cudaDeviceProp prop;
   cudaGetDeviceProperties(&prop, s->device);
@@ -587,8 +607,8 @@ std::string tune_key(const mx_system* s) {
   for (auto& p : s->params) gas |= (p.gas.enabled != 0);
   char buf[256];
   // kTuneTag: the kernels the choice was timed on (a cache file outlives a build)
-  std::snprintf(buf, sizeof(buf), "%s|%s/%d|nsys%d|N%d|NB%d|gas%d", kTuneTag, prop.name, prop.multiProcessorCount,
-                bucket(s->params.size()), bucket(s->N), bucket(s->NB), gas ? 1 : 0);
+  std::snprintf(buf, sizeof(buf), "%s|%s/%d|nsys%d|N%d|NB%d|gas%d|split%d", kTuneTag, prop.name, prop.multiProcessorCount,
+                bucket(s->params.size()), bucket(s->N), bucket(s->NB), gas ? 1 : 0, s->d.split_mode);
   return buf;
 }
 
@@ -733,6 +753,9 @@ mx_status build(mx_system* s, const std::vector<const double*>& m_big,
   for (int k = 0; k < nsys; ++k) {
     const int n = s->nbig[k] + s->nsmall[k];
     sys[k] = make_sysdev(s->params[k], off, s->nbig[k], n, boff);
+    double heaviest = 0.0;
+    for (int i = 0; i < s->nbig[k]; ++i) heaviest = std::max(heaviest, m_big[k][i]);
+    sys[k].split = heaviest <= kSplitMaxMass * s->params[k].m_star ? 1 : 0;
     tiles_cap += (n + kMinTile - 1) / kMinTile;
     off += n;
     boff += s->nbig[k];
@@ -837,6 +860,7 @@ mx_status build(mx_system* s, const std::vector<const double*>& m_big,
   d.tile = s->tile;
   d.big_max = 0;
   for (auto& q : sys) d.big_max = std::max(d.big_max, q.nbig);
+  d.split_mode = split_mode(sys);
   d.pair_cap = cap;
   d.work_cap = work_cap;
   d.mem_cap = mem_cap;
@@ -1176,6 +1200,7 @@ mx_status mx_step(mx_system* s, int n_steps) {
     }
   }
   s->step += n_steps;
+  s->stepped = true;
   // a deferred body's drift is the catch-up's; only planetesimals of systems
   // with at most kDeferMaxBig big bodies are ever deferred
   bool deferrable = false;
@@ -1310,6 +1335,7 @@ mx_status profiled_run(mx_system* s, int n_steps, void* flush, size_t flush_byte
     if (launches) launches[k] = cnt[k];
   }
   s->step += n_steps;
+  s->stepped = true;
   return sync_status(s);
 }
 
@@ -1429,6 +1455,7 @@ mx_status timed_graph_run(mx_system* s, int n_steps, void* flush, size_t flush_b
   }
   if (total_ms) *total_ms = tot;
   s->step += n_steps;
+  s->stepped = true;
   return sync_status(s);
 }
 
@@ -1497,6 +1524,7 @@ mx_status mx_step_wall(mx_system* s, int n_steps, void* dev_flush, size_t flush_
   for (auto& q : ev) cudaEventDestroy(q);
   if (e != cudaSuccess) return fail(MX_ERR_CUDA, std::string("wall step: ") + cudaGetErrorString(e));
   s->step += n_steps;
+  s->stepped = true;
   return sync_status(s);
 }
 
@@ -1695,6 +1723,12 @@ mx_status mx_set_growth(mx_system* s, int sys, const mx_growth* g, double gap_c)
   MX_TRY(set_device(s));
   MX_TRY(settle(s));
   mx::SysDev& S = s->h_sys[sys];
+  if (any && S.split) {   // masses change from here on: the FP64 kick, and its tile
+    S.split = 0;
+    MX_CUDA(cudaMemcpyAsync(s->d_sys + sys, &S, sizeof(mx::SysDev), cudaMemcpyHostToDevice, s->st));
+    s->d.split_mode = split_mode(s->h_sys);
+    if (!s->stepped && !s->grow_any) MX_TRY(autotune(s));   // its trials start from a fresh system
+  }
   if (nb > 0)
     MX_CUDA(cudaMemcpyAsync(s->d_grow + S.boff, gr.data(), nb * sizeof(mx::Growth),
                             cudaMemcpyHostToDevice, s->st));
@@ -1978,6 +2012,7 @@ mx_status mx_set_gas_params(mx_system* s, int k, double sigma1, double gamma, do
   p.gas.cd_scale = cd_scale;
   const mx::SysDev old = s->h_sys[k];
   mx::SysDev nw = make_sysdev(p, old.off, old.nbig, old.n, old.boff);
+  nw.split = old.split;
   s->h_sys[k] = nw;
   MX_CUDA(cudaMemcpyAsync(s->d_sys + k, &s->h_sys[k], sizeof(mx::SysDev), cudaMemcpyHostToDevice, s->st));
   MX_CUDA(cudaStreamSynchronize(s->st));

@@ -29,6 +29,9 @@ constexpr int kMaxBigPairs = 512; // big-big encounter pairs handled per step
 // the direct path's order), so with many big bodies a replay costs more than
 // the encounter it moves off the step.
 constexpr int kDeferMaxBig = 64;
+// Kick kernels by the systems' SysDev::split: no system; every system, none
+// with more than kDeferMaxBig big bodies; any mix.
+enum : int { kSplitNone = 0, kSplitFew = 1, kSplitAny = 2 };
 // Status of a body removed from the integration as ejected (Sec. 3.5).
 constexpr signed char kStatEjected = -3;
 
@@ -56,7 +59,8 @@ struct SysDev {
   double inv_G, m_star;
   // gas (Sec. 3.1)
   int gas_on, cd_mode, gamma_one, flare_quarter;
-  int rc_inf, pad0;
+  int rc_inf;
+  int split;      // the kick in FP32 pairs (mx_split.cuh): light big bodies, masses fixed
   double sigma1, gamma, inv_rc, r_in, hr1, flare, cd_scale;
   double c_rho;   // rho_g = c_rho * Sigma * R^-(1+flare)     [g/cm^3]
   double c_cs;    // c_s  = c_cs * R^(flare-1/2)              [AU/d]
@@ -135,6 +139,7 @@ struct Dev {
   int N, NB, nsys, ntiles;
   int tile;        // targets per tile = threads per block of the per-body kernels
   int big_max;     // most big bodies of any system (sizes the kernels' shared staging)
+  int split_mode;  // kick kernel: kSplitNone, kSplitFew or kSplitAny
   int pair_cap, work_cap, mem_cap;
   int kepler_max_iter, bs_max_sub;
   double bs_tol;

@@ -6,6 +6,7 @@
 #include "mx_growth.cuh"
 #include "mx_physics.cuh"
 #include "mx_split.cuh"
+#include "mx_split_gas.cuh"
 
 namespace mx {
 
@@ -70,11 +71,10 @@ __device__ __forceinline__ void gravity_all(const Dev& d, const SysDev& S, BigSm
   }
 }
 
-// Systems with more big bodies than can defer planetesimals sum the kick's
-// gravity in FP32 pairs (mx_split.cuh).  With few big bodies the pair sum is a
-// small part of the kick, and the catch-up of deferred planetesimals repeats
-// it term by term.
-__host__ __device__ __forceinline__ bool split_gravity(int nbig) { return nbig > kDeferMaxBig; }
+// Systems with at most kDeferMaxBig big bodies keep the pair sum in FP32 pairs
+// up to the velocity update (split_kicks), which the catch-up of deferred
+// planetesimals repeats; with more, it goes into FP64 every kSplitRun bodies.
+__host__ __device__ __forceinline__ bool split_flushes(int nbig) { return nbig > kDeferMaxBig; }
 
 // Bytes of the FP64 staging (nine arrays of doubles), rounded up for the
 // SplitBig records behind it.
@@ -82,17 +82,36 @@ __host__ __device__ __forceinline__ size_t stage_bytes(int big_max) {
   return (9 * sizeof(double) * (size_t)big_chunk(big_max) + 15) & ~(size_t)15;
 }
 
-// gravity_all with far pairs in FP32 pairs; pairs inside the changeover shell
-// and targets off the positions' grid go through the FP64 pair_acc.  Every
-// thread of the block must call it.
+// The staged big bodies' parts on the grid of kg, for split_term.
+__device__ __forceinline__ SplitBig split_big(double x, double y, double z, double mu, double rc2,
+                                              int kg) {
+  SplitBig b;
+  split3(x, kg, b.x0, b.x1, b.x2);
+  split3(y, kg, b.y0, b.y1, b.y2);
+  split3(z, kg, b.z0, b.z1, b.z2);
+  const FF m = ff_of(mu);
+  b.muh = m.h;
+  b.mul = m.l;
+  b.near2 = near2_of(rc2);
+  return b;
+}
+
+// Gravity on target j (local index jl, own changeover radius rcj) from all big
+// bodies of its system.  Far pairs are formed in FP32 pairs and summed (sign
+// reversed) in acc, which a system with many big bodies (split_flushes) empties
+// into (ax, ay, az) as it goes; pairs inside the changeover shell, and every
+// pair of a target off the positions' grid, go through the FP64 pair_acc into
+// (ax, ay, az).  Every thread of the block must call it.
+template <bool MANY>
 __device__ __forceinline__ void gravity_split(const Dev& d, const SysDev& S, BigSmem& sb,
                                               bool act, int jl, double rcj, double x, double y,
                                               double z, double& ax, double& ay, double& az,
-                                              const double* dj) {
+                                              SplitAcc& acc, const double* dj) {
   __shared__ int s_hi;
   SplitBig* sp = reinterpret_cast<SplitBig*>(reinterpret_cast<unsigned char*>(sb.x) +
                                              stage_bytes(d.big_max));
   const bool jbig = jl < S.nbig;
+  const bool flush = MANY && split_flushes(S.nbig);
   const float near_own = jbig ? near2_of(rcj * rcj) : 0.0f;
   SplitPos t{};
   int kt = INT_MIN;   // the grid t was cut on
@@ -103,24 +122,23 @@ __device__ __forceinline__ void gravity_split(const Dev& d, const SysDev& S, Big
     if (threadIdx.x == 0) s_hi = 0;
     __syncthreads();
     int hi = 0;
-    for (int k = threadIdx.x; k < cn; k += blockDim.x)
-      hi = max(hi, max(abs_hi(sb.x[k]), max(abs_hi(sb.y[k]), abs_hi(sb.z[k]))));
-    hi = __reduce_max_sync(0xffffffffu, hi);
-    if ((threadIdx.x & 31) == 0) atomicMax(&s_hi, hi);
-    __syncthreads();
-    const int kg = split_k(s_hi);
+    if (cn <= 32) {   // every warp for itself
+      const int k = threadIdx.x & 31;
+      if (k < cn) hi = max(abs_hi(sb.x[k]), max(abs_hi(sb.y[k]), abs_hi(sb.z[k])));
+      hi = __reduce_max_sync(0xffffffffu, hi);
+    } else {
+      for (int k = threadIdx.x; k < cn; k += blockDim.x)
+        hi = max(hi, max(abs_hi(sb.x[k]), max(abs_hi(sb.y[k]), abs_hi(sb.z[k]))));
+      hi = __reduce_max_sync(0xffffffffu, hi);
+      if ((threadIdx.x & 31) == 0) atomicMax(&s_hi, hi);
+      __syncthreads();
+      hi = s_hi;
+    }
+    const int kg = split_k(hi);
     const bool grid = kg <= kSplitMaxK;
     if (grid)
-      for (int k = threadIdx.x; k < cn; k += blockDim.x) {
-        SplitBig b;
-        split3(sb.x[k], kg, b.x0, b.x1, b.x2);
-        split3(sb.y[k], kg, b.y0, b.y1, b.y2);
-        split3(sb.z[k], kg, b.z0, b.z1, b.z2);
-        b.muh = (float)sb.mu[k];
-        b.mul = (float)(sb.mu[k] - (double)b.muh);
-        b.near2 = near2_of(sb.rc2[k]);
-        sp[k] = b;
-      }
+      for (int k = threadIdx.x; k < cn; k += blockDim.x)
+        sp[k] = split_big(sb.x[k], sb.y[k], sb.z[k], sb.mu[k], sb.rc2[k], kg);
     __syncthreads();
     if (!act) continue;
     auto pair64 = [&](int k) {
@@ -148,11 +166,14 @@ __device__ __forceinline__ void gravity_split(const Dev& d, const SysDev& S, Big
 #pragma unroll 1
     for (int k0 = 0; k0 < cn; k0 += kSplitRun) {
       const int kn = min(cn, k0 + kSplitRun);
-      SplitAcc acc{};
 #pragma unroll 2
-      for (int k = k0; k < kn; ++k)
-        if (!split_pair(t, sp[k], fmaxf(sp[k].near2, near_own), acc)) pair64(k);
-      split_flush(acc, ax, ay, az);
+      for (int k = k0; k < kn; ++k) {
+        SplitTerm f;
+        if (split_term(t, sp[k], fmaxf(sp[k].near2, near_own), f)) split_sum(acc, f);
+        else pair64(k);
+      }
+      if (flush) split_flush(acc, ax, ay, az);
+      else split_renorm(acc);
     }
   }
 }
@@ -396,8 +417,10 @@ __device__ __forceinline__ FusedPrep fused_prep(const Dev& d, const SysDev& S, c
 // registers set residency, and the extra warps outweigh the few spills
 // (measured on the gas disk and the semi-active disk).  `bid` is the tile,
 // `dsm` the block's dynamic shared memory (kick_smem_bytes).
-// SPLIT: the gravity of systems that split_gravity names in FP32 pairs.
-template <int NKICK, bool FUSED, bool SPLIT>
+// MODE (kSplitNone, kSplitFew, kSplitAny): which of the two kicks the batch's
+// systems need, FP64 (kick_fp64) or FP32 pairs (kick_split_tile), and whether
+// some system may have more than kDeferMaxBig big bodies.
+template <int NKICK, bool FUSED, int MODE>
 __device__ __forceinline__ void jump_kick_tile(const Dev& d, double jump_frac, double kick_frac,
                                                int bid, double* dsm) {
   BigSmem sb(dsm, big_chunk(d.big_max));
@@ -436,8 +459,11 @@ __device__ __forceinline__ void jump_kick_tile(const Dev& d, double jump_frac, d
     if (jl < S.nbig) rcj = d.brc[S.boff + jl];
   }
   double ax = 0, ay = 0, az = 0;
-  if (SPLIT && split_gravity(S.nbig))
-    gravity_split(d, S, sb, act, jl, rcj, x, y, z, ax, ay, az, FUSED ? dj : nullptr);
+  SplitAcc acc{};
+  const bool split = MODE == kSplitFew || (MODE == kSplitAny && S.split);
+  if (split)
+    gravity_split<MODE == kSplitAny>(d, S, sb, act, jl, rcj, x, y, z, ax, ay, az, acc,
+                                     FUSED ? dj : nullptr);
   else
     gravity_all(d, S, sb, act, jl, rcj, x, y, z, ax, ay, az, FUSED ? dj : nullptr);
   if (!act) return;
@@ -451,30 +477,50 @@ __device__ __forceinline__ void jump_kick_tile(const Dev& d, double jump_frac, d
   const double hp0 = hp[0], hp1 = hp[1], hp2 = hp[2];
   const double rp = drag ? d.rp_cm[j] : 0.0, kd = drag ? d.kdrag[j] : 0.0;
   const int kbase = d.kmode ? d.kick_ctr[1] : 0;
-  // the gas at the (fixed) position, shared by the launch's half kicks
-  GasAt gq = drag ? gas_at(S, x, y) : GasAt{false, 0.0, 0.0, 0.0};
-  if (drag && S.grow_on) gq.rho *= gap_factor(d, S, x, y);
-  if (drag && S.dg_on) {   // disk gravity: fixed over the launch, like the big bodies' gravity
-    ax += gq.adg[0];
-    ay += gq.adg[1];
-  }
-  const DragConst dc = drag ? drag_const(S, gq, x, y, hp0, hp1, hp2, rp, kd) : DragConst{};
-#pragma unroll
-  for (int kk = 0; kk < NKICK; ++kk) {
+  if (split && (drag || MODE == kSplitFew || !split_flushes(S.nbig))) {
+    // the gas at the (fixed) position, shared by the launch's half kicks
+    DragSplit dc{};
     if (drag) {
-      const int kidx = kbase + kk;
-      const bool kuse = d.kmode != 0 && kidx < d.kcap;
-      const size_t word = (size_t)kidx * d.kwords + (j >> 5);
-      int kin = -1, kout = 0;
-      if (kuse && d.kmode == 2) kin = (d.kbits[word] >> (j & 31)) & 1u;
-      double dvec[3];
-      const double coef = gas_drag_coef(S, dc, u, v, w, dvec, kin, &kout);
-      if (kuse && d.kmode == 1 && kout) atomicOr(&d.kbits[word], 1u << (j & 31));
-      kick_with_drag(kick_h, ax, ay, az, coef, dvec, u, v, w);
-    } else {
-      u = fma(kick_h, ax, u);
-      v = fma(kick_h, ay, v);
-      w = fma(kick_h, az, w);
+      dc = drag_split(S, x, y, hp0, hp1, hp2, rp, kd);
+      ax += dc.adg[0];   // disk gravity: fixed over the launch, like the big bodies'
+      ay += dc.adg[1];
+    }
+    const SplitGrav g = split_gravity(acc, ax, ay, az);
+    auto word = [&](int kk) { return (size_t)(kbase + kk) * d.kwords + (j >> 5); };
+    auto branch = [&](int kk) {
+      return (d.kmode == 2 && kbase + kk < d.kcap) ? (int)((d.kbits[word(kk)] >> (j & 31)) & 1u) : -1;
+    };
+    auto keep = [&](int kk, int kb) {
+      if (d.kmode == 1 && kb && kbase + kk < d.kcap) atomicOr(&d.kbits[word(kk)], 1u << (j & 31));
+    };
+    split_kicks(S, kick_h, NKICK, g, drag, dc, x, y, hp0, hp1, hp2, rp, kd, u, v, w, branch,
+                keep);
+  } else {
+    // the gas at the (fixed) position, shared by the launch's half kicks
+    GasAt gq = drag ? gas_at(S, x, y) : GasAt{false, 0.0, 0.0, 0.0};
+    if (drag && S.grow_on) gq.rho *= gap_factor(d, S, x, y);
+    if (drag && S.dg_on) {   // disk gravity: fixed over the launch, like the big bodies' gravity
+      ax += gq.adg[0];
+      ay += gq.adg[1];
+    }
+    const DragConst dc = drag ? drag_const(S, gq, x, y, hp0, hp1, hp2, rp, kd) : DragConst{};
+#pragma unroll
+    for (int kk = 0; kk < NKICK; ++kk) {
+      if (drag) {
+        const int kidx = kbase + kk;
+        const bool kuse = d.kmode != 0 && kidx < d.kcap;
+        const size_t word = (size_t)kidx * d.kwords + (j >> 5);
+        int kin = -1, kout = 0;
+        if (kuse && d.kmode == 2) kin = (d.kbits[word] >> (j & 31)) & 1u;
+        double dvec[3];
+        const double coef = gas_drag_coef(S, dc, u, v, w, dvec, kin, &kout);
+        if (kuse && d.kmode == 1 && kout) atomicOr(&d.kbits[word], 1u << (j & 31));
+        kick_with_drag(kick_h, ax, ay, az, coef, dvec, u, v, w);
+      } else {
+        u = fma(kick_h, ax, u);
+        v = fma(kick_h, ay, v);
+        w = fma(kick_h, az, w);
+      }
     }
   }
   if (big) {
@@ -497,12 +543,12 @@ __device__ __forceinline__ void jump_kick_tile(const Dev& d, double jump_frac, d
 }
 
 // Dynamic shared memory of a kick: the big bodies' staging (and their FP32
-// parts behind it, where a system's gravity takes them), and for a fused
+// parts behind it), and for a fused
 // kick with more than 32 big bodies the momentum tree (in the same space,
 // before the staging).
 __host__ __device__ __forceinline__ size_t kick_smem_bytes(const Dev& d, bool fused) {
   size_t n = stage_bytes(d.big_max);
-  if (split_gravity(d.big_max)) n += sizeof(SplitBig) * (size_t)big_chunk(d.big_max);
+  n += sizeof(SplitBig) * (size_t)big_chunk(d.big_max);
   if (fused && d.big_max > 32) n = n < 3 * kThreads * sizeof(double) ? 3 * kThreads * sizeof(double) : n;
   return n;
 }

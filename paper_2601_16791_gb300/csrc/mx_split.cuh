@@ -1,5 +1,6 @@
-// mx_split.cuh -- the kick's pair sum in FP32 pairs (arXiv 2601.16791,
-// Sec. 2.1.3), for targets outside a big body's changeover shell.
+// mx_split.cuh -- the kick's pair sum in pairs of FP32 numbers (arXiv
+// 2601.16791, Sec. 2.1.3), for systems of light big bodies (SysDev::split) and
+// targets outside a big body's changeover shell.
 //
 // What bounds the pair sum: FP64 issues one warp instruction per scheduler in
 // 64 cycles on sm_103a, FP32 one per cycle (both measured), so the 17 FP64
@@ -7,21 +8,22 @@
 // same pair in pairs of FP32 numbers (a value kept as hi + lo, 48 bits) takes
 // about 115 instructions.
 //
-// What the precision is: the state, the jump, the velocity update and the sum
-// over blocks of kSplitRun big bodies stay FP64; only a far pair's
-// acceleration mu d/s^3 is formed in FP32 pairs, with a relative error of
-// about 1.5e-14 (rms, against 80-bit arithmetic).  A half kick adds
-// (h/2) a to a velocity; for a body outside the changeover shell (3 Hill
-// radii) that is at most a few 1e-4 of the velocity, so the split's share of
+// What the precision is: the state, the jump and the velocity update stay
+// FP64; only a far pair's acceleration mu d/s^3 is formed in FP32 pairs, with
+// a relative error of about 1.5e-14 (rms, against 80-bit arithmetic).  A half
+// kick adds (h/2) a to a velocity; outside the changeover shell (3 Hill radii)
+// that is at most a few 1e-4 of the velocity, so the split's share of
 // the new velocity's error is below 1e-17 of it, where the FP64 rounding of
 // the velocity itself is 1e-16.  A pair inside the shell, where the
 // acceleration is largest and K varies, goes through the FP64 pair_acc, and
 // so does a target outside the positions' grid below.  mx_accel, which returns
-// accelerations, keeps FP64 throughout.
+// accelerations, does not use it.
 //
 // Measured: k_jump_kick with 2,000 big bodies and 200,000 planetesimals 11.8 ->
 // 1.73 ms a launch (34 -> 233 G pairs/s), two steps of that disk 40.2 -> 9.9 ms;
-// 301 big bodies and 20,011 planetesimals 0.43 -> 0.068 ms a launch.
+// 301 big bodies and 20,011 planetesimals 0.43 -> 0.068 ms a launch.  64 gas
+// disks of 2 to 50 light bodies (2.4 million bodies; with the drag, see
+// mx_split_gas.cuh) 2.35 -> 0.45 ms a launch, three steps 12.0 -> 4.34 ms.
 //
 // Positions: each coordinate is cut on one grid for target and sources into
 // three FP32 parts, x = x0 + x1 + x2 with x0 a multiple of 2^(k-23), x1 of
@@ -76,6 +78,103 @@ __device__ __forceinline__ bool split_in_range(double x, double y, double z, int
   return abs_hi(x) < lim && abs_hi(y) < lim && abs_hi(z) < lim;
 }
 
+// ------------------------------------------------------- pairs of FP32 numbers
+// A value kept as h + l, l at most about an ulp of h: 48 bits.  Only rounding
+// intrinsics, so that the compiler contracts nothing and every caller gets the
+// same bits.
+struct FF {
+  float h, l;
+};
+
+__device__ __forceinline__ FF ff_fast(float a, float b) {   // |a| >= |b| or a = 0
+  const float s = __fadd_rn(a, b);
+  return FF{s, __fsub_rn(b, __fsub_rn(s, a))};
+}
+
+__device__ __forceinline__ FF ff_two_sum(float a, float b) {
+  const float s = __fadd_rn(a, b);
+  const float v = __fsub_rn(s, a);
+  return FF{s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, v)), __fsub_rn(b, v))};
+}
+
+__device__ __forceinline__ FF ff_add(FF a, FF b) {
+  const FF s = ff_two_sum(a.h, b.h);
+  return ff_fast(s.h, __fadd_rn(s.l, __fadd_rn(a.l, b.l)));
+}
+
+__device__ __forceinline__ FF ff_mul(FF a, FF b) {
+  const float p = __fmul_rn(a.h, b.h);
+  return ff_fast(p, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.l, __fmaf_rn(a.h, b.h, -p))));
+}
+
+__device__ __forceinline__ FF ff_neg(FF a) { return FF{-a.h, -a.l}; }
+
+// A product with a power of two, exactly.
+__device__ __forceinline__ FF ff_scale(FF a, float s) {
+  return FF{__fmul_rn(a.h, s), __fmul_rn(a.l, s)};
+}
+
+// x^2 + y^2 + z^2 of three pairs.
+__device__ __forceinline__ FF ff_norm2(float hx, float mx, float hy, float my, float hz, float mz) {
+  const float px = __fmul_rn(hx, hx), py = __fmul_rn(hy, hy), pz = __fmul_rn(hz, hz);
+  const float qx = __fmaf_rn(hx, hx, -px), qy = __fmaf_rn(hy, hy, -py),
+              qz = __fmaf_rn(hz, hz, -pz);
+  const FF s1 = ff_two_sum(px, py);
+  const FF s = ff_two_sum(s1.h, pz);
+  const float hm = __fmaf_rn(hx, mx, __fmaf_rn(hy, my, __fmul_rn(hz, mz)));
+  return FF{s.h, __fmaf_rn(2.0f, hm, __fadd_rn(__fadd_rn(__fadd_rn(qx, qy), qz),
+                                               __fadd_rn(s1.l, s.l)))};
+}
+
+// 1 - x y^2 = a + c for an estimate y of x^(-1/2), with y^2 = y2 + y2l:
+// 1 - x.h y2 exactly as a = 1 - p and p's rounding, then the low parts.
+__device__ __forceinline__ void ff_rsqrt_residual(FF x, float y, float& y2, float& y2l, float& a,
+                                                  float& c) {
+  y2 = __fmul_rn(y, y);
+  y2l = __fmaf_rn(y, y, -y2);
+  const float p = __fmul_rn(y2, x.h);
+  const float pe = __fmaf_rn(y2, x.h, -p);
+  a = __fsub_rn(1.0f, p);
+  c = -__fmaf_rn(y2, x.l, __fmaf_rn(y2l, x.h, pe));
+}
+
+// x^(-1/2) = y (1 + e/2 + 3 e^2/8), x > 0 (x.h normal)
+__device__ __forceinline__ FF ff_rsqrt(FF x) {
+  const float y = rsqrtf(x.h);
+  float y2, y2l, a, c;
+  ff_rsqrt_residual(x, y, y2, y2l, a, c);
+  const float e = __fadd_rn(a, c);
+  const FF g = ff_fast(y, __fmul_rn(__fmul_rn(0.5f, y), a));
+  return FF{g.h, __fadd_rn(g.l, __fmul_rn(y, __fmaf_rn(0.5f, c, __fmul_rn(__fmul_rn(0.375f, e), e))))};
+}
+
+// 1/x = y (1 + e + e^2)
+__device__ __forceinline__ FF ff_rcp(FF x) {
+  float y;
+  asm("rcp.approx.f32 %0, %1;" : "=f"(y) : "f"(x.h));
+  const float e = __fmaf_rn(-x.l, y, __fmaf_rn(-x.h, y, 1.0f));
+  return ff_fast(y, __fmul_rn(y, __fmaf_rn(e, e, e)));
+}
+
+// A double's leading 48 bits, read off its bit pattern (zero below 2^-126;
+// valid for |x| < 2^127).  Integer and FP32 instructions only.
+__device__ __forceinline__ FF ff_of(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const unsigned a = hi & 0x7fffffffu, sg = hi & 0x80000000u;
+  if (a < (897u << 20)) return FF{0.0f, 0.0f};
+  const float h = __uint_as_float(sg | ((a - (896u << 20)) << 3) | (lo >> 29));
+  const float r = __fmul_rn(__uint2float_rn(lo & 0x1fffffffu), 0x1p-52f);
+  const float sc = __uint_as_float(sg | (((a >> 20) - 896u) << 23));
+  return FF{h, __fmul_rn(r, sc)};
+}
+
+// A float as a double, exactly, by moving its bits (zero for a subnormal).
+__device__ __forceinline__ double bits_to_double(float f) {
+  const unsigned u = __float_as_uint(f), a = u & 0x7fffffffu;
+  if (a < 0x00800000u) return 0.0;
+  return __hiloint2double((int)((u & 0x80000000u) | ((a >> 3) + (896u << 20))), (int)(a << 29));
+}
+
 // One staged big body: its position in parts, mu as a pair, and the squared
 // separation below which the pair belongs to the FP64 path.
 struct alignas(16) SplitBig {
@@ -95,13 +194,11 @@ __device__ __forceinline__ float near2_of(double rc2) {
   return fmaxf(to_float_bits(rc2) * 1.0001f, 1e-30f);
 }
 
-// s + c + (error): a two-sum into the pair (h, l), with the product's low part.
+// A two-sum into the pair (h, l), with the term's low part.
 __device__ __forceinline__ void split_add(float& h, float& l, float ph, float pl) {
-  const float s = __fadd_rn(h, ph);
-  const float b = __fsub_rn(s, h);
-  const float er = __fadd_rn(__fsub_rn(h, __fsub_rn(s, b)), __fsub_rn(ph, b));
-  h = s;
-  l = __fadd_rn(l, __fadd_rn(er, pl));
+  const FF s = ff_two_sum(h, ph);
+  h = s.h;
+  l = __fadd_rn(l, __fadd_rn(s.l, pl));
 }
 
 // d = a - b of parts, as hi + lo.
@@ -112,37 +209,25 @@ __device__ __forceinline__ void split_sub(float a0, float a1, float a2, float b0
   m = __fadd_rn(__fsub_rn(d1, __fsub_rn(h, d0)), d2);
 }
 
-// A pair's mu d/s^3 added to acc; returns false, with nothing added, for a
-// pair inside near2.  1/s^3 = y^3 (1 + 3e/2 + 15e^2/8) from the single-
-// precision estimate y of 1/s, e = 1 - s^2 y^2, as in pair_weight.
-__device__ __forceinline__ bool split_pair(const SplitPos& t, const SplitBig& b, float near2,
-                                           SplitAcc& acc) {
+// A far pair's mu d/s^3 as hi + lo by component.
+struct SplitTerm {
+  float xh, xl, yh, yl, zh, zl;
+};
+
+// A pair's mu d/s^3; returns false, f not set, for a pair inside near2.
+// 1/s^3 = y^3 (1 + 3e/2 + 15e^2/8) from the single-precision estimate y of
+// 1/s, e = 1 - s^2 y^2, as in pair_weight.
+__device__ __forceinline__ bool split_term(const SplitPos& t, const SplitBig& b, float near2,
+                                           SplitTerm& f) {
   float hx, mx, hy, my, hz, mz;
   split_sub(t.x0, t.x1, t.x2, b.x0, b.x1, b.x2, hx, mx);
   split_sub(t.y0, t.y1, t.y2, b.y0, b.y1, b.y2, hy, my);
   split_sub(t.z0, t.z1, t.z2, b.z0, b.z1, b.z2, hz, mz);
-  // s^2 = s + l
-  const float px = __fmul_rn(hx, hx), py = __fmul_rn(hy, hy), pz = __fmul_rn(hz, hz);
-  const float qx = __fmaf_rn(hx, hx, -px), qy = __fmaf_rn(hy, hy, -py),
-              qz = __fmaf_rn(hz, hz, -pz);
-  const float s1 = __fadd_rn(px, py);
-  const float b1 = __fsub_rn(s1, px);
-  const float e1 = __fadd_rn(__fsub_rn(px, __fsub_rn(s1, b1)), __fsub_rn(py, b1));
-  const float s = __fadd_rn(s1, pz);
-  const float b2 = __fsub_rn(s, s1);
-  const float e2 = __fadd_rn(__fsub_rn(s1, __fsub_rn(s, b2)), __fsub_rn(pz, b2));
-  if (s < near2) return false;
-  const float hm = __fmaf_rn(hx, mx, __fmaf_rn(hy, my, __fmul_rn(hz, mz)));
-  const float l = __fmaf_rn(2.0f, hm, __fadd_rn(__fadd_rn(__fadd_rn(qx, qy), qz),
-                                                __fadd_rn(e1, e2)));
-  const float y = rsqrtf(s);
-  const float y2 = __fmul_rn(y, y);
-  const float y2l = __fmaf_rn(y, y, -y2);
-  // e = a + c: 1 - y2 s exactly as 1 - p (exact) - pe, then the low parts
-  const float p = __fmul_rn(y2, s);
-  const float pe = __fmaf_rn(y2, s, -p);
-  const float a = __fsub_rn(1.0f, p);
-  const float c = -__fmaf_rn(y2, l, __fmaf_rn(y2l, s, pe));
+  const FF s2 = ff_norm2(hx, mx, hy, my, hz, mz);
+  if (s2.h < near2) return false;
+  const float y = rsqrtf(s2.h);
+  float y2, y2l, a, c;
+  ff_rsqrt_residual(s2, y, y2, y2l, a, c);
   const float e = __fadd_rn(a, c);
   const float k1 = __fmul_rn(1.5f, a);
   const float k2 = __fmaf_rn(1.5f, c, __fmul_rn(__fmul_rn(1.875f, e), e));
@@ -155,17 +240,31 @@ __device__ __forceinline__ bool split_pair(const SplitPos& t, const SplitBig& b,
   wl = __fmaf_rn(b.mul, y3, wl);
   wl = __fmaf_rn(wh, k2, wl);
   wl = __fmaf_rn(wh, k1, wl);
-  const float fx = __fmul_rn(wh, hx), fy = __fmul_rn(wh, hy), fz = __fmul_rn(wh, hz);
-  split_add(acc.xh, acc.xl, fx, __fmaf_rn(wl, hx, __fmaf_rn(wh, mx, __fmaf_rn(wh, hx, -fx))));
-  split_add(acc.yh, acc.yl, fy, __fmaf_rn(wl, hy, __fmaf_rn(wh, my, __fmaf_rn(wh, hy, -fy))));
-  split_add(acc.zh, acc.zl, fz, __fmaf_rn(wl, hz, __fmaf_rn(wh, mz, __fmaf_rn(wh, hz, -fz))));
+  f.xh = __fmul_rn(wh, hx);
+  f.yh = __fmul_rn(wh, hy);
+  f.zh = __fmul_rn(wh, hz);
+  f.xl = __fmaf_rn(wl, hx, __fmaf_rn(wh, mx, __fmaf_rn(wh, hx, -f.xh)));
+  f.yl = __fmaf_rn(wl, hy, __fmaf_rn(wh, my, __fmaf_rn(wh, hy, -f.yh)));
+  f.zl = __fmaf_rn(wl, hz, __fmaf_rn(wh, mz, __fmaf_rn(wh, hz, -f.zh)));
   return true;
 }
 
+__device__ __forceinline__ void split_sum(SplitAcc& acc, const SplitTerm& f) {
+  split_add(acc.xh, acc.xl, f.xh, f.xl);
+  split_add(acc.yh, acc.yl, f.yh, f.yl);
+  split_add(acc.zh, acc.zl, f.zh, f.zl);
+}
+
+// Puts the low parts back below the high ones' last place.
+__device__ __forceinline__ void split_renorm(SplitAcc& acc) {
+  const FF x = ff_fast(acc.xh, acc.xl), y = ff_fast(acc.yh, acc.yl), z = ff_fast(acc.zh, acc.zl);
+  acc = SplitAcc{x.h, x.l, y.h, y.l, z.h, z.l};
+}
+
 __device__ __forceinline__ void split_flush(SplitAcc& acc, double& ax, double& ay, double& az) {
-  ax -= (double)acc.xh + (double)acc.xl;
-  ay -= (double)acc.yh + (double)acc.yl;
-  az -= (double)acc.zh + (double)acc.zl;
+  ax -= bits_to_double(acc.xh) + bits_to_double(acc.xl);
+  ay -= bits_to_double(acc.yh) + bits_to_double(acc.yl);
+  az -= bits_to_double(acc.zh) + bits_to_double(acc.zl);
   acc = SplitAcc{};
 }
 

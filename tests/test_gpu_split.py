@@ -1,5 +1,5 @@
-"""The kick's gravity in FP32 pairs (systems with more than 64 big bodies)
-against the FP64 pair sum of mx_accel, at the same positions.
+"""The kick's gravity and drag in FP32 pairs against the FP64 ones of mx_accel, at the same
+positions.
 
 With every velocity zero, the pre-drift velocity of a step is (h/2) a, a the
 acceleration of the first half kick (the momentum is zero, so nothing jumps).
@@ -41,8 +41,9 @@ def place(w, far, shell):
 
 
 @pytest.mark.parametrize("nbig,nsmall,scale,far,shell", [
-    (64, 300, 1.0, False, False),      # the FP64 rule
-    (65, 1, 1.0, False, False),
+    (2, 700, 1.0, True, True),
+    (64, 300, 1.0, False, False),      # one sum in FP32 pairs
+    (65, 1, 1.0, False, False),        # emptied into FP64 every 32
     (65, 1000, 1.0, True, True),
     (96, 333, 0.01, False, True),
     (256, 500, 1.0, False, True),
@@ -76,7 +77,53 @@ def test_split_kick_against_fp64(nbig, nsmall, scale, far, shell):
     size = 0.5 * w.params["dt"] * (W.G * w.m_big / s2).sum(1)
     err = np.linalg.norm(got - want, axis=0) / size
     assert err.max() <= TOL, err.max()
-    if nbig <= 64 or scale > 1000:
+    if scale > 1000:
         assert err.max() <= 4e-16
     else:
         assert err.max() > 0.0     # the split path ran
+
+
+@pytest.mark.parametrize("nbig,nsmall,gas", [
+    (1, 257, {}),                      # a core: the FP64 kick
+    (3, 3000, {}),
+    (33, 1000, {}),                    # a second run of the pair sum
+    (64, 500, dict(cd_mode=1)),
+    (65, 500, {}),                     # the pair sum goes through FP64
+    (4, 2000, dict(gamma=1.5, flare=0.2, r_c_au=20.0, r_in_au=2.0)),
+    (4, 2000, dict(gamma=1.5, r_in_au=0.5, disk_gravity=True)),
+])
+def test_split_drag_against_fp64(nbig, nsmall, gas):
+    """A half kick with drag: v1 - v0 against (h/2) mx_accel.  Bound: two
+    roundings of the velocity (3e-16 of it), the pairs' 2e-13, and for the drag
+    a chain of about twenty products of FP32 pairs, 20 x 2^-45 = 6e-13: 1e-12.
+    Radii from a centimetre to a thousand km reach both sides of Re = 1e5 and
+    the values that go back to FP64."""
+    w = W.gas_4core_100k(seed=5, nbig=nbig, nsmall=nsmall)
+    if nbig > 2:
+        w.m_big *= 1e-3        # light big bodies; with cores the kick is FP64
+    w.params["gas"].update(gas)
+    w.params["dt"] = 1e-2      # small bodies stop within days
+    rng = np.random.default_rng(2)
+    w.rp_km = np.exp(rng.uniform(np.log(1e-5), np.log(1e3), nsmall))
+    g = mx.System(w)
+    mx.mx_set_defer_window(g.h, 0)
+    start = torch.empty((6, w.n), dtype=torch.float64, device="cuda")
+    mx.mx_get_state_device(g.h, start)
+    acc = torch.empty((3, w.n), dtype=torch.float64, device="cuda")
+    drag = torch.empty((3, nsmall), dtype=torch.float64, device="cuda")
+    mx.mx_accel(g.h, acc)
+    mx.mx_gas_drag(g.h, drag)
+    pre = torch.empty((6, w.n), dtype=torch.float64, device="cuda")
+    mx.mx_step(g.h, 1)
+    mx.mx_predrift_state(g.h, pre)
+    g.close()
+    h2 = 0.5 * w.params["dt"]
+    v0 = start[3:].cpu().numpy()
+    x = start[:3].cpu().numpy()
+    err = np.linalg.norm(pre[3:].cpu().numpy() - (v0 + h2 * acc.cpu().numpy()), axis=0)
+    d = x[:, :, None] - x[:, None, :nbig]
+    s2 = (d * d).sum(0)
+    s2[s2 == 0] = np.inf
+    bound = 3e-16 * np.linalg.norm(v0, axis=0) + TOL * h2 * (W.G * w.m_big / s2).sum(1)
+    bound[nbig:] += 1e-12 * h2 * np.linalg.norm(drag.cpu().numpy(), axis=0)
+    assert (err / bound).max() <= 1.0, (err / bound).max()
