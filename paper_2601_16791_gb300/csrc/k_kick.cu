@@ -39,9 +39,10 @@ KickKernel kick_kernel(int mode) {
 }
 
 // Kick acceleration (gravity + drag) without changing the state: 3 x N.
-__global__ void __launch_bounds__(kThreads) k_accel(Dev d, double* acc, int drag_only,
-                                                    int acc_stride, int acc_base) {
-  extern __shared__ double dsm[];
+// The gravity's far pairs in three FP32 parts (split_term3).
+__global__ void __launch_bounds__(kThreads, 2) k_accel(Dev d, double* acc, int drag_only,
+                                                       int acc_stride, int acc_base) {
+  extern __shared__ __align__(16) double dsm[];
   BigSmem sb(dsm, big_chunk(d.big_max));
   const Tile t = d.tiles[blockIdx.x];
   const SysDev& S = d.sys[t.sys];
@@ -62,7 +63,9 @@ __global__ void __launch_bounds__(kThreads) k_accel(Dev d, double* acc, int drag
     if (jl < S.nbig) rcj = d.brc[S.boff + jl];
   }
   double ax = 0, ay = 0, az = 0;
-  if (!drag_only) gravity_all(d, S, sb, act, jl, rcj, x, y, z, ax, ay, az);
+  SplitAcc3 sum{};
+  if (!drag_only)
+    gravity_split<TripleSum, true>(d, S, sb, act, jl, rcj, x, y, z, ax, ay, az, sum, nullptr);
   if (!valid) return;
   const bool drag = act && S.gas_on && jl >= S.nbig;
   double a[3] = {0.0, 0.0, 0.0};
@@ -105,8 +108,8 @@ void launch_jump_kick_fused(const Dev& d, cudaStream_t st) {
 
 void launch_accel(const Dev& d, double* acc, int drag_only, int acc_stride, int acc_base,
                   cudaStream_t st) {
-  k_accel<<<d.ntiles, d.tile, stage_bytes(d.big_max), st>>>(d, acc, drag_only, acc_stride,
-                                                              acc_base);
+  const size_t sm = stage_bytes(d.big_max) + sizeof(SplitBig3) * (size_t)big_chunk(d.big_max);
+  k_accel<<<d.ntiles, d.tile, sm, st>>>(d, acc, drag_only, acc_stride, acc_base);
 }
 
 // The kernels of a step share one shared-memory carveout (the largest), so

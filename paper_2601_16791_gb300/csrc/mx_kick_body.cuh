@@ -2,6 +2,7 @@
 // momentum prep (k_kick.cu), shared by their kernels and the persistent step
 // kernel.
 #pragma once
+#include <type_traits>
 #include "mx_common.cuh"
 #include "mx_growth.cuh"
 #include "mx_physics.cuh"
@@ -102,16 +103,16 @@ __device__ __forceinline__ SplitBig split_big(double x, double y, double z, doub
 // into (ax, ay, az) as it goes; pairs inside the changeover shell, and every
 // pair of a target off the positions' grid, go through the FP64 pair_acc into
 // (ax, ay, az).  Every thread of the block must call it.
-template <bool MANY>
+template <class Sum, bool MANY>
 __device__ __forceinline__ void gravity_split(const Dev& d, const SysDev& S, BigSmem& sb,
                                               bool act, int jl, double rcj, double x, double y,
                                               double z, double& ax, double& ay, double& az,
-                                              SplitAcc& acc, const double* dj) {
+                                              typename Sum::Acc& acc, const double* dj) {
   __shared__ int s_hi;
-  SplitBig* sp = reinterpret_cast<SplitBig*>(reinterpret_cast<unsigned char*>(sb.x) +
-                                             stage_bytes(d.big_max));
+  using Big = typename Sum::Big;
+  Big* sp = reinterpret_cast<Big*>(reinterpret_cast<unsigned char*>(sb.x) + stage_bytes(d.big_max));
   const bool jbig = jl < S.nbig;
-  const bool flush = MANY && split_flushes(S.nbig);
+  const bool flush = MANY && (!std::is_same<Sum, PairSum>::value || split_flushes(S.nbig));
   const float near_own = jbig ? near2_of(rcj * rcj) : 0.0f;
   SplitPos t{};
   int kt = INT_MIN;   // the grid t was cut on
@@ -138,7 +139,7 @@ __device__ __forceinline__ void gravity_split(const Dev& d, const SysDev& S, Big
     const bool grid = kg <= kSplitMaxK;
     if (grid)
       for (int k = threadIdx.x; k < cn; k += blockDim.x)
-        sp[k] = split_big(sb.x[k], sb.y[k], sb.z[k], sb.mu[k], sb.rc2[k], kg);
+        sp[k] = Sum::make(split_big(sb.x[k], sb.y[k], sb.z[k], sb.mu[k], sb.rc2[k], kg), sb.mu[k]);
     __syncthreads();
     if (!act) continue;
     auto pair64 = [&](int k) {
@@ -167,13 +168,10 @@ __device__ __forceinline__ void gravity_split(const Dev& d, const SysDev& S, Big
     for (int k0 = 0; k0 < cn; k0 += kSplitRun) {
       const int kn = min(cn, k0 + kSplitRun);
 #pragma unroll 2
-      for (int k = k0; k < kn; ++k) {
-        SplitTerm f;
-        if (split_term(t, sp[k], fmaxf(sp[k].near2, near_own), f)) split_sum(acc, f);
-        else pair64(k);
-      }
-      if (flush) split_flush(acc, ax, ay, az);
-      else split_renorm(acc);
+      for (int k = k0; k < kn; ++k)
+        if (!Sum::term(t, sp[k], fmaxf(Sum::near2(sp[k]), near_own), acc)) pair64(k);
+      if (flush) Sum::flush(acc, ax, ay, az);
+      else Sum::renorm(acc);
     }
   }
 }
@@ -462,7 +460,7 @@ __device__ __forceinline__ void jump_kick_tile(const Dev& d, double jump_frac, d
   SplitAcc acc{};
   const bool split = MODE == kSplitFew || (MODE == kSplitAny && S.split);
   if (split)
-    gravity_split<MODE == kSplitAny>(d, S, sb, act, jl, rcj, x, y, z, ax, ay, az, acc,
+    gravity_split<PairSum, MODE == kSplitAny>(d, S, sb, act, jl, rcj, x, y, z, ax, ay, az, acc,
                                      FUSED ? dj : nullptr);
   else
     gravity_all(d, S, sb, act, jl, rcj, x, y, z, ax, ay, az, FUSED ? dj : nullptr);
