@@ -930,7 +930,7 @@ void launch_adjoint_bs_plan(const Dev& d, const Adj& a, cudaStream_t st) {
   cudaMemsetAsync(d.pair_count, 0, sizeof(int), st);
   launch_detect(dd, a.x2, a.xv3, d.flags, d.keys, d.pair_count, d.pair_cap, 1, st);
   // sorted keys give the work items a fixed order (the shares' fold follows it)
-  launch_sort_keys(d.keys, d.pair_count, d.pair_cap, 0, st);
+  launch_sort_keys(d.keys, d.pair_count, d.pair_cap, 0, d.sort_tmp, st);
   launch_groups(dd, st);   // the step's own groups: big groups, then test-particle groups
   k_adj_tape<<<1, 1024, 0, st>>>(dd, a);
 }
@@ -939,7 +939,7 @@ void launch_adjoint_bs_fwd(const Dev& d, const Adj& a, int nblocks, cudaStream_t
   if (a.sorted_shares) {
     cudaMemsetAsync(a.scount, 0, sizeof(int), st);
     k_adj_share_keys<<<a.bs_blocks, kThreads, 0, st>>>(d, a);
-    launch_sort_keys(a.skeys, a.scount, a.skeys_cap, 0, st);
+    launch_sort_keys(a.skeys, a.scount, a.skeys_cap, 0, d.sort_tmp, st);
   }
   k_adj_bs_fwd<<<nblocks, 32, 0, st>>>(d, a);    // every item but the test-particle pairs
   k_adj_bs_fwd2<<<nblocks, 128, 0, st>>>(d, a);  // test-particle pairs

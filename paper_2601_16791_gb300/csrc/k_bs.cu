@@ -2092,7 +2092,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_step_persist(Dev d, long long s
   for (int t = next_tile(ctr); t < d.ntiles; t = next_tile(ctr)) jump_drift_tile(d, 0.5, t);
   if (!grid_sync(d.gbar, spin, d.status)) return;
   for (int t = next_tile(ctr + 1); t < d.ntiles; t = next_tile(ctr + 1))
-    detect_tile(d, d.xv0, d.xv, d.flags, d.keys, d.pair_count, d.pair_cap, 1, t, dsm_p);
+    detect_tile<false>(d, d.xv0, d.xv, d.flags, d.keys, d.pair_count, d.pair_cap, 1, t, dsm_p);
   if (!grid_sync(d.gbar, spin, d.status)) return;
   if (blockIdx.x == 0) groups_block(d);
   if (!grid_sync(d.gbar, spin, d.status)) return;
@@ -2105,7 +2105,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_step_persist(Dev d, long long s
 }
 
 static size_t persist_smem_bytes(const Dev& d) {
-  const size_t a = det_smem_bytes(det_chunk(d.tile, d.big_max));
+  const size_t a = det_smem_bytes(det_chunk(d.tile, d.big_max), false);
   const size_t b = kick_smem_bytes(d, true);
   return a > b ? a : b;
 }

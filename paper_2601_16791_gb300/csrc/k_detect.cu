@@ -17,29 +17,60 @@
 
 namespace mx {
 
+template <bool FEW>
 __global__ void __launch_bounds__(kThreads) k_detect(Dev d, const double* xv0, const double* xv1,
                                                      unsigned char* flags,
                                                      unsigned long long* keys, int* count,
                                                      int cap, int runs) {
   extern __shared__ __align__(16) unsigned char dsm_det[];
-  detect_tile(d, xv0, xv1, flags, keys, count, cap, runs, blockIdx.x, dsm_det);
+  detect_tile<FEW>(d, xv0, xv1, flags, keys, count, cap, runs, blockIdx.x, dsm_det);
+}
+
+// The step's (small-flag, j, i) key as an (i, j) key.
+__device__ __forceinline__ unsigned long long swapped(unsigned long long k) {
+  return ((k & 0xffffffffull) << 32) | ((k >> 32) & 0x7fffffffull);
+}
+
+// Ranks of up to kRankMax keys, all SMs together: a key's place is the number
+// of smaller ones (the keys are distinct pairs), counted by eight lanes.  The
+// n^2 compares of 5,500 keys (2,000 big bodies + 200,000 planetesimals) take
+// 39 us where one block's bitonic sort took 120; beyond kRankMax the sort's
+// n log^2 n wins (16,384 keys: 2.7e8 compares, about 40 us).
+constexpr int kRankMax = kSortTmp;
+__global__ void __launch_bounds__(256) k_rank_keys(const unsigned long long* keys, const int* count,
+                                                   int cap, int swap_ij, unsigned long long* out) {
+  const int n = min(*count, cap);
+  if (n > kRankMax) return;
+  const int sub = threadIdx.x & 7;
+  const unsigned gmask = 0xffu << (threadIdx.x & 24);
+  const int per = (gridDim.x * blockDim.x) >> 3;
+  for (int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 3; i < n; i += per) {
+    const unsigned long long k = swap_ij ? swapped(keys[i]) : keys[i];
+    int r = 0;
+#pragma unroll 8
+    for (int m = sub; m < n; m += 8) r += ((swap_ij ? swapped(keys[m]) : keys[m]) < k) ? 1 : 0;
+    for (int o = 4; o > 0; o >>= 1) r += __shfl_xor_sync(gmask, r, o);
+    if (sub == 0) out[r] = k;
+  }
 }
 
 // Sorts min(*count, cap) keys ascending in one block (bitonic; shared memory
-// up to kSortSmem keys, global memory beyond).  swap_ij turns the step's
+// up to kSortSmem keys, global memory beyond), or copies them back from
+// `ranked`, where k_rank_keys has put them.  swap_ij turns the step's
 // (small-flag, j, i) keys into (i, j) keys first.
 constexpr int kSortSmem = 4096;   // 32 KB of static shared memory
 __global__ void __launch_bounds__(1024) k_sort_keys(unsigned long long* keys, const int* count,
-                                                    int cap, int swap_ij) {
+                                                    int cap, int swap_ij,
+                                                    const unsigned long long* ranked) {
   __shared__ unsigned long long sk[kSortSmem];
   const int n = min(*count, cap);
   if (n <= 0) return;
+  if (ranked && n <= kRankMax) {
+    for (int i = threadIdx.x; i < n; i += blockDim.x) keys[i] = ranked[i];
+    return;
+  }
   if (swap_ij) {
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-      const unsigned long long k = keys[i];
-      const unsigned long long jj = (k >> 32) & 0x7fffffffull, ii = k & 0xffffffffull;
-      keys[i] = (ii << 32) | jj;
-    }
+    for (int i = threadIdx.x; i < n; i += blockDim.x) keys[i] = swapped(keys[i]);
     __syncthreads();
   }
   int P2 = 1;
@@ -90,21 +121,25 @@ void launch_keys_to_pairs(const unsigned long long* keys, const int* count, int 
 
 void launch_detect(const Dev& d, const double* xv0, const double* xv1, unsigned char* flags,
                    unsigned long long* keys, int* count, int cap, int runs, cudaStream_t st) {
-  const size_t sm = det_smem_bytes(det_chunk(d.tile, d.big_max));
-  k_detect<<<d.ntiles, d.tile, sm, st>>>(d, xv0, xv1, flags, keys, count, cap, runs);
+  const bool few = det_few(d.big_max);
+  const size_t sm = det_smem_bytes(det_chunk(d.tile, d.big_max), few);
+  auto* k = few ? k_detect<true> : k_detect<false>;
+  k<<<d.ntiles, d.tile, sm, st>>>(d, xv0, xv1, flags, keys, count, cap, runs);
 }
 
 void launch_sort_keys(unsigned long long* keys, const int* count, int cap, int swap_ij,
-                      cudaStream_t st) {
-  k_sort_keys<<<1, 1024, 0, st>>>(keys, count, cap, swap_ij);
+                      unsigned long long* tmp, cudaStream_t st) {
+  if (tmp) k_rank_keys<<<256, 256, 0, st>>>(keys, count, cap, swap_ij, tmp);
+  k_sort_keys<<<1, 1024, 0, st>>>(keys, count, cap, swap_ij, tmp);
 }
 
 // The kernels of a step share one shared-memory carveout (the largest), so
 // the SMs are not reconfigured between consecutive kernels with different
 // shared-memory needs (measured: ~12 us bubbles before k_detect and the kick).
 void configure_detect() {
-  cudaFuncSetAttribute(k_detect, cudaFuncAttributePreferredSharedMemoryCarveout,
-                       cudaSharedmemCarveoutMaxShared);
+  for (auto* k : {k_detect<true>, k_detect<false>})
+    cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout,
+                         cudaSharedmemCarveoutMaxShared);
 }
 
 }  // namespace mx

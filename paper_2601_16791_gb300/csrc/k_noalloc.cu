@@ -118,7 +118,7 @@ extern "C" mx_status mx_detect_encounters_noalloc(const mx_params* p, int n_big,
   if (cudaGetLastError() != cudaSuccess) return MX_ERR_CUDA;
   mx::launch_detect(d, dev_xv0, dev_xv1, dev_flags, keys, count, MX_NOALLOC_MAX_PAIRS, 0, st);
   if (cudaGetLastError() != cudaSuccess) return MX_ERR_CUDA;
-  mx::launch_sort_keys(keys, count, MX_NOALLOC_MAX_PAIRS, 1, st);
+  mx::launch_sort_keys(keys, count, MX_NOALLOC_MAX_PAIRS, 1, nullptr, st);
   if (cudaGetLastError() != cudaSuccess) return MX_ERR_CUDA;
   if (cap > 0) {
     mx::launch_keys_to_pairs(keys, count, cap < MX_NOALLOC_MAX_PAIRS ? cap : MX_NOALLOC_MAX_PAIRS,

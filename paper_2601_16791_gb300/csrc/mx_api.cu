@@ -788,6 +788,7 @@ mx_status build(mx_system* s, const std::vector<const double*>& m_big,
   MX_TRY(dalloc(s, &d.arrive, 1));
   MX_TRY(dalloc(s, &d.flags, N));
   MX_TRY(dalloc(s, &d.keys, cap2));
+  MX_TRY(dalloc(s, &d.sort_tmp, mx::kSortTmp));
   MX_TRY(dalloc(s, &d.pair_count, 2));
   d.work_count = d.pair_count + 1;
   const int work_cap = cap + NB;
@@ -1586,7 +1587,7 @@ mx_status mx_detect_encounters(mx_system* s, const double* dev_xv0, const double
   dd.bb_count = nullptr;
   dd.defer = 0;
   mx::launch_detect(dd, dev_xv0, dev_xv1, flags, s->d.keys, s->d.pair_count, s->d.pair_cap, 0, s->st);
-  mx::launch_sort_keys(s->d.keys, s->d.pair_count, s->d.pair_cap, 1, s->st);
+  mx::launch_sort_keys(s->d.keys, s->d.pair_count, s->d.pair_cap, 1, s->d.sort_tmp, s->st);
   if (dev_pairs && cap > 0)
     mx::launch_keys_to_pairs(s->d.keys, s->d.pair_count, std::min(cap, s->d.pair_cap), dev_pairs, s->st);
   MX_CUDA(cudaMemcpyAsync(s->h_count, s->d.pair_count, sizeof(int), cudaMemcpyDeviceToHost, s->st));

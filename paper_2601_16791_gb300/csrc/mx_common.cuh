@@ -29,6 +29,7 @@ constexpr int kMaxBigPairs = 512; // big-big encounter pairs handled per step
 // the direct path's order), so with many big bodies a replay costs more than
 // the encounter it moves off the step.
 constexpr int kDeferMaxBig = 64;
+constexpr int kSortTmp = 1 << 14;   // keys that are sorted by rank over all SMs (k_detect.cu)
 // Kick kernels by the systems' SysDev::split: no system; every system, none
 // with more than kDeferMaxBig big bodies; any mix.
 enum : int { kSplitNone = 0, kSplitFew = 1, kSplitAny = 2 };
@@ -104,6 +105,7 @@ struct Dev {
   int* arrive;     // [1] blocks of a kick with its own prep that have read the history slot
   unsigned char* flags;               // N
   unsigned long long* keys;           // pair keys [pair_cap]
+  unsigned long long* sort_tmp;       // [kSortTmp] scratch of launch_sort_keys
   int* pair_count;
   int* work_count;
   int* work_off;   // [work_cap + 1]

@@ -26,6 +26,30 @@ __device__ __forceinline__ bool encounter_screen(const float* a, const float* b,
   return lb <= 1.1f * rc2f + 1e-3f * (d0 + d1 + D0 + D1);
 }
 
+// A body's reach A over the step, for the first screen: a pair whose starting
+// separation s0 is at least A_a + A_b cannot be flagged, whatever its motion.
+// With D the sum of both bodies' displacements over the step, V the sum of
+// their largest speeds, q = (8/27) |h| V and rc the larger changeover radius,
+// the separation at the end is at least s0 - D, the slopes are at most
+// 2 |h| V s0 and 2 |h| V (s0 + D), so a flagged pair (the bound of
+// encounter_screen) has (s0 - D)^2 <= rc^2 + q (2 s0 + D), that is
+//   s0 <= D + q + sqrt(3 q D + q^2 + rc^2).
+// With w = max(displacement, |h| speed) of each body and W = w_a + w_b, D <= W
+// and q <= (8/27) W, so s0 <= 1.2963 W + 0.9885 W + rc <= sum of
+// (2.285 w + rc) over the two bodies.  The states' FP32 copies are cut at
+// 2^-20 of each coordinate: 1e-3 of A and 1.6e-5 of the largest coordinate
+// cover that and the FP32 rounding.  a: as for encounter_screen; the body's rc.
+__device__ __forceinline__ float encounter_reach(const float* a, float rc, float hf) {
+  const float dx = a[6] - a[0], dy = a[7] - a[1], dz = a[8] - a[2];
+  const float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+  const float v0 = fmaf(a[3], a[3], fmaf(a[4], a[4], a[5] * a[5]));
+  const float v1 = fmaf(a[9], a[9], fmaf(a[10], a[10], a[11] * a[11]));
+  const float w = sqrtf(fmaxf(d2, hf * hf * fmaxf(v0, v1)));
+  float m = 0.0f;
+  for (int q = 0; q < 3; ++q) m = fmaxf(m, fmaxf(fabsf(a[q]), fabsf(a[6 + q])));
+  return 1.001f * fmaf(2.285f, w, rc) + 1.6e-5f * m;
+}
+
 // Exact FP64 encounter test between target a and big b (6 doubles each at
 // the start, 0, and end, 1, of the step).
 static __device__ __noinline__ bool encounter_fp64(const double* a0, const double* b0, const double* a1,
