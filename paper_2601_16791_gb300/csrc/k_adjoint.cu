@@ -18,6 +18,7 @@
 #include "mx_kepler.cuh"
 #include "mx_kernels.h"
 #include "mx_physics.cuh"
+#include "mx_kick_body.cuh"
 
 namespace mx {
 
@@ -26,103 +27,118 @@ namespace mx {
 // (x, y, z), heliocentric velocity (u, v, w), radius rp_cm, kd = 3/(8 r_p rho_p),
 // k branch kb of Eq. 7; la is the cotangent of the acceleration.  Adds the
 // cotangents of position (gx), velocity (gv) and of (sigma1, gamma, cd_scale)
-// (gp).  The forward quantities are recomputed here in plain form.
+// (gp).  Bound by FP64 issue: reciprocals are formed once (rsqrt_d, rcp_d, five
+// instructions each, where a library division or square root takes ten) and the
+// powers of R come from rsqrt chains when flare = 1/4 and gamma = 1, as in
+// gas_at, so that one logarithm (the gamma cotangent's) is the only library
+// call left there: 4 cores + 50,000 planetesimals, the drag-only reverse of a
+// half kick: 93 -> 50 us.
 __device__ void drag_vjp(const SysDev& S, double x, double y, double u, double v, double w,
                          double rp_cm, double kd, int kb, const double* la, double* gx,
                          double* gv, double* gp) {
-  const double R2 = x * x + y * y;
-  const double R = sqrt(R2);
-  if (!(R >= S.r_in) || R2 == 0.0) return;
+  const double R2 = fma(x, x, y * y);
+  if (R2 == 0.0) return;
+  const double iR = rsqrt_d(R2);
+  const double R = R2 * iR;
+  if (!(R >= S.r_in)) return;
   const double lnR = log(R);
+  const double ih = rsqrt_d(R);                  // R^-1/2
   double E = 1.0, dlnE_dR = 0.0, dlnE_dg = 0.0;
   if (!S.rc_inf) {
     const double lr = log(R * S.inv_rc);
     const double p = exp((2.0 - S.gamma) * lr);
     E = exp(-p);
-    dlnE_dR = -(2.0 - S.gamma) * p / R;
+    dlnE_dR = -(2.0 - S.gamma) * p * iR;
     dlnE_dg = p * lr;
   }
-  const double sigma = S.sigma1 * exp(-S.gamma * lnR) * E;
-  const double vk = S.sqrt_mu0 / sqrt(R);
-  const double cs = S.c_cs * exp((S.flare - 0.5) * lnR);
-  const double rho = S.c_rho * sigma * exp(-(1.0 + S.flare) * lnR);
-  const double Rf2 = exp(2.0 * S.flare * lnR);
+  double rmh, ics, Rf2;                          // R^-(1+f), 1/c_s, R^(2f)
+  if (S.flare_quarter) {
+    const double q = rsqrt_d(ih);                // R^1/4
+    rmh = iR * (q * ih);
+    ics = q * S.inv_c_cs;
+    Rf2 = R * ih;
+  } else {
+    rmh = exp(-(1.0 + S.flare) * lnR);
+    ics = rcp_d(S.c_cs * exp((S.flare - 0.5) * lnR));
+    Rf2 = exp(2.0 * S.flare * lnR);
+  }
+  const double sig1 = (S.gamma_one ? iR : exp(-S.gamma * lnR)) * E;   // Sigma / sigma1
+  const double vk = S.sqrt_mu0 * ih;
+  const double rho = S.c_rho * (S.sigma1 * sig1) * rmh;
   const double eta = S.c_eta * Rf2;
-  const double t = 1.0 - 2.0 * eta;
-  const double st = sqrt(t);
-  const double vg = vk * st;
-  const double gf = vg / R;
-  const double du = u + gf * y, dv = v - gf * x, dw = w;
-  const double D2 = du * du + dv * dv + dw * dw;
+  const double t = fma(-2.0, eta, 1.0);
+  const double ist = rsqrt_d(t);                 // (1 - 2 eta)^-1/2
+  const double vg = vk * (t * ist);
+  const double gf = vg * iR;
+  const double du = fma(gf, y, u), dv = fma(-gf, x, v), dw = w;
+  const double D2 = fma(du, du, fma(dv, dv, dw * dw));
   if (D2 == 0.0) return;
-  const double Dm = sqrt(D2);
-  const double Ma = Dm / cs;
-  const double Re = S.c_re * rp_cm * Ma * rho;
-  const double k = kb ? 0.2 : 0.4;
-  const double Dn = 240.0 + 64.0 * Re;
-  const double den1 = Re * (10.0 + Re) + 0.23 * Ma * Dn;
-  const double first0 = Dn / den1;
+  const double iDm = rsqrt_d(D2);
+  const double Dm = D2 * iDm;
+  const double Ma = Dm * ics;
+  const double re_k = S.c_re * rp_cm;            // Re = re_k Ma rho
+  const double Re = re_k * Ma * rho;
+  const double k16 = kb ? 1.6 * 0.2 : 1.6 * 0.4;
+  const double Dn = fma(64.0, Re, 240.0);
+  const double den1 = fma(0.23 * Ma, Dn, Re * (10.0 + Re));
+  const double iden = rcp_d(den1);
+  const double first0 = Dn * iden;
   const double first = (S.cd_mode == 1) ? first0 * first0 : first0;
-  const double A = 1.6 + Ma;
-  const double second = (1.6 * k + 2.0 * Ma) / A;
+  const double iA = rcp_d(1.6 + Ma);
+  const double second = fma(2.0, Ma, k16) * iA;
   const double CD = first + second;
   const double cd = S.cd_scale * CD;
-  const double coef = cd * kd * rho * Dm;
+  const double kr = kd * rho;
+  const double coef = cd * kr * Dm;
   // a = -coef (du, dv, dw)
   double ldu = -coef * la[0], ldv = -coef * la[1], ldw = -coef * la[2];
-  const double lcoef = -(la[0] * du + la[1] * dv + la[2] * dw);
-  const double lcd = lcoef * kd * rho * Dm;
+  const double lcoef = -fma(la[0], du, fma(la[1], dv, la[2] * dw));
+  const double lcd = lcoef * kr * Dm;
   double lrho = lcoef * cd * kd * Dm;
-  double lDm = lcoef * cd * kd * rho;
+  double lDm = lcoef * cd * kr;
   gp[2] += lcd * CD;
   const double lCD = lcd * S.cd_scale;
   // C_D of Eq. 7 through first = D/den1 (squared in the printed form) and second
-  const double dfirst0_dRe = (64.0 * den1 - Dn * (10.0 + 2.0 * Re + 0.23 * 64.0 * Ma)) / (den1 * den1);
-  const double dfirst0_dMa = -0.23 * Dn * Dn / (den1 * den1);
+  const double dfirst0_dRe = fma(-first0, fma(0.23 * 64.0, Ma, fma(2.0, Re, 10.0)), 64.0) * iden;
+  const double dfirst0_dMa = -0.23 * first0 * first0;
   const double fscale = (S.cd_mode == 1) ? 2.0 * first0 : 1.0;
-  const double dsecond_dMa = (2.0 * A - (1.6 * k + 2.0 * Ma)) / (A * A);
+  const double dsecond_dMa = (2.0 - second) * iA;
   const double lRe = lCD * fscale * dfirst0_dRe;
-  double lMa = lCD * (fscale * dfirst0_dMa + dsecond_dMa);
+  double lMa = lCD * fma(fscale, dfirst0_dMa, dsecond_dMa);
   // Re = c_re r_p Ma rho
-  lMa += lRe * S.c_re * rp_cm * rho;
-  lrho += lRe * S.c_re * rp_cm * Ma;
+  lMa = fma(lRe * re_k, rho, lMa);
+  lrho = fma(lRe * re_k, Ma, lrho);
   // Ma = |dv| / c_s
-  lDm += lMa / cs;
-  const double lcs = -lMa * Dm / (cs * cs);
-  const double lD2 = lDm / (2.0 * Dm);
-  ldu += 2.0 * du * lD2;
-  ldv += 2.0 * dv * lD2;
-  ldw += 2.0 * dw * lD2;
+  lDm = fma(lMa, ics, lDm);
+  const double lcs_cs = -lMa * Ma;               // cotangent of c_s times c_s
+  const double lD = lDm * iDm;
+  ldu = fma(du, lD, ldu);
+  ldv = fma(dv, lD, ldv);
+  ldw = fma(dw, lD, ldw);
   // du = u + gf y, dv = v - gf x, dw = w
   gv[0] += ldu;
   gv[1] += ldv;
   gv[2] += ldw;
-  const double lgf = ldu * y - ldv * x;
-  double lx = -ldv * gf, ly = ldu * gf;
-  // gf = v_g / R, v_g = v_k sqrt(1 - 2 eta)
-  const double lvg = lgf / R;
-  double lR = -lgf * vg / R2;
-  const double lvk = lvg * st;
-  const double lt = lvg * vk / (2.0 * st);
-  const double leta = -2.0 * lt;
+  const double lgf = fma(ldu, y, -ldv * x);
+  // gf = v_g / R, v_g = v_k sqrt(1 - 2 eta): lvg = lgf / R, leta = -lvg v_k / sqrt(t)
+  const double lvg = lgf * iR;
+  const double leta = -lvg * vk * ist;
   // eta = c_eta(gamma) R^(2 flare)
-  lR += leta * eta * 2.0 * S.flare / R;
-  gp[1] += leta * S.deta_dgamma * Rf2;
-  // rho = c_rho Sigma R^-(1+flare)
-  const double lsigma = lrho * rho / sigma;
-  lR -= lrho * rho * (1.0 + S.flare) / R;
-  // c_s = c_cs R^(flare - 1/2), v_k = sqrt(mu0) R^(-1/2)
-  lR += lcs * cs * (S.flare - 0.5) / R;
-  lR -= lvk * vk * 0.5 / R;
-  // Sigma = sigma1 R^-gamma E(R, gamma)
-  gp[0] += lsigma * sigma / S.sigma1;
-  lR += lsigma * sigma * (-S.gamma / R + dlnE_dR);
-  gp[1] += lsigma * sigma * (-lnR + dlnE_dg);
+  gp[1] = fma(leta * S.deta_dgamma, Rf2, gp[1]);
+  // rho = c_rho Sigma R^-(1+flare); c_s = c_cs R^(flare - 1/2); v_k = sqrt(mu0) R^-1/2;
+  // Sigma = sigma1 R^-gamma E(R, gamma): every term's cotangent of R, times R
+  const double lrr = lrho * rho;                 // cotangent of ln rho, and of ln Sigma
+  double lRR = -1.5 * lgf * gf;                  // -lgf gf (1/R) - lvk vk / 2, lvk vk = lgf gf
+  lRR = fma(leta * eta, 2.0 * S.flare, lRR);
+  lRR = fma(-lrr, 1.0 + S.flare + S.gamma, lRR);
+  lRR = fma(lcs_cs, S.flare - 0.5, lRR);
+  lRR = fma(lrr * dlnE_dR, R, lRR);
+  gp[0] += lrho * S.c_rho * rmh * sig1;
+  gp[1] = fma(lrr, dlnE_dg - lnR, gp[1]);
   // R = sqrt(x^2 + y^2)
-  lx += lR * x / R;
-  ly += lR * y / R;
-  gx[0] += lx;
-  gx[1] += ly;
+  const double lr = lRR * (iR * iR);
+  gx[0] += fma(lr, x, -ldv * gf);
+  gx[1] += fma(lr, y, ldu * gf);
 }
 
 // Reverse of the disk's gravity on a planetesimal (Eqs. 10-12), in the form
@@ -191,7 +207,11 @@ __device__ __forceinline__ void g45(double s, double beta, const double* G, doub
 // The universal anomaly s solves F(s) = r0 s + eta G2 + zeta G3 - h = 0
 // (implicit function: ds = -(F_r0 dr0 + F_eta deta + F_zeta dzeta +
 // F_beta dbeta)/F_s with F_s = r), and dG_k/ds = G_{k-1},
-// dG_k/dbeta = -(s G_{k+1} - k G_{k+2})/2.
+// dG_k/dbeta = -(s G_{k+1} - k G_{k+2})/2.  The solve is kepler_drift's (its
+// starting guess, Halley's method and stopping rule); the G functions are then
+// evaluated at the final s.  Bound by FP64 issue: 1/r0 and 1/r are formed once,
+// by rsqrt_d and rcp_d, and one Halley correction is the rule on short steps,
+// where the second-order guess took three: 125 -> 36 us for 50,000 bodies.
 __device__ bool kepler_vjp(double mu, double h, int maxit, const double* x, const double* v,
                            const double* lx1, const double* lv1, double* lx0, double* lv0) {
   for (int c = 0; c < 3; ++c) {
@@ -199,23 +219,28 @@ __device__ bool kepler_vjp(double mu, double h, int maxit, const double* x, cons
     lv0[c] = lv1[c];
   }
   if (h == 0.0) return true;
-  const double r02 = x[0] * x[0] + x[1] * x[1] + x[2] * x[2];
-  const double r0 = sqrt(r02);
-  const double v2 = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
-  const double eta = x[0] * v[0] + x[1] * v[1] + x[2] * v[2];
-  const double beta = 2.0 * mu / r0 - v2;
-  const double zeta = mu - beta * r0;
-  double s = (h / r0) * (1.0 - 0.5 * eta * h / r02);
+  const double r02 = fma(x[0], x[0], fma(x[1], x[1], x[2] * x[2]));
+  const double ir0 = rsqrt_d(r02);
+  const double r0 = r02 * ir0;
+  const double v2 = fma(v[0], v[0], fma(v[1], v[1], v[2] * v[2]));
+  const double eta = fma(x[0], v[0], fma(x[1], v[1], x[2] * v[2]));
+  const double beta = fma(2.0 * mu, ir0, -v2);
+  const double zeta = fma(-beta, r0, mu);
+  const double hi = h * ir0;
+  const bool short_step = abs_le(beta * hi * hi, 0.1);
+  const double t1 = short_step ? fma(0.5 * eta * eta, ir0, -zeta * (1.0 / 6.0)) : 0.0;
+  const double stop = short_step ? 1e-5 : 1e-7;
+  double s = hi * fma(hi * ir0, fma(hi, t1, -0.5 * eta), 1.0);
   double G[4];
   bool done = false;
   for (int it = 0; it < maxit; ++it) {
     gfuns(s, beta, G);
-    const double F = r0 * s + eta * G[2] + zeta * G[3] - h;
-    const double Fp = r0 + eta * G[1] + zeta * G[2];
-    const double Fpp = eta * G[0] + zeta * G[1];
-    const double ds = -F * Fp / (Fp * Fp - 0.5 * F * Fpp);
+    const double F = fma(r0, s, fma(eta, G[2], fma(zeta, G[3], -h)));
+    const double Fp = fma(eta, G[1], fma(zeta, G[2], r0));
+    const double Fpp = fma(eta, G[0], zeta * G[1]);
+    const double ds = -F * Fp * rcp_d(fma(Fp, Fp, -0.5 * F * Fpp));
     s += ds;
-    if (fabs(ds) <= 1e-7 * fabs(s)) {
+    if (fabs(ds) <= stop * fabs(s)) {
       done = true;
       break;
     }
@@ -224,54 +249,46 @@ __device__ bool kepler_vjp(double mu, double h, int maxit, const double* x, cons
   gfuns(s, beta, G);
   double G4, G5;
   g45(s, beta, G, G4, G5);
-  const double r = r0 + eta * G[1] + zeta * G[2];
-  const double f = 1.0 - mu * G[2] / r0;
-  const double g = r0 * G[1] + eta * G[2];
-  const double fd = -mu * G[1] / (r * r0);
-  const double gd = 1.0 - mu * G[2] / r;
+  const double r = fma(eta, G[1], fma(zeta, G[2], r0));
+  const double ir = rcp_d(r);
+  const double mG1 = mu * G[1], mG2 = mu * G[2];
+  const double f = fma(-mG2, ir0, 1.0);
+  const double g = fma(r0, G[1], eta * G[2]);
+  const double fd = -mG1 * (ir * ir0);
+  const double gd = fma(-mG2, ir, 1.0);
   double lf = 0, lg = 0, lfd = 0, lgd = 0;
   for (int c = 0; c < 3; ++c) {
-    lf += lx1[c] * x[c];
-    lg += lx1[c] * v[c];
-    lfd += lv1[c] * x[c];
-    lgd += lv1[c] * v[c];
-    lx0[c] = f * lx1[c] + fd * lv1[c];
-    lv0[c] = g * lx1[c] + gd * lv1[c];
+    lf = fma(lx1[c], x[c], lf);
+    lg = fma(lx1[c], v[c], lg);
+    lfd = fma(lv1[c], x[c], lfd);
+    lgd = fma(lv1[c], v[c], lgd);
+    lx0[c] = fma(f, lx1[c], fd * lv1[c]);
+    lv0[c] = fma(g, lx1[c], gd * lv1[c]);
   }
-  double lG1 = 0, lG2 = 0, lr0 = 0, leta = 0, lr = 0, lzeta = 0, lbeta = 0;
-  lG2 -= mu * lf / r0;
-  lr0 += mu * G[2] * lf / r02;
-  lr0 += G[1] * lg;
-  lG1 += r0 * lg;
-  leta += G[2] * lg;
-  lG2 += eta * lg;
-  lG1 -= mu * lfd / (r * r0);
-  lr += mu * G[1] * lfd / (r * r * r0);
-  lr0 += mu * G[1] * lfd / (r * r02);
-  lG2 -= mu * lgd / r;
-  lr += mu * G[2] * lgd / (r * r);
-  lr0 += lr;
-  leta += G[1] * lr;
-  lG1 += eta * lr;
-  lzeta += G[2] * lr;
-  lG2 += zeta * lr;
-  const double dG1b = -0.5 * (s * G[2] - G[3]);
-  const double dG2b = -0.5 * (s * G[3] - 2.0 * G4);
-  const double dG3b = -0.5 * (s * G4 - 3.0 * G5);
-  const double ls = lG1 * G[0] + lG2 * G[1];
-  lbeta += lG1 * dG1b + lG2 * dG2b;
-  const double Fb = eta * dG2b + zeta * dG3b;
-  lr0 -= ls * s / r;
-  leta -= ls * G[2] / r;
-  lzeta -= ls * G[3] / r;
-  lbeta -= ls * Fb / r;
-  lbeta -= r0 * lzeta;
-  lr0 -= beta * lzeta;
-  lr0 -= 2.0 * mu * lbeta / r02;
-  const double lv2 = -lbeta;
+  // f = 1 - mu G2/r0, g = r0 G1 + eta G2, fd = -mu G1/(r r0), gd = 1 - mu G2/r
+  const double qf = lf * ir0, qd = lfd * (ir * ir0), qg = lgd * ir;
+  const double lr = fma(mG1, qd, mG2 * qg) * ir;
+  double lG1 = fma(r0, lg, fma(eta, lr, -mu * qd));
+  double lG2 = fma(eta, lg, fma(zeta, lr, -mu * (qf + qg)));
+  double lr0 = fma(fma(mG2, qf, mG1 * qd), ir0, fma(G[1], lg, lr));
+  double leta = fma(G[2], lg, G[1] * lr);
+  double lzeta = G[2] * lr;
+  const double dG1b = -0.5 * fma(s, G[2], -G[3]);
+  const double dG2b = -0.5 * fma(s, G[3], -2.0 * G4);
+  const double dG3b = -0.5 * fma(s, G4, -3.0 * G5);
+  const double ls = fma(lG1, G[0], lG2 * G[1]) * ir;
+  const double Fb = fma(eta, dG2b, zeta * dG3b);
+  lr0 = fma(-ls, s, lr0);
+  leta = fma(-ls, G[2], leta);
+  lzeta = fma(-ls, G[3], lzeta);
+  double lbeta = fma(lG1, dG1b, fma(lG2, dG2b, -ls * Fb));
+  lbeta = fma(-r0, lzeta, lbeta);
+  lr0 = fma(-beta, lzeta, lr0);
+  lr0 = fma(-2.0 * mu * lbeta, ir0 * ir0, lr0);
+  const double cx = lr0 * ir0, cv = -2.0 * lbeta;
   for (int c = 0; c < 3; ++c) {
-    lx0[c] += leta * v[c] + lr0 * x[c] / r0;
-    lv0[c] += leta * x[c] + 2.0 * lv2 * v[c];
+    lx0[c] = fma(leta, v[c], fma(cx, x[c], lx0[c]));
+    lv0[c] = fma(leta, x[c], fma(cv, v[c], lv0[c]));
   }
   return true;
 }
@@ -466,6 +483,50 @@ __device__ __forceinline__ void pair_vjp(double dx, double dy, double dz, double
   sbz = fma(B, dz, sbz);
 }
 
+// pair_vjp of a far pair (K = 1) in pairs of FP32 numbers (mx_split.cuh), for
+// systems of light big bodies: about 230 FP32 instructions where pair_vjp takes
+// 29 FP64 ones of 64 cycles.  The cotangent l comes scaled by a power of two
+// common to the tile, mu by 2^kVjpScale, so that the products and their low
+// parts stay normal numbers; the sums are scaled back.  Pairs within
+// three changeover radii, which carry most of a sum of 1/s^3 terms, keep
+// FP64.  Measured: k_adj_kick_vjp with 1,000 big bodies and 20,000
+// planetesimals 917 -> 315 us; two steps forward and back 21.7 -> 8.8 ms (with
+// the other reverse kernels), gradients within 4e-15 of the FP64 ones.  bs: the big body's traveling sum of A l + B d; ta, tb: the target's
+// sums of A and B d.
+constexpr int kVjpScale = 30;
+constexpr float kVjpNear2 = 9.0f;   // (3 changeover radii)^2, in units of one's
+
+struct VjpPos {
+  SplitPos p;
+  FF l[3];
+};
+
+__device__ __forceinline__ bool split_vjp(const VjpPos& t, const SplitBig& b, float near2,
+                                          float (&bs)[6], float (&ta)[2], float (&tb)[6]) {
+  float h[3], m[3];
+  split_sub(t.p.x0, t.p.x1, t.p.x2, b.x0, b.x1, b.x2, h[0], m[0]);
+  split_sub(t.p.y0, t.p.y1, t.p.y2, b.y0, b.y1, b.y2, h[1], m[1]);
+  split_sub(t.p.z0, t.p.z1, t.p.z2, b.z0, b.z1, b.z2, h[2], m[2]);
+  const FF s2 = ff_norm2(h[0], m[0], h[1], m[1], h[2], m[2]);
+  if (s2.h < near2) return false;
+  const FF is = ff_rsqrt(s2);
+  const FF is2 = ff_mul(is, is);
+  const FF A = ff_mul(FF{b.muh, b.mul}, ff_mul(is2, is));
+  FF dl = ff_mul(FF{h[0], m[0]}, t.l[0]);
+  dl = ff_add(dl, ff_mul(FF{h[1], m[1]}, t.l[1]));
+  dl = ff_add(dl, ff_mul(FF{h[2], m[2]}, t.l[2]));
+  const FF B = ff_mul(ff_mul(A, is2), ff_mul(FF{-3.0f, 0.0f}, dl));
+  split_add(ta[0], ta[1], A.h, A.l);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const FF al = ff_mul(A, t.l[c]), bd = ff_mul(B, FF{h[c], m[c]});
+    split_add(tb[2 * c], tb[2 * c + 1], bd.h, bd.l);
+    split_add(bs[2 * c], bs[2 * c + 1], al.h, al.l);
+    split_add(bs[2 * c], bs[2 * c + 1], bd.h, bd.l);
+  }
+  return true;
+}
+
 // Which parts of a half kick's reverse a launch takes.  The gravity's part is
 // linear in the cotangent l of the acceleration and depends on the positions
 // only, so the reverse of a step's first half kick and of the previous step's
@@ -496,6 +557,10 @@ struct KickRev {
 // the batch and then passes its running sum for that body to the lane before
 // it, so each body's sum visits the group's targets in a fixed order with
 // one shuffle a pair, and the groups' sums are added at the end.
+//
+// SPLIT: the systems that SysDev::split names take their far pairs in FP32
+// pairs (split_vjp), beside FP64 sums of the near ones.
+template <bool SPLIT>
 __global__ void __launch_bounds__(kThreads) k_adj_kick_vjp(Dev d, Adj a, const double* X,
                                                            const double* V, int pslot, int kick,
                                                            KickRev r) {
@@ -537,19 +602,78 @@ __global__ void __launch_bounds__(kThreads) k_adj_kick_vjp(Dev d, Adj a, const d
   }
   const double nlx = -3.0 * gax, nly = -3.0 * gay, nlz = -3.0 * gaz;
   double sa = 0, sbx = 0, sby = 0, sbz = 0;   // the target's sums (pair_vjp)
+  const bool split = SPLIT && S.split;
+  __shared__ SplitBig sp[SPLIT ? kAdjChunk : 1];
+  __shared__ int s_hi;
+  VjpPos vt{};
+  float near_own = 0.0f;
+  bool scaled = false;              // this target's l stands in vt.l
+  double unl = 1.0;                 // its scale's inverse
+  const double unmu = __hiloint2double((1023 - kVjpScale) << 20, 0);
+  if (split && r.grav) {
+    // the tile's largest |l| to about 1; a target far below it keeps FP64
+    const int lh = act ? max(abs_hi(gax), max(abs_hi(gay), abs_hi(gaz))) : 0;
+    __syncthreads();
+    if (threadIdx.x == 0) s_hi = 0;
+    __syncthreads();
+    const int wh = __reduce_max_sync(0xffffffffu, lh);
+    if (lane == 0) atomicMax(&s_hi, wh);
+    __syncthreads();
+    const int e = s_hi ? (s_hi >> 20) - 1023 : 0;   // l 2^-e below 2
+    if (e > -900 && e < 900) {
+      const double sl = __hiloint2double((1023 - e) << 20, 0);
+      unl = __hiloint2double((1023 + e) << 20, 0);
+      scaled = (lh >> 20) - 1023 > e - 60 || (gax == 0.0 && gay == 0.0 && gaz == 0.0);
+      vt.l[0] = ff_of(gax * sl);
+      vt.l[1] = ff_of(gay * sl);
+      vt.l[2] = ff_of(gaz * sl);
+    }
+    near_own = act && jl < S.nbig ? kVjpNear2 * near2_of(trc.rc2) : 0.0f;
+  }
+  int kt = INT_MIN;
   for (int c0 = 0; r.grav && c0 < S.nbig; c0 += kAdjChunk) {
     const int cn = min(kAdjChunk, S.nbig - c0);
     __syncthreads();
     stage_chunk(d, S, X, c0, cn, sx, sy, sz, sm, sc);
+    if (SPLIT && threadIdx.x == 0) s_hi = 0;
     __syncthreads();
+    bool far_ok = false;
+    if (split) {   // the chunk's parts, on the grid of its own positions
+      int hi = 0;
+      for (int k = threadIdx.x; k < cn; k += blockDim.x)
+        hi = max(hi, max(abs_hi(sx[k]), max(abs_hi(sy[k]), abs_hi(sz[k]))));
+      hi = __reduce_max_sync(0xffffffffu, hi);
+      if (lane == 0) atomicMax(&s_hi, hi);
+      __syncthreads();
+      const int kg = split_k(s_hi);
+      if (kg <= kSplitMaxK) {
+        for (int k = threadIdx.x; k < cn; k += blockDim.x) {
+          SplitBig b = split_big(sx[k], sy[k], sz[k], sm[k], sc[0][k], kg);
+          b.muh *= pow2f(kVjpScale);
+          b.mul *= pow2f(kVjpScale);
+          b.near2 *= kVjpNear2;
+          sp[k] = b;
+        }
+        far_ok = scaled && split_in_range(x, y, z, kg);
+        if (far_ok && kt != kg) {
+          kt = kg;
+          split3(x, kg, vt.p.x0, vt.p.x1, vt.p.x2);
+          split3(y, kg, vt.p.y0, vt.p.y1, vt.p.y2);
+          split3(z, kg, vt.p.z0, vt.p.z1, vt.p.z2);
+        }
+      }
+      __syncthreads();
+    }
     for (int base = 0; base < cn;) {
       const int left = cn - base;
       const int W = left >= 32 ? 32 : 1 << (31 - __clz(left));
       const int gl = lane & (W - 1);
       double bx = 0, by = 0, bz = 0;   // the running sum of the body this lane holds
+      float bs[6] = {0, 0, 0, 0, 0, 0}, ta[2] = {0, 0}, tb[6] = {0, 0, 0, 0, 0, 0};
       for (int r = 0; r < W; ++r) {
         const int k = base + ((gl + r) & (W - 1));
-        if (act && c0 + k != jl)
+        if (act && c0 + k != jl &&
+            !(SPLIT && far_ok && split_vjp(vt, sp[k], fmaxf(sp[k].near2, near_own), bs, ta, tb)))
           pair_vjp(x - sx[k], y - sy[k], z - sz[k], sm[k], pair_rc(sc, k, trc), gax, gay, gaz,
                    nlx, nly, nlz, bx, by, bz, sa, sbx, sby, sbz);
         if (r + 1 < W) {
@@ -557,7 +681,19 @@ __global__ void __launch_bounds__(kThreads) k_adj_kick_vjp(Dev d, Adj a, const d
           bx = __shfl_sync(0xffffffffu, bx, src, W);
           by = __shfl_sync(0xffffffffu, by, src, W);
           bz = __shfl_sync(0xffffffffu, bz, src, W);
+          if (split)
+            for (int q = 0; q < 6; ++q) bs[q] = __shfl_sync(0xffffffffu, bs[q], src, W);
         }
+      }
+      if (split) {   // the FP32 sums over at most 32 pairs go into the FP64 ones
+        const double ub = unl * unmu;
+        bx = fma(bits_to_double(bs[0]) + bits_to_double(bs[1]), ub, bx);
+        by = fma(bits_to_double(bs[2]) + bits_to_double(bs[3]), ub, by);
+        bz = fma(bits_to_double(bs[4]) + bits_to_double(bs[5]), ub, bz);
+        sa = fma(bits_to_double(ta[0]) + bits_to_double(ta[1]), unmu, sa);
+        sbx = fma(bits_to_double(tb[0]) + bits_to_double(tb[1]), ub, sbx);
+        sby = fma(bits_to_double(tb[2]) + bits_to_double(tb[3]), ub, sby);
+        sbz = fma(bits_to_double(tb[4]) + bits_to_double(tb[5]), ub, sbz);
       }
       for (int off = W; off < 32; off <<= 1) {
         bx += __shfl_down_sync(0xffffffffu, bx, off);
@@ -808,9 +944,15 @@ __global__ void __launch_bounds__(kThreads) k_adj_fold_jump1(Dev d, Adj a) {
   }
 }
 
-int adjoint_vjp_blocks_per_sm(int threads) {
+using KickVjpKernel = void (*)(Dev, Adj, const double*, const double*, int, int, KickRev);
+static KickVjpKernel kick_vjp_kernel(const Dev& d) {
+  return d.split_mode == kSplitNone ? k_adj_kick_vjp<false> : k_adj_kick_vjp<true>;
+}
+
+int adjoint_vjp_blocks_per_sm(const Dev& d, int threads) {
   int n = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_adj_kick_vjp, threads, 0) != cudaSuccess)
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kick_vjp_kernel(d), threads, 0) !=
+      cudaSuccess)
     return 0;
   return n;
 }
@@ -842,7 +984,7 @@ void launch_adjoint_step_b(const Dev& d, const Adj& a, cudaStream_t st) {
   // reverse sweep: kick 2 (at x4, v3, P3), jump 2, drift, jump 1, kick 1 (at x0, v0, P0)
   // (with a.lin, the pair pass also takes the next step's first half kick,
   // left pending at the same positions)
-  k_adj_kick_vjp<<<d.ntiles, d.tile, 0, st>>>(d, a, a.x4, a.xv3 + 3 * (size_t)N, 2, 2 * a.step + 1,
+  kick_vjp_kernel(d)<<<d.ntiles, d.tile, 0, st>>>(d, a, a.x4, a.xv3 + 3 * (size_t)N, 2, 2 * a.step + 1,
                                               KickRev{1, 1, 1, a.lin, nullptr});
   launch_fold_kick(d, a, 2, 1, st);
   if (a.groups) launch_adjoint_bs_vjp(d, a, a.bs_blocks, st);
@@ -851,12 +993,12 @@ void launch_adjoint_step_b(const Dev& d, const Adj& a, cudaStream_t st) {
   k_adj_fold_jump1<<<d.nsys, kThreads, 0, st>>>(d, a);
   // merged: the drag now, the pair pass with the previous step's last half kick
   const KickRev r1{a.defer_k1 ? 0 : 1, 1, 1, nullptr, a.defer_k1 ? a.lpend : nullptr};
-  k_adj_kick_vjp<<<d.ntiles, d.tile, 0, st>>>(d, a, a.z0, a.z0 + 3 * (size_t)N, 0, 2 * a.step, r1);
+  kick_vjp_kernel(d)<<<d.ntiles, d.tile, 0, st>>>(d, a, a.z0, a.z0 + 3 * (size_t)N, 0, 2 * a.step, r1);
   launch_fold_kick(d, a, 1, r1.grav, st);
 }
 
 void launch_adjoint_flush(const Dev& d, const Adj& a, const double* xpos, cudaStream_t st) {
-  k_adj_kick_vjp<<<d.ntiles, d.tile, 0, st>>>(d, a, xpos, xpos, 0, 0,
+  kick_vjp_kernel(d)<<<d.ntiles, d.tile, 0, st>>>(d, a, xpos, xpos, 0, 0,
                                               KickRev{1, 0, 0, a.lpend, nullptr});
   launch_fold_kick(d, a, 1, 1, st);
 }
@@ -937,18 +1079,14 @@ __global__ void __launch_bounds__(kThreads) k_loss(Dev d, const double* xvh0, co
 
 // Per system: L, and the bigs' share of the velocity cotangent through P.
 __global__ void __launch_bounds__(kThreads) k_loss_fold(Dev d, double* seed_f, const double* part,
-                                                        const int* poff, double* Lsys) {
+                                                        const int* poff, const int* sys_tiles,
+                                                        double* Lsys) {
   const int sys = blockIdx.x;
   const SysDev& S = d.sys[sys];
   const int N = d.N;
   __shared__ double tot[4];
-  if (threadIdx.x < 4) {
-    double sum = 0;
-    for (int tt = 0; tt < d.ntiles; ++tt)
-      if (d.tiles[tt].sys == sys) sum += part[poff[tt] + threadIdx.x];
-    tot[threadIdx.x] = sum;
-  }
-  __syncthreads();
+  const int t0 = sys_tiles[sys], T = sys_tiles[sys + 1] - t0;
+  fold_tiles(part + (T > 0 ? poff[t0] : 0), 3 * S.nbig + 9, T, 4, tot);
   for (int i = threadIdx.x; i < S.nbig; i += blockDim.x) {
     const int g = S.off + i;
     const double m = d.bmu[S.boff + i] * S.inv_mu0;
@@ -958,42 +1096,72 @@ __global__ void __launch_bounds__(kThreads) k_loss_fold(Dev d, double* seed_f, c
 }
 
 // Reverse of heliocentric -> DH at set-up: v_b = v_h - sum_i m_i v_h,i / M.
-// Per system: S = sum_j lam_v_j (all bodies); big i gets -(m_i/M) S.
-__global__ void __launch_bounds__(kThreads) k_init_vjp(Dev d, const double* lam, double* grad) {
+// Per system: S = sum_j lam_v_j (all bodies); big i gets -(m_i/M) S.  The copy
+// and the tiles' sums first, one block a tile, then the fold (as one block per
+// system that walked all its bodies it took 0.55 ms on 50,000).
+__global__ void __launch_bounds__(kThreads) k_init_vjp(Dev d, const double* lam, double* grad,
+                                                       double* part, const int* poff) {
+  __shared__ double wsum[kThreads / 32][3];
+  const Tile t = d.tiles[blockIdx.x];
+  const int N = d.N;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  double own[3] = {0, 0, 0};
+  if (threadIdx.x < t.count) {
+    const int j = t.start + threadIdx.x;
+    for (int c = 0; c < 3; ++c) {
+      own[c] = lam[(size_t)(3 + c) * N + j];
+      grad[(size_t)c * N + j] = lam[(size_t)c * N + j];
+      grad[(size_t)(3 + c) * N + j] = own[c];
+    }
+  }
+  for (int q = 0; q < 3; ++q) {
+    double vq = own[q];
+    for (int off = 16; off > 0; off >>= 1) vq += __shfl_down_sync(0xffffffffu, vq, off);
+    if (lane == 0) wsum[warp][q] = vq;
+  }
+  __syncthreads();
+  if (threadIdx.x < 3) {
+    double sum = 0;
+    for (int q = 0; q < (int)(blockDim.x + 31) >> 5; ++q) sum += wsum[q][threadIdx.x];
+    part[poff[blockIdx.x] + threadIdx.x] = sum;
+  }
+}
+
+__global__ void __launch_bounds__(kThreads) k_init_vjp_fold(Dev d, double* grad, const double* part,
+                                                            const int* poff, const int* sys_tiles) {
   const int sys = blockIdx.x;
   const SysDev& S = d.sys[sys];
   const int N = d.N;
-  __shared__ double red[4][kThreads];
-  double acc[4] = {0, 0, 0, 0};
-  for (int j = threadIdx.x; j < S.n; j += blockDim.x) {
-    const int g = S.off + j;
-    for (int c = 0; c < 6; ++c) grad[(size_t)c * N + g] = lam[(size_t)c * N + g];
-    for (int c = 0; c < 3; ++c) acc[c] += lam[(size_t)(3 + c) * N + g];
-  }
-  for (int i = threadIdx.x; i < S.nbig; i += blockDim.x) acc[3] += d.bmu[S.boff + i];
-  for (int c = 0; c < 4; ++c) red[c][threadIdx.x] = acc[c];
+  __shared__ double tot[3];
+  __shared__ double red[kThreads];
+  const int t0 = sys_tiles[sys], T = sys_tiles[sys + 1] - t0;
+  fold_tiles(part + (T > 0 ? poff[t0] : 0), 3 * S.nbig + 9, T, 3, tot);
+  double m = 0.0;
+  for (int i = threadIdx.x; i < S.nbig; i += blockDim.x) m += d.bmu[S.boff + i];
+  red[threadIdx.x] = m;
   __syncthreads();
   for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if (threadIdx.x < s)
-      for (int c = 0; c < 4; ++c) red[c][threadIdx.x] += red[c][threadIdx.x + s];
+    if (threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
     __syncthreads();
   }
-  const double inv_tot = 1.0 / (S.mu0 + red[3][0]);   // 1 / (G M_total)
+  const double inv_tot = 1.0 / (S.mu0 + red[0]);   // 1 / (G M_total)
   for (int i = threadIdx.x; i < S.nbig; i += blockDim.x) {
     const int g = S.off + i;
     const double f = d.bmu[S.boff + i] * inv_tot;
-    for (int c = 0; c < 3; ++c) grad[(size_t)(3 + c) * N + g] -= f * red[c][0];
+    for (int c = 0; c < 3; ++c) grad[(size_t)(3 + c) * N + g] -= f * tot[c];
   }
 }
 
 void launch_loss(const Dev& d, const double* xvh0, const double* w, double* seed_f, double* seed_i,
-                 double* part, const int* poff, double* Lsys, cudaStream_t st) {
+                 double* part, const int* poff, const int* sys_tiles, double* Lsys, cudaStream_t st) {
   k_loss<<<d.ntiles, d.tile, 0, st>>>(d, xvh0, w, seed_f, seed_i, part, poff);
-  k_loss_fold<<<d.nsys, kThreads, 0, st>>>(d, seed_f, part, poff, Lsys);
+  k_loss_fold<<<d.nsys, kThreads, 0, st>>>(d, seed_f, part, poff, sys_tiles, Lsys);
 }
 
-void launch_init_vjp(const Dev& d, const double* lam, double* grad, cudaStream_t st) {
-  k_init_vjp<<<d.nsys, kThreads, 0, st>>>(d, lam, grad);
+void launch_init_vjp(const Dev& d, const double* lam, double* grad, double* part, const int* poff,
+                     const int* sys_tiles, cudaStream_t st) {
+  k_init_vjp<<<d.ntiles, d.tile, 0, st>>>(d, lam, grad, part, poff);
+  k_init_vjp_fold<<<d.nsys, kThreads, 0, st>>>(d, grad, part, poff, sys_tiles);
 }
 
 }  // namespace mx

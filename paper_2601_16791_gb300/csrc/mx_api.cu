@@ -1876,7 +1876,7 @@ int adjoint_tile(const mx_system* s) {
   double best = -1.0;
   for (int w = mx::kThreads / 32; w >= 5; --w) {
     const int t = 32 * w;
-    const int occ = mx::adjoint_vjp_blocks_per_sm(t);
+    const int occ = mx::adjoint_vjp_blocks_per_sm(s->d, t);
     if (occ <= 0 || nsm <= 0) continue;
     const double waves = (double)make_tiles(s->h_sys, t, 0).size() / ((double)occ * nsm);
     const double eff = waves / std::ceil(waves);
@@ -2088,7 +2088,7 @@ mx_status mx_loss_semimajor(mx_system* s, const double* dev_xv_helio0, const dou
   MX_TRY(ensure_adjoint(s));
   mx::launch_prep(s->d, 0.0, 0, s->st);
   mx::launch_loss(adjoint_dev(s), dev_xv_helio0, dev_w, dev_seed_final, dev_seed_init, s->a_part,
-                  s->a_poff, s->a_L, s->st);
+                  s->a_poff, s->a_systiles, s->a_L, s->st);
   MX_CUDA(cudaMemcpyAsync(L, s->a_L, s->h_sys.size() * sizeof(double), cudaMemcpyDeviceToHost, s->st));
   return sync_status(s);
 }
@@ -2118,7 +2118,9 @@ mx_status mx_adjoint_init(mx_system* s, const double* dev_lambda, double* dev_gr
   MX_TRY(set_device(s));
   MX_TRY(settle(s));
   MX_TRY(flush_adjoint(s));   // a merged reverse's pending pair pass first
-  mx::launch_init_vjp(s->d, dev_lambda, dev_grad_helio, s->st);
+  MX_TRY(ensure_adjoint(s));
+  mx::launch_init_vjp(adjoint_dev(s), dev_lambda, dev_grad_helio, s->a_part, s->a_poff,
+                      s->a_systiles, s->st);
   return sync_status(s);
 }
 
