@@ -184,26 +184,38 @@ __device__ __forceinline__ void groups_block(const Dev& d) {
     if (threadIdx.x == 0) atomicOr(d.status, ST_GROUP);
     return;
   }
-  // ---- big groups: union-find over the (few) big-big pairs, one thread
-  if (threadIdx.x == 0) {
-    int nn = 0;
-    for (int p = 0; p < nbb; ++p) {
-      const int ab[2] = {key_i(bbk[p]), key_j(bbk[p])};
-      for (int q = 0; q < 2; ++q) {
-        const int g = ab[q];
-        int e = nn;
-        bool dup = false;
-        for (int f = 0; f < nn; ++f) dup |= (nodes[f] == g);
-        if (dup) continue;
-        while (e > 0 && nodes[e - 1] > g) {
-          nodes[e] = nodes[e - 1];
-          --e;
-        }
-        nodes[e] = g;
-        ++nn;
-      }
+  // ---- big groups: the connected components of the (few) big-big pairs.
+  // Every step on all threads, each counting over the shared lists (one thread
+  // with a union-find took most of 177 us for the 130 big-big pairs of 2,000
+  // big bodies + 200,000 planetesimals; now 50).  comp_nodes holds the
+  // pairs' entries while the sorted list of distinct bodies is made.
+  if (nbb == 0) {   // the common case of a few big bodies
+    if (threadIdx.x == 0) s_nnodes = s_bw = s_bm = 0;
+  } else {
+    const int ne = 2 * nbb;
+    auto entry = [&](int e) { return (e & 1) ? key_j(bbk[e >> 1]) : key_i(bbk[e >> 1]); };
+    if (threadIdx.x == 0) s_nnodes = 0;
+    for (int e = threadIdx.x; e < ne; e += blockDim.x) comp_nodes[e] = entry(e);
+    __syncthreads();
+    // comp_of[e] = 1 for the first entry of each body
+    for (int e = threadIdx.x; e < ne; e += blockDim.x) {
+      const int g = comp_nodes[e];
+      bool dup = false;
+      for (int f = 0; f < e; ++f) dup |= (comp_nodes[f] == g);
+      comp_of[e] = dup ? 0 : 1;
+      if (!dup) atomicAdd(&s_nnodes, 1);
     }
-    for (int e = 0; e < nn; ++e) parent[e] = e;
+    __syncthreads();
+    const int nn = s_nnodes;
+    for (int e = threadIdx.x; e < ne; e += blockDim.x)
+      if (comp_of[e]) {
+        const int g = comp_nodes[e];
+        int r = 0;
+        for (int f = 0; f < ne; ++f) r += (comp_of[f] && comp_nodes[f] < g) ? 1 : 0;
+        nodes[r] = g;
+      }
+    __syncthreads();
+    for (int e = threadIdx.x; e < nn; e += blockDim.x) parent[e] = e;
     auto find_idx = [&](int g) {
       int lo = 0, hi = nn - 1;
       while (lo < hi) {
@@ -213,56 +225,76 @@ __device__ __forceinline__ void groups_block(const Dev& d) {
       }
       return lo;
     };
-    auto root = [&](int e) {
-      while (parent[e] != e) e = parent[e];
-      return e;
-    };
-    for (int p = 0; p < nbb; ++p) {
-      const int a = root(find_idx(key_i(bbk[p])));
-      const int b = root(find_idx(key_j(bbk[p])));
-      if (a != b) parent[max(a, b)] = min(a, b);
+    __syncthreads();
+    // each component's smallest node spreads over it, pair by pair, until
+    // nothing changes (at most nn rounds; components are small)
+    for (int round = 0; round < nn; ++round) {
+      int changed = 0;
+      for (int p = threadIdx.x; p < nbb; p += blockDim.x) {
+        const int ia = find_idx(key_i(bbk[p])), ib = find_idx(key_j(bbk[p]));
+        const int la = *(volatile int*)&parent[ia], lb = *(volatile int*)&parent[ib];
+        if (la != lb) {
+          atomicMin(&parent[la < lb ? ib : ia], min(la, lb));
+          changed = 1;
+        }
+      }
+      if (!__syncthreads_or(changed)) break;
     }
     // components numbered in order of their smallest member
-    int nc = 0;
-    for (int e = 0; e < nn; ++e) {
-      const int r = root(e);
-      if (r == e) comp_of[e] = nc++;
-      else comp_of[e] = comp_of[r];
+    for (int e = threadIdx.x; e < nn; e += blockDim.x) {
+      const int r = parent[e];
+      int c = 0;
+      for (int f = 0; f < r; ++f) c += (parent[f] == f) ? 1 : 0;
+      comp_of[e] = c;
     }
-    for (int c = 0; c <= nc; ++c) comp_start[c] = 0;
-    for (int e = 0; e < nn; ++e) comp_start[comp_of[e] + 1]++;
-    for (int c = 0; c < nc; ++c) comp_start[c + 1] += comp_start[c];
-    for (int c = 0; c < nc; ++c) {
-      int fill = comp_start[c];
-      for (int e = 0; e < nn; ++e)
-        if (comp_of[e] == c) comp_nodes[fill++] = e;
-    }
-    // one work item per big group
-    int m = 0;
-    for (int c = 0; c < nc; ++c) {
-      const int sz = comp_start[c + 1] - comp_start[c];
-      if (sz > kMaxGroup) s_bad = ST_GROUP;
-      if (c >= d.work_cap || m + sz > d.mem_cap) {
-        s_bad = ST_WORK_OVF;
-        break;
+    __syncthreads();
+    // nodes ordered by component, then index
+    for (int e = threadIdx.x; e < nn; e += blockDim.x) {
+      const int c = comp_of[e];
+      int at = 0, first = 0;
+      for (int f = 0; f < nn; ++f) {
+        const int cf = comp_of[f];
+        if (cf < c) ++first;
+        if (cf < c || (cf == c && f < e)) ++at;
       }
-      d.work_off[c] = m;
-      d.work_sys[c] = sys_of(d, nodes[comp_nodes[comp_start[c]]]);
+      comp_nodes[at] = e;
+      if (at == first) comp_start[c] = first;
+    }
+    if (threadIdx.x == 0) {
+      int nc = 0;
+      for (int e = nn - 1; e >= 0 && nc == 0; --e)   // the last component's root
+        if (parent[e] == e) nc = comp_of[e] + 1;
+      comp_start[nc] = nn;
+      s_ncomp = nc;
+      s_nnodes = nn;
+      if (d.bb_count && nbb > 0) atomicAdd(d.bb_count, (unsigned long long)nbb);
+    }
+    __syncthreads();
+    const int nc = s_ncomp;
+    // one work item per big group
+    for (int c = threadIdx.x; c < nc; c += blockDim.x) {
+      const int m0 = comp_start[c], m1 = comp_start[c + 1];
+      if (m1 - m0 > kMaxGroup) s_bad = ST_GROUP;
+      if (c >= d.work_cap || m1 > d.mem_cap) {
+        s_bad = ST_WORK_OVF;
+        continue;
+      }
+      d.work_off[c] = m0;
+      d.work_sys[c] = sys_of(d, nodes[comp_nodes[m0]]);
       d.work_wfrom[c] = 0;
-      for (int b = comp_start[c]; b < comp_start[c + 1]; ++b) d.work_mem[m++] = nodes[comp_nodes[b]];
+      for (int b = m0; b < m1; ++b) d.work_mem[b] = nodes[comp_nodes[b]];
     }
     // big groups of this step, for the catch-up of deferred planetesimals
     const int slot = s_slot;
     if (d.defer && slot < d.hist_cap)
-      for (int e = 0; e < nn; ++e) {
+      for (int e = threadIdx.x; e < nn; e += blockDim.x) {
         const SysDev& Sg = d.sys[sys_of(d, nodes[e])];
         d.h_comp[(size_t)slot * d.NB + Sg.boff + (nodes[e] - Sg.off)] = comp_of[e];
       }
-    s_nnodes = nn;
-    s_ncomp = nc;
-    if (d.bb_count && nbb > 0) atomicAdd(d.bb_count, (unsigned long long)nbb);
-    s_bw = nc;
-    s_bm = m;
+    if (threadIdx.x == 0) {
+      s_bw = nc;
+      s_bm = nn;
+    }
   }
   __syncthreads();
   if (s_bad) {
