@@ -93,7 +93,8 @@ __device__ __forceinline__ SplitBig split_big(double x, double y, double z, doub
   const FF m = ff_of(mu);
   b.muh = m.h;
   b.mul = m.l;
-  b.near2 = near2_of(rc2);
+  // a mass off FP32's range: no pair of it is a far one
+  b.near2 = split_mass(mu) ? near2_of(rc2) : __int_as_float(0x7f800000);
   return b;
 }
 

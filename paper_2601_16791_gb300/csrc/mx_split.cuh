@@ -156,22 +156,26 @@ __device__ __forceinline__ FF ff_rcp(FF x) {
   return ff_fast(y, __fmul_rn(y, __fmaf_rn(e, e, e)));
 }
 
-// A double's leading 48 bits, read off its bit pattern (zero below 2^-126;
-// valid for |x| < 2^127).  Integer and FP32 instructions only.
+// A double's leading 48 bits, read off its bit pattern (zero below 2^-126; a
+// NaN from 2^127 on, infinities and NaNs among them, so that the kick still
+// reports them).  Integer and FP32 instructions only.
 __device__ __forceinline__ FF ff_of(double x) {
   const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
   const unsigned a = hi & 0x7fffffffu, sg = hi & 0x80000000u;
   if (a < (897u << 20)) return FF{0.0f, 0.0f};
+  if (a >= (1150u << 20)) return FF{__uint_as_float(0x7fc00000u), 0.0f};
   const float h = __uint_as_float(sg | ((a - (896u << 20)) << 3) | (lo >> 29));
   const float r = __fmul_rn(__uint2float_rn(lo & 0x1fffffffu), 0x1p-52f);
   const float sc = __uint_as_float(sg | (((a >> 20) - 896u) << 23));
   return FF{h, __fmul_rn(r, sc)};
 }
 
-// A float as a double, exactly, by moving its bits (zero for a subnormal).
+// A float as a double, exactly, by moving its bits (zero for a subnormal, a
+// NaN for an infinity).
 __device__ __forceinline__ double bits_to_double(float f) {
   const unsigned u = __float_as_uint(f), a = u & 0x7fffffffu;
   if (a < 0x00800000u) return 0.0;
+  if (a >= 0x7f800000u) return __hiloint2double(0x7ff80000, 0);
   return __hiloint2double((int)((u & 0x80000000u) | ((a >> 3) + (896u << 20))), (int)(a << 29));
 }
 
@@ -190,8 +194,17 @@ struct SplitAcc {
   float xh, xl, yh, yl, zh, zl;
 };
 
+// At least (1e-6 AU)^2: mu/s^3 and the reverse's mu/s^5 stay in FP32's range.
 __device__ __forceinline__ float near2_of(double rc2) {
-  return fmaxf(to_float_bits(rc2) * 1.0001f, 1e-30f);
+  return fmaxf(to_float_bits(rc2) * 1.0001f, 1e-12f);
+}
+
+// Whether the products of mu with powers of a far pair's 1/s keep their parts
+// normal FP32 numbers: zero, or between 1e-18 and 1e3 (a body of 1e-14 of the
+// Sun has 3e-18 AU^3/d^2); false for a NaN.
+__device__ __forceinline__ bool split_mass(double mu) {
+  const int hi = abs_hi(mu);
+  return (hi >= 0x3c327000 && hi < 0x408f4000) || (hi == 0 && __double2loint(mu) == 0);
 }
 
 // A two-sum into the pair (h, l), with the term's low part.

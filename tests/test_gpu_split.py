@@ -127,3 +127,32 @@ def test_split_drag_against_fp64(nbig, nsmall, gas):
     bound = 3e-16 * np.linalg.norm(v0, axis=0) + TOL * h2 * (W.G * w.m_big / s2).sum(1)
     bound[nbig:] += 1e-12 * h2 * np.linalg.norm(drag.cpu().numpy(), axis=0)
     assert (err / bound).max() <= 1.0, (err / bound).max()
+
+
+def test_split_keeps_what_fp32_cannot_hold():
+    """Masses below FP32's range keep FP64's accuracy in mx_accel (bound: two
+    roundings a pair and one of each partial sum, 65 x 2^-52 of the pairs'
+    magnitudes), and a drag without bound is reported, not rounded away."""
+    w = W.semiactive_2000big_200k(seed=3, nbig=65, nsmall=300)
+    w.m_big *= 1e-24
+    g = mx.System(w)
+    start = torch.empty((6, w.n), dtype=torch.float64, device="cuda")
+    acc = torch.empty((3, w.n), dtype=torch.float64, device="cuda")
+    mx.mx_get_state_device(g.h, start)
+    mx.mx_accel(g.h, acc)
+    g.close()
+    x = start[:3].cpu().numpy()
+    d = x[:, :, None] - x[:, None, :65]
+    s2 = (d * d).sum(0)
+    s2[s2 == 0] = np.inf
+    f = W.G * w.m_big / (s2 * np.sqrt(s2))
+    err = np.linalg.norm(acc.cpu().numpy() + (f * d).sum(2), axis=0)
+    assert (err / (W.G * w.m_big / s2).sum(1)).max() <= 65 * 2.0 ** -52
+    w = W.gas_4core_100k(seed=5, nbig=4, nsmall=500)
+    w.m_big *= 1e-3
+    w.rp_km[7] = 0.0
+    g = mx.System(w)
+    with pytest.raises(mx.MxError) as e:
+        g.step(1)
+    g.close()
+    assert e.value.code == 7   # MX_ERR_NONFINITE
