@@ -18,7 +18,6 @@
 #include "mx_kepler.cuh"
 #include "mx_kernels.h"
 #include "mx_physics.cuh"
-#include "mx_kick_body.cuh"
 
 namespace mx {
 
@@ -252,18 +251,20 @@ __device__ bool kepler_vjp(double mu, double h, int maxit, const double* x, cons
   const double r = fma(eta, G[1], fma(zeta, G[2], r0));
   const double ir = rcp_d(r);
   const double mG1 = mu * G[1], mG2 = mu * G[2];
-  const double f = fma(-mG2, ir0, 1.0);
+  // f - 1 and gd - 1, small on a short step: their roundings do not reach the
+  // cotangents' last places
+  const double f1 = -mG2 * ir0;
   const double g = fma(r0, G[1], eta * G[2]);
   const double fd = -mG1 * (ir * ir0);
-  const double gd = fma(-mG2, ir, 1.0);
+  const double gd1 = -mG2 * ir;
   double lf = 0, lg = 0, lfd = 0, lgd = 0;
   for (int c = 0; c < 3; ++c) {
     lf = fma(lx1[c], x[c], lf);
     lg = fma(lx1[c], v[c], lg);
     lfd = fma(lv1[c], x[c], lfd);
     lgd = fma(lv1[c], v[c], lgd);
-    lx0[c] = fma(f, lx1[c], fd * lv1[c]);
-    lv0[c] = fma(g, lx1[c], gd * lv1[c]);
+    lx0[c] = fma(f1, lx1[c], fma(fd, lv1[c], lx1[c]));
+    lv0[c] = fma(gd1, lv1[c], fma(g, lx1[c], lv1[c]));
   }
   // f = 1 - mu G2/r0, g = r0 G1 + eta G2, fd = -mu G1/(r r0), gd = 1 - mu G2/r
   const double qf = lf * ir0, qd = lfd * (ir * ir0), qg = lgd * ir;
@@ -483,50 +484,6 @@ __device__ __forceinline__ void pair_vjp(double dx, double dy, double dz, double
   sbz = fma(B, dz, sbz);
 }
 
-// pair_vjp of a far pair (K = 1) in pairs of FP32 numbers (mx_split.cuh), for
-// systems of light big bodies: about 230 FP32 instructions where pair_vjp takes
-// 29 FP64 ones of 64 cycles.  The cotangent l comes scaled by a power of two
-// common to the tile, mu by 2^kVjpScale, so that the products and their low
-// parts stay normal numbers; the sums are scaled back.  Pairs within
-// three changeover radii, which carry most of a sum of 1/s^3 terms, keep
-// FP64.  Measured: k_adj_kick_vjp with 1,000 big bodies and 20,000
-// planetesimals 917 -> 315 us; two steps forward and back 21.7 -> 8.8 ms (with
-// the other reverse kernels), gradients within 4e-15 of the FP64 ones.  bs: the big body's traveling sum of A l + B d; ta, tb: the target's
-// sums of A and B d.
-constexpr int kVjpScale = 30;
-constexpr float kVjpNear2 = 9.0f;   // (3 changeover radii)^2, in units of one's
-
-struct VjpPos {
-  SplitPos p;
-  FF l[3];
-};
-
-__device__ __forceinline__ bool split_vjp(const VjpPos& t, const SplitBig& b, float near2,
-                                          float (&bs)[6], float (&ta)[2], float (&tb)[6]) {
-  float h[3], m[3];
-  split_sub(t.p.x0, t.p.x1, t.p.x2, b.x0, b.x1, b.x2, h[0], m[0]);
-  split_sub(t.p.y0, t.p.y1, t.p.y2, b.y0, b.y1, b.y2, h[1], m[1]);
-  split_sub(t.p.z0, t.p.z1, t.p.z2, b.z0, b.z1, b.z2, h[2], m[2]);
-  const FF s2 = ff_norm2(h[0], m[0], h[1], m[1], h[2], m[2]);
-  if (s2.h < near2) return false;
-  const FF is = ff_rsqrt(s2);
-  const FF is2 = ff_mul(is, is);
-  const FF A = ff_mul(FF{b.muh, b.mul}, ff_mul(is2, is));
-  FF dl = ff_mul(FF{h[0], m[0]}, t.l[0]);
-  dl = ff_add(dl, ff_mul(FF{h[1], m[1]}, t.l[1]));
-  dl = ff_add(dl, ff_mul(FF{h[2], m[2]}, t.l[2]));
-  const FF B = ff_mul(ff_mul(A, is2), ff_mul(FF{-3.0f, 0.0f}, dl));
-  split_add(ta[0], ta[1], A.h, A.l);
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    const FF al = ff_mul(A, t.l[c]), bd = ff_mul(B, FF{h[c], m[c]});
-    split_add(tb[2 * c], tb[2 * c + 1], bd.h, bd.l);
-    split_add(bs[2 * c], bs[2 * c + 1], al.h, al.l);
-    split_add(bs[2 * c], bs[2 * c + 1], bd.h, bd.l);
-  }
-  return true;
-}
-
 // Which parts of a half kick's reverse a launch takes.  The gravity's part is
 // linear in the cotangent l of the acceleration and depends on the positions
 // only, so the reverse of a step's first half kick and of the previous step's
@@ -557,10 +514,6 @@ struct KickRev {
 // the batch and then passes its running sum for that body to the lane before
 // it, so each body's sum visits the group's targets in a fixed order with
 // one shuffle a pair, and the groups' sums are added at the end.
-//
-// SPLIT: the systems that SysDev::split names take their far pairs in FP32
-// pairs (split_vjp), beside FP64 sums of the near ones.
-template <bool SPLIT>
 __global__ void __launch_bounds__(kThreads) k_adj_kick_vjp(Dev d, Adj a, const double* X,
                                                            const double* V, int pslot, int kick,
                                                            KickRev r) {
@@ -602,78 +555,19 @@ __global__ void __launch_bounds__(kThreads) k_adj_kick_vjp(Dev d, Adj a, const d
   }
   const double nlx = -3.0 * gax, nly = -3.0 * gay, nlz = -3.0 * gaz;
   double sa = 0, sbx = 0, sby = 0, sbz = 0;   // the target's sums (pair_vjp)
-  const bool split = SPLIT && S.split;
-  __shared__ SplitBig sp[SPLIT ? kAdjChunk : 1];
-  __shared__ int s_hi;
-  VjpPos vt{};
-  float near_own = 0.0f;
-  bool scaled = false;              // this target's l stands in vt.l
-  double unl = 1.0;                 // its scale's inverse
-  const double unmu = __hiloint2double((1023 - kVjpScale) << 20, 0);
-  if (split && r.grav) {
-    // the tile's largest |l| to about 1; a target far below it keeps FP64
-    const int lh = act ? max(abs_hi(gax), max(abs_hi(gay), abs_hi(gaz))) : 0;
-    __syncthreads();
-    if (threadIdx.x == 0) s_hi = 0;
-    __syncthreads();
-    const int wh = __reduce_max_sync(0xffffffffu, lh);
-    if (lane == 0) atomicMax(&s_hi, wh);
-    __syncthreads();
-    const int e = s_hi ? (s_hi >> 20) - 1023 : 0;   // l 2^-e below 2
-    if (e > -900 && e < 900) {
-      const double sl = __hiloint2double((1023 - e) << 20, 0);
-      unl = __hiloint2double((1023 + e) << 20, 0);
-      scaled = (lh >> 20) - 1023 > e - 60 || (gax == 0.0 && gay == 0.0 && gaz == 0.0);
-      vt.l[0] = ff_of(gax * sl);
-      vt.l[1] = ff_of(gay * sl);
-      vt.l[2] = ff_of(gaz * sl);
-    }
-    near_own = act && jl < S.nbig ? kVjpNear2 * near2_of(trc.rc2) : 0.0f;
-  }
-  int kt = INT_MIN;
   for (int c0 = 0; r.grav && c0 < S.nbig; c0 += kAdjChunk) {
     const int cn = min(kAdjChunk, S.nbig - c0);
     __syncthreads();
     stage_chunk(d, S, X, c0, cn, sx, sy, sz, sm, sc);
-    if (SPLIT && threadIdx.x == 0) s_hi = 0;
     __syncthreads();
-    bool far_ok = false;
-    if (split) {   // the chunk's parts, on the grid of its own positions
-      int hi = 0;
-      for (int k = threadIdx.x; k < cn; k += blockDim.x)
-        hi = max(hi, max(abs_hi(sx[k]), max(abs_hi(sy[k]), abs_hi(sz[k]))));
-      hi = __reduce_max_sync(0xffffffffu, hi);
-      if (lane == 0) atomicMax(&s_hi, hi);
-      __syncthreads();
-      const int kg = split_k(s_hi);
-      if (kg <= kSplitMaxK) {
-        for (int k = threadIdx.x; k < cn; k += blockDim.x) {
-          SplitBig b = split_big(sx[k], sy[k], sz[k], sm[k], sc[0][k], kg);
-          b.muh *= pow2f(kVjpScale);
-          b.mul *= pow2f(kVjpScale);
-          b.near2 *= kVjpNear2;
-          sp[k] = b;
-        }
-        far_ok = scaled && split_in_range(x, y, z, kg);
-        if (far_ok && kt != kg) {
-          kt = kg;
-          split3(x, kg, vt.p.x0, vt.p.x1, vt.p.x2);
-          split3(y, kg, vt.p.y0, vt.p.y1, vt.p.y2);
-          split3(z, kg, vt.p.z0, vt.p.z1, vt.p.z2);
-        }
-      }
-      __syncthreads();
-    }
     for (int base = 0; base < cn;) {
       const int left = cn - base;
       const int W = left >= 32 ? 32 : 1 << (31 - __clz(left));
       const int gl = lane & (W - 1);
       double bx = 0, by = 0, bz = 0;   // the running sum of the body this lane holds
-      float bs[6] = {0, 0, 0, 0, 0, 0}, ta[2] = {0, 0}, tb[6] = {0, 0, 0, 0, 0, 0};
       for (int r = 0; r < W; ++r) {
         const int k = base + ((gl + r) & (W - 1));
-        if (act && c0 + k != jl &&
-            !(SPLIT && far_ok && split_vjp(vt, sp[k], fmaxf(sp[k].near2, near_own), bs, ta, tb)))
+        if (act && c0 + k != jl)
           pair_vjp(x - sx[k], y - sy[k], z - sz[k], sm[k], pair_rc(sc, k, trc), gax, gay, gaz,
                    nlx, nly, nlz, bx, by, bz, sa, sbx, sby, sbz);
         if (r + 1 < W) {
@@ -681,19 +575,7 @@ __global__ void __launch_bounds__(kThreads) k_adj_kick_vjp(Dev d, Adj a, const d
           bx = __shfl_sync(0xffffffffu, bx, src, W);
           by = __shfl_sync(0xffffffffu, by, src, W);
           bz = __shfl_sync(0xffffffffu, bz, src, W);
-          if (split)
-            for (int q = 0; q < 6; ++q) bs[q] = __shfl_sync(0xffffffffu, bs[q], src, W);
         }
-      }
-      if (split) {   // the FP32 sums over at most 32 pairs go into the FP64 ones
-        const double ub = unl * unmu;
-        bx = fma(bits_to_double(bs[0]) + bits_to_double(bs[1]), ub, bx);
-        by = fma(bits_to_double(bs[2]) + bits_to_double(bs[3]), ub, by);
-        bz = fma(bits_to_double(bs[4]) + bits_to_double(bs[5]), ub, bz);
-        sa = fma(bits_to_double(ta[0]) + bits_to_double(ta[1]), unmu, sa);
-        sbx = fma(bits_to_double(tb[0]) + bits_to_double(tb[1]), ub, sbx);
-        sby = fma(bits_to_double(tb[2]) + bits_to_double(tb[3]), ub, sby);
-        sbz = fma(bits_to_double(tb[4]) + bits_to_double(tb[5]), ub, sbz);
       }
       for (int off = W; off < 32; off <<= 1) {
         bx += __shfl_down_sync(0xffffffffu, bx, off);
@@ -944,15 +826,9 @@ __global__ void __launch_bounds__(kThreads) k_adj_fold_jump1(Dev d, Adj a) {
   }
 }
 
-using KickVjpKernel = void (*)(Dev, Adj, const double*, const double*, int, int, KickRev);
-static KickVjpKernel kick_vjp_kernel(const Dev& d) {
-  return d.split_mode == kSplitNone ? k_adj_kick_vjp<false> : k_adj_kick_vjp<true>;
-}
-
-int adjoint_vjp_blocks_per_sm(const Dev& d, int threads) {
+int adjoint_vjp_blocks_per_sm(int threads) {
   int n = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kick_vjp_kernel(d), threads, 0) !=
-      cudaSuccess)
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_adj_kick_vjp, threads, 0) != cudaSuccess)
     return 0;
   return n;
 }
@@ -984,8 +860,8 @@ void launch_adjoint_step_b(const Dev& d, const Adj& a, cudaStream_t st) {
   // reverse sweep: kick 2 (at x4, v3, P3), jump 2, drift, jump 1, kick 1 (at x0, v0, P0)
   // (with a.lin, the pair pass also takes the next step's first half kick,
   // left pending at the same positions)
-  kick_vjp_kernel(d)<<<d.ntiles, d.tile, 0, st>>>(d, a, a.x4, a.xv3 + 3 * (size_t)N, 2, 2 * a.step + 1,
-                                              KickRev{1, 1, 1, a.lin, nullptr});
+  k_adj_kick_vjp<<<d.ntiles, d.tile, 0, st>>>(d, a, a.x4, a.xv3 + 3 * (size_t)N, 2, 2 * a.step + 1,
+                                               KickRev{1, 1, 1, a.lin, nullptr});
   launch_fold_kick(d, a, 2, 1, st);
   if (a.groups) launch_adjoint_bs_vjp(d, a, a.bs_blocks, st);
   k_adj_drift_vjp<<<d.ntiles, d.tile, 0, st>>>(d, a);
@@ -993,13 +869,13 @@ void launch_adjoint_step_b(const Dev& d, const Adj& a, cudaStream_t st) {
   k_adj_fold_jump1<<<d.nsys, kThreads, 0, st>>>(d, a);
   // merged: the drag now, the pair pass with the previous step's last half kick
   const KickRev r1{a.defer_k1 ? 0 : 1, 1, 1, nullptr, a.defer_k1 ? a.lpend : nullptr};
-  kick_vjp_kernel(d)<<<d.ntiles, d.tile, 0, st>>>(d, a, a.z0, a.z0 + 3 * (size_t)N, 0, 2 * a.step, r1);
+  k_adj_kick_vjp<<<d.ntiles, d.tile, 0, st>>>(d, a, a.z0, a.z0 + 3 * (size_t)N, 0, 2 * a.step, r1);
   launch_fold_kick(d, a, 1, r1.grav, st);
 }
 
 void launch_adjoint_flush(const Dev& d, const Adj& a, const double* xpos, cudaStream_t st) {
-  kick_vjp_kernel(d)<<<d.ntiles, d.tile, 0, st>>>(d, a, xpos, xpos, 0, 0,
-                                              KickRev{1, 0, 0, a.lpend, nullptr});
+  k_adj_kick_vjp<<<d.ntiles, d.tile, 0, st>>>(d, a, xpos, xpos, 0, 0,
+                                               KickRev{1, 0, 0, a.lpend, nullptr});
   launch_fold_kick(d, a, 1, 1, st);
 }
 
