@@ -466,6 +466,18 @@ mx_status mx_adjoint_step_predrift(mx_system* s, const double* dev_state_k,
                                    const double* dev_predrift_k, long long step_k,
                                    double* dev_lambda, double* dev_dparams);
 
+/* The recomputation of a segment for the reverse sweep: n_steps steps from the
+ * current state, step k's starting state into dev_states + k 6N and its
+ * pre-drift state into dev_predrift + k 6N (device buffers), as
+ * mx_get_state_device, mx_step(1) and mx_predrift_state would leave them one
+ * step at a time (deferral off), with one synchronisation.  Of the encounter
+ * groups it integrates those that mx_adjoint_encounters names: every group
+ * (1), the groups of big bodies (2) or none (0); the bodies of the others keep
+ * their drifted state, in the states returned and in the system's own, which
+ * the mode's loss gives weight 0.  The encounter log is left as it was.
+ * MX_ERR_ARG with the ejection test or growth tracks. */
+mx_status mx_adjoint_recompute(mx_system* s, int n_steps, double* dev_states, double* dev_predrift);
+
 /* Which of the step's encounter groups mx_adjoint_step integrates and
  * differentiates.  The groups are the step's own (rebuilt from the
  * recomputed endpoints): groups of big bodies joined by big-big encounters,

@@ -20,8 +20,10 @@ recorded in the forward run and replayed in the recomputation, so the
 reverse sweep sees the branches the forward run took.  Consecutive steps are
 reversed with mx_adjoint_merge on: the pair pass of a step's first half kick
 joins that of the previous step's last half kick, at the same positions.  The
-recomputation keeps each step's pre-drift state (mx_predrift_state), so the
-adjoint does not recompute the first half kick (mx_adjoint_step_predrift).
+recomputation (mx_adjoint_recompute) keeps each step's pre-drift state, so the
+adjoint does not recompute the first half kick (mx_adjoint_step_predrift), and
+leaves out the encounter groups the adjoint skips: their bodies' states carry
+no derivative.
 
 Inputs: the initial heliocentric state (6 x N float64 CUDA tensor) and the
 gas parameters (sigma1 [g/cm^2], gamma, cd_scale) as a 3-vector.
@@ -116,12 +118,8 @@ class SemimajorLoss(torch.autograd.Function):
             length = min(ctx.every, ctx.nsteps - start)
             mx.mx_set_state_device(h, ck)
             mx.mx_set_step_index(h, start)
-            # each step's start and pre-drift state (the branch replay keeps
-            # deferral off, so the step leaves every body's)
-            for k in range(length):
-                mx.mx_get_state_device(h, seg[k])
-                mx.mx_step(h, 1)
-                mx.mx_predrift_state(h, pre[k])
+            # each step's start and pre-drift state
+            mx.mx_adjoint_recompute(h, length, seg, pre)
             for k in reversed(range(length)):
                 mx.mx_adjoint_step_predrift(h, seg[k], pre[k], start + k, lam, dpar)
         grad0 = torch.empty((6, traj.n), dtype=torch.float64, device="cuda")

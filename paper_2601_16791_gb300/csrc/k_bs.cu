@@ -302,7 +302,8 @@ __device__ __forceinline__ void groups_block(const Dev& d) {
     return;
   }
   // ---- test-particle groups: one per run of pairs with the same small body
-  for (int cs = 0; cs < n; cs += blockDim.x) {
+  // (d.bb_only: none, mx_adjoint_recompute)
+  for (int cs = 0; cs < n && !d.bb_only; cs += blockDim.x) {
     const int p = cs + threadIdx.x;
     const bool start = p < n && key_small(keys[p]) && (p == 0 || key_j(keys[p]) != key_j(keys[p - 1]));
     int mem[kMaxGroup];

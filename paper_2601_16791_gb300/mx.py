@@ -105,6 +105,7 @@ _SIGS = {
     "mx_predrift_state": (_I, [_P, _P]),
     "mx_adjoint_step_predrift": (_I, [_P, _P, _P, ctypes.c_longlong, _P, _P]),
     "mx_adjoint_flush": (_I, [_P]),
+    "mx_adjoint_recompute": (_I, [_P, _I, _P, _P]),
     "mx_planets": (_I, [_P, _P, _P]),
 }
 
@@ -534,6 +535,11 @@ def mx_adjoint_step_predrift(sys, dev_state_k, dev_predrift_k, step_k, dev_lambd
     _check(load().mx_adjoint_step_predrift(sys, _dptr(dev_state_k), _dptr(dev_predrift_k),
                                            int(step_k), _dptr(dev_lambda), _dptr(dev_dparams)),
            "mx_adjoint_step_predrift")
+
+
+def mx_adjoint_recompute(sys, n_steps, dev_states, dev_predrift):
+    _check(load().mx_adjoint_recompute(sys, int(n_steps), _dptr(dev_states), _dptr(dev_predrift)),
+           "mx_adjoint_recompute")
 
 
 def mx_adjoint_merge(sys, on):
