@@ -17,8 +17,8 @@
 // (k = 1..8), Aitken-Neville extrapolation in (H/n)^2, error = max over
 // bodies of max(|dx|^2 xscal, |dv|^2 vscal) <= tol^2; accepted sub-steps grow
 // by 1.3 (capped by what remains), failed ones halve.  Groups of up to four
-// bodies run on lanes (k_bs_pack, then k_bs_spread for the long ones); larger
-// groups run one per thread (k_bs).  On this part an FP64 instruction has
+// bodies run on a warp's lanes (k_bs_all, then k_bs_spread2 for the long ones);
+// larger groups run one per thread.  On this part an FP64 instruction has
 // ~67-cycle latency and costs the same for 1 or 32 active lanes, so a group's
 // serial chain, not its arithmetic, sets the time: the rows and step
 // candidates of a macro sub-step go on separate lanes to shorten it.
@@ -352,44 +352,71 @@ __device__ __forceinline__ void groups_block(const Dev& d) {
 __global__ void __launch_bounds__(1024) k_groups(Dev d) { groups_block(d); }
 
 // ------------------------------------------------- warp-cooperative groups
-// Groups of up to kLaneMaxNB bodies run on lanes: lane 8c + r of a group
-// integrates extrapolation row r (n = 2(r+1) Stoermer sub-steps) with the
-// candidate step H/2^c.  The rows of a macro sub-step advance side by side;
-// the Aitken-Neville table of each candidate is a wavefront across its 8
-// lanes (row r takes row r-1's column j-1 by a shuffle); every lane checks its
-// own row's error, and the lowest converged lane of the group's vote (smallest
-// c, then smallest r) is accepted -- exactly what trying H, then H/2 after a
-// failure, and so on, with the rows in order, would accept.
+// Groups of up to kLaneMaxNB bodies run on a warp's lanes, one extrapolation
+// row (n = 2(r+1) Stoermer sub-steps) per four lanes.  The rows of a macro
+// sub-step advance side by side; the Aitken-Neville table is a wavefront across
+// the rows (row r takes row r-1's column j-1 by a shuffle); every row's error
+// is checked, and the lowest converged row is accepted -- exactly what trying
+// H, then H/2 after a failure, and so on, with the rows in order, would accept.
 //
-// Two phases.  k_bs_pack runs four groups per warp with one candidate (8
-// lanes each) for at most kPackRounds macro sub-steps: cheap in FP64 issue
-// slots, which cost the same for 1 or 32 active lanes.  Groups still running
-// are saved to a continuation list, and k_bs_spread finishes them one per
-// warp with four candidates on a grid of one warp per SM, so the few long
-// chains (deep fly-bys) neither wait behind failed attempts nor share an
-// SM's FP64 pipe.
+// With deferral on, k_bs_all is the whole step: a test-particle group that
+// needs a second macro sub-step leaves it (pack_tail).  With deferral off,
+// two-body groups that need more than kPackRounds macro sub-steps are saved to
+// a continuation list, and k_bs_spread2 finishes them on a cluster pair each,
+// so the few long chains (deep fly-bys) neither wait behind failed attempts nor
+// share an SM's FP64 pipe.
 constexpr int kLaneMaxNB = 4;
 constexpr int kPackRounds = 3;
 // With deferral on, the one round of a two-body group in the packed phase
 // stops at the check after this row when nothing has converged yet.
 constexpr int kDeferRow = 3;
 
+// Up to max_rounds macro sub-steps of a group of three or four bodies on one
+// warp: lane 4r + b advances body b in row r (with three bodies lane 4r + 3
+// repeats body 2, which no other lane reads), the sources' positions come by
+// shuffles, and the rows are checked as they complete (kBs2Checks), so that a
+// sub-step accepted at row 2 takes 7 force evaluations.  What bounds it is the
+// chain of FP64 instructions of one warp, 64 cycles each: about 50 to 65 a
+// force evaluation here, where every lane carried all bodies (150 to 290, all
+// 17 evaluations of a macro sub-step, four groups a warp).  Measured: four
+// steps of 301 big bodies + 20,011 planetesimals 1.157 -> 0.939 ms; twenty of 4
+// cores + 100,000, whose catch-up runs it too, 8.2 -> 7.4 ms.
+// Returns 1 when the step is done, 0 when rounds ran out, -1 at the cap.
 template <int NB>
-__device__ __forceinline__ void acc_nb(double mu0, const double* mu, const MemberK* K,
-                                       const double (&X)[3][NB], double (&A)[3][NB]) {
+__device__ int bsn_rounds(int lane, double mu0, const double* mu, const MemberK* K, double tol,
+                          int max_sub, int max_rounds, GroupRun<NB>& g) {
+  static_assert(NB == 3 || NB == 4, "four lanes a row");
+  const int row = lane >> 2, base = lane & ~3, b = min(lane & 3, NB - 1);
+  const int n = 2 * (row + 1);
+  const double tol2 = tol * tol;
+  MemberK kb = K[0];
+  double Y[6];   // this lane's body
 #pragma unroll
-  for (int b = 0; b < NB; ++b) {
-    const double x = X[0][b], y = X[1][b], z = X[2][b];
+  for (int m = 0; m < NB; ++m)
+    if (b == m) {
+      kb = K[m];
+#pragma unroll
+      for (int c = 0; c < 6; ++c) Y[c] = g.Y[c][m];
+    }
+  auto accel = [&](const double (&X)[3], double (&A)[3]) {
+    double sx[NB], sy[NB], sz[NB];
+#pragma unroll
+    for (int i = 0; i < NB; ++i) {
+      sx[i] = __shfl_sync(0xffffffffu, X[0], base + i);
+      sy[i] = __shfl_sync(0xffffffffu, X[1], base + i);
+      sz[i] = __shfl_sync(0xffffffffu, X[2], base + i);
+    }
+    const double x = X[0], y = X[1], z = X[2];
     const double ir = rsqrt_d(fma(x, x, fma(y, y, z * z)));
     const double f = mu0 * (ir * ir) * ir;
     double ax = -f * x, ay = -f * y, az = -f * z;
 #pragma unroll
     for (int i = 0; i < NB; ++i) {
       if (i == b || mu[i] == 0.0) continue;
-      const double dx = x - X[0][i], dy = y - X[1][i], dz = z - X[2][i];
+      const double dx = x - sx[i], dy = y - sy[i], dz = z - sz[i];
       const double s2 = fma(dx, dx, fma(dy, dy, dz * dz));
       // rc = max(rcrit_b, rcrit_i): the constants of the member with the larger radius
-      const MemberK& k = (K[b].rc > K[i].rc) ? K[b] : K[i];
+      const MemberK& k = (kb.rc > K[i].rc) ? kb : K[i];
       if (s2 >= k.rc2) continue;
       const double yy = rsqrt_d(s2);
       double wgt = (yy * yy) * (yy * mu[i]);
@@ -401,129 +428,99 @@ __device__ __forceinline__ void acc_nb(double mu0, const double* mu, const Membe
       ay = fma(-wgt, dy, ay);
       az = fma(-wgt, dz, az);
     }
-    A[0][b] = ax;
-    A[1][b] = ay;
-    A[2][b] = az;
-  }
-}
-
-// Up to max_rounds macro sub-steps of one group on the lanes of `gmask`
-// (8 * NCAND lanes starting at warp lane `base`; this lane is base + 8c + r).
-// Returns 1 when the step is done, 0 when rounds ran out, -1 at the cap.
-template <int NB, int NCAND>
-__device__ int bs_rounds(unsigned gmask, int base, int lane, double mu0, const double* mu,
-                         const MemberK* K, double tol, int max_sub, int max_rounds,
-                         GroupRun<NB>& g) {
-  const int rel = lane - base;
-  const int row = rel & 7, cand = rel >> 3;
-  const double tol2 = tol * tol;
-  double inv_den[kBsRows];
-#pragma unroll
-  for (int j = 1; j < kBsRows; ++j) {
-    const double r = (double)(row + 1) / (double)(row - j + 1);
-    inv_den[j] = (j <= row) ? 1.0 / (r * r - 1.0) : 0.0;
-  }
-  const int n = 2 * (row + 1);
-  const double inv_n = 1.0 / n;
-  const double cscale = pow2_neg(cand);   // 2^-cand, exact
+    A[0] = ax;
+    A[1] = ay;
+    A[2] = az;
+    __syncwarp();
+  };
+  int res = 2;
   for (int round = 0; round < max_rounds; ++round) {
-    if (g.rem == 0.0) return 1;
-    if (g.nsub >= max_sub) return -1;
+    if (g.rem == 0.0) {
+      res = 1;
+      break;
+    }
+    if (g.nsub >= max_sub) {
+      res = -1;
+      break;
+    }
     if (fabs(g.H) > fabs(g.rem)) g.H = g.rem;
-    const double Hc = g.H * cscale;
-    double xscal[NB], vscal[NB];
-#pragma unroll
-    for (int b = 0; b < NB; ++b) {
-      xscal[b] = rcp_d(fma(g.Y[0][b], g.Y[0][b], fma(g.Y[1][b], g.Y[1][b], g.Y[2][b] * g.Y[2][b])));
-      vscal[b] = rcp_d(fma(g.Y[3][b], g.Y[3][b], fma(g.Y[4][b], g.Y[4][b], g.Y[5][b] * g.Y[5][b])));
-    }
-    double X[3][NB], A[3][NB], D[3][NB];
-    const double dd = Hc * inv_n;
+    const double xs = rcp_d(fma(Y[0], Y[0], fma(Y[1], Y[1], Y[2] * Y[2])));
+    const double vs = rcp_d(fma(Y[3], Y[3], fma(Y[4], Y[4], Y[5] * Y[5])));
+    const double dd = g.H * c_bs_inv_n[row];
     const double d2 = dd * dd;
+    double X[3] = {Y[0], Y[1], Y[2]}, A[3], D[3], Traw[6] = {}, T[6];
+    accel(X, A);
 #pragma unroll
-    for (int c = 0; c < 3; ++c)
-#pragma unroll
-      for (int b = 0; b < NB; ++b) X[c][b] = g.Y[c][b];
-    acc_nb<NB>(mu0, mu, K, X, A);
-#pragma unroll
-    for (int c = 0; c < 3; ++c)
-#pragma unroll
-      for (int b = 0; b < NB; ++b) {
-        D[c][b] = dd * fma(0.5 * dd, A[c][b], g.Y[3 + c][b]);
-        X[c][b] += D[c][b];
-      }
-    for (int s = 1; s < n; ++s) {
-      acc_nb<NB>(mu0, mu, K, X, A);
-#pragma unroll
-      for (int c = 0; c < 3; ++c)
-#pragma unroll
-        for (int b = 0; b < NB; ++b) {
-          D[c][b] = fma(d2, A[c][b], D[c][b]);
-          X[c][b] += D[c][b];
-        }
+    for (int c = 0; c < 3; ++c) {
+      D[c] = dd * fma(0.5 * dd, A[c], Y[3 + c]);
+      X[c] += D[c];
     }
-    acc_nb<NB>(mu0, mu, K, X, A);
-    double T[6][NB], Tp[6][NB];
-    const double idd = n * rcp_d(Hc);
-#pragma unroll
-    for (int c = 0; c < 3; ++c)
-#pragma unroll
-      for (int b = 0; b < NB; ++b) {
-        T[c][b] = X[c][b];
-        T[3 + c][b] = fma(D[c][b], idd, 0.5 * dd * A[c][b]);
-        Tp[c][b] = T[c][b];
-        Tp[3 + c][b] = T[3 + c][b];
-      }
-    __syncwarp(gmask);
-#pragma unroll
-    for (int j = 1; j < kBsRows; ++j) {
-#pragma unroll
-      for (int c = 0; c < 6; ++c)
-#pragma unroll
-        for (int b = 0; b < NB; ++b) {
-          const double up = __shfl_up_sync(gmask, T[c][b], 1, 8);
-          if (row >= j) {
-            if (row == j) Tp[c][b] = T[c][b];
-            T[c][b] = fma(T[c][b] - up, inv_den[j], T[c][b]);
-          }
-        }
-    }
-    bool ok = false;
-    if (row >= 1) {
-      double err = 0.0;
-#pragma unroll
-      for (int b = 0; b < NB; ++b) {
-        double ex = 0.0, ev = 0.0;
+    int acc = -1;
+    for (int s = 1; s <= 2 * kBsRows && acc < 0; ++s) {
+      accel(X, A);
+      if (s < n) {
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-          const double dx = T[c][b] - Tp[c][b];
-          const double dv = T[3 + c][b] - Tp[3 + c][b];
-          ex = fma(dx, dx, ex);
-          ev = fma(dv, dv, ev);
+          D[c] = fma(d2, A[c], D[c]);
+          X[c] += D[c];
         }
-        err = fmax(err, fmax(ex * xscal[b], ev * vscal[b]));
+      } else if (s == n) {
+        const double idd = n * rcp_d(g.H);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          Traw[c] = X[c];
+          Traw[3 + c] = fma(D[c], idd, 0.5 * dd * A[c]);
+        }
       }
-      ok = err <= tol2;
+      const int R = (s >> 1) - 1;   // the row that completed at this sub-step
+      if ((s & 1) || !((kBs2Checks >> R) & 1u)) continue;
+      double Tp[6];
+#pragma unroll
+      for (int c = 0; c < 6; ++c) T[c] = Tp[c] = Traw[c];
+#pragma unroll 1
+      for (int j = 1; j <= R; ++j) {
+        const double den = c_bs_inv_den[row][j];
+#pragma unroll
+        for (int c = 0; c < 6; ++c) {
+          const double up = __shfl_up_sync(0xffffffffu, T[c], 4);
+          if (row >= j && row <= R) {
+            if (row == j) Tp[c] = T[c];
+            T[c] = fma(T[c] - up, den, T[c]);
+          }
+        }
+      }
+      double ex = 0.0, ev = 0.0;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const double dx = T[c] - Tp[c], dv = T[3 + c] - Tp[3 + c];
+        ex = fma(dx, dx, ex);
+        ev = fma(dv, dv, ev);
+      }
+      double err = fmax(0.0, fmax(ex * xs, ev * vs));
+      err = fmax(err, __shfl_xor_sync(0xffffffffu, err, 1));
+      err = fmax(err, __shfl_xor_sync(0xffffffffu, err, 2));
+      const unsigned v = __ballot_sync(0xffffffffu, row >= 1 && row <= R && err <= tol2);
+      if (v) acc = (__ffs(v) - 1) >> 2;
     }
-    const unsigned vote = __ballot_sync(gmask, ok) & gmask;
-    if (vote) {
-      const int src = __ffs(vote) - 1;
-      const int c_acc = (src - base) >> 3;
-      g.nsub += c_acc + 1;                   // attempts a one-at-a-time search makes
-      if (g.nsub > max_sub) return -1;
+    g.nsub += 1;
+    if (acc >= 0) {
 #pragma unroll
-      for (int c = 0; c < 6; ++c)
-#pragma unroll
-        for (int b = 0; b < NB; ++b) g.Y[c][b] = __shfl_sync(gmask, T[c][b], src);
-      const double Hacc = g.H * pow2_neg(c_acc);   // exact: a power of two
-      g.rem -= Hacc;
-      g.H = 1.3 * Hacc;
+      for (int c = 0; c < 6; ++c) Y[c] = __shfl_sync(0xffffffffu, T[c], 4 * acc + b);
+      if (g.nsub > max_sub) {
+        res = -1;
+        break;
+      }
+      g.rem -= g.H;
+      g.H = 1.3 * g.H;
     } else {
-      g.nsub += NCAND;
-      g.H *= 1.0 / (double)(1 << NCAND);
+      g.H *= 0.5;
     }
   }
-  return (g.rem == 0.0) ? 1 : 0;
+#pragma unroll
+  for (int m = 0; m < NB; ++m)
+#pragma unroll
+    for (int c = 0; c < 6; ++c) g.Y[c][m] = __shfl_sync(0xffffffffu, Y[c], m);
+  return res != 2 ? res : (g.rem == 0.0) ? 1 : 0;
 }
 
 // The members' masses and changeover constants (a big body's from set_rcrit's
@@ -990,8 +987,9 @@ __device__ void pack_tail(const Dev& d, int w, unsigned gmask, int base, int lan
   }
 }
 
+// A group of three or four bodies on one warp.
 template <int NB>
-__device__ __noinline__ void pack_group(const Dev& d, int w, unsigned gmask, int base, int lane) {
+__device__ __noinline__ void pack_group(const Dev& d, int w, int lane) {
   const int o0 = d.work_off[w];
   const SysDev& S = d.sys[d.work_sys[w]];
   double mu[NB];
@@ -1006,10 +1004,9 @@ __device__ __noinline__ void pack_group(const Dev& d, int w, unsigned gmask, int
   g.H = S.h;
   g.nsub = 0;
   // with deferral on, a group that needs a second round leaves the step at once
-  const int r = bs_rounds<NB, 1>(gmask, base, lane, S.mu0, mu, K, d.bs_tol, d.bs_max_sub,
-                                 d.defer ? 1 : kPackRounds, g);
-  pack_tail<NB>(d, w, gmask, base, lane, o0, r, g, [&](GroupRun<NB>& gg) {
-    return bs_rounds<NB, 1>(gmask, base, lane, S.mu0, mu, K, d.bs_tol, d.bs_max_sub, 1 << 30, gg);
+  const int r = bsn_rounds<NB>(lane, S.mu0, mu, K, d.bs_tol, d.bs_max_sub, d.defer ? 1 : 1 << 30, g);
+  pack_tail<NB>(d, w, 0xffffffffu, 0, lane, o0, r, g, [&](GroupRun<NB>& gg) {
+    return bsn_rounds<NB>(lane, S.mu0, mu, K, d.bs_tol, d.bs_max_sub, 1 << 30, gg);
   });
 }
 
@@ -1017,21 +1014,13 @@ __device__ void pack_two(const Dev& d, int w, int lane);
 __device__ void pack_two_pair(const Dev& d, int a, int b, int lane);
 __device__ __noinline__ void thread_group(const Dev& d, int w);
 
-// Two-body groups, one per warp (term lanes, one candidate).
-__global__ void __launch_bounds__(32) k_bs_pack2(Dev d) {
-  const int W = *d.work_count;
-  for (int w = blockIdx.x; w < W; w += gridDim.x)
-    if (d.work_off[w + 1] - d.work_off[w] == 2) pack_two(d, w, threadIdx.x);
-}
-
-// Every group, one per warp, in one launch: two bodies on term lanes, three
-// or four on the lane integrator (eight lanes), more on one thread.  Used
-// with deferral on, where nothing is handed to a spread phase.
+// One group on one warp: two bodies on term lanes, three or four on body lanes,
+// more on one thread.
 __device__ __forceinline__ void bs_one_warp(const Dev& d, int w, int lane) {
   const int nb = d.work_off[w + 1] - d.work_off[w];
   if (nb == 2) pack_two(d, w, lane);
-  else if (nb == 3) { if (lane < 8) pack_group<3>(d, w, 0xffu, 0, lane); }
-  else if (nb == 4) { if (lane < 8) pack_group<4>(d, w, 0xffu, 0, lane); }
+  else if (nb == 3) pack_group<3>(d, w, lane);
+  else if (nb == 4) pack_group<4>(d, w, lane);
   else if (nb > kLaneMaxNB && lane == 0) thread_group(d, w);
   __syncwarp();
 }
@@ -1044,12 +1033,17 @@ __device__ __forceinline__ bool two_deferrable(const Dev& d, int w) {
          d.sys[d.work_sys[w]].nbig <= kDeferMaxBig;
 }
 
-// The work items go to the warps in pairs (2s, 2s + 1).  A pair of deferrable
-// two-body groups shares the warp (pack_two_pair, 16 lanes each); any other
-// pair is taken one item after the other.
+// With deferral on, the work items go to the warps in pairs (2s, 2s + 1).  A
+// pair of deferrable two-body groups shares the warp (pack_two_pair, 16 lanes
+// each); any other pair is taken one item after the other.  With deferral off,
+// one item a warp.
 __device__ __forceinline__ void bs_all_warps(const Dev& d, int w0, int nw) {
   const int W = *d.work_count;
   const int lane = threadIdx.x & 31;
+  if (!d.defer) {
+    for (int w = w0; w < W; w += nw) bs_one_warp(d, w, lane);
+    return;
+  }
   for (int sp = w0; 2 * sp < W; sp += nw) {
     const int a = 2 * sp, b = 2 * sp + 1;
     if (b < W && two_deferrable(d, a) && two_deferrable(d, b)) {
@@ -1267,7 +1261,7 @@ __device__ void pack_two_pair(const Dev& d, int a, int b, int lane) {
   __syncwarp();
 }
 
-// Two-body groups handed over by k_bs_pack2, one per cluster of two CTAs: the
+// Two-body groups handed over by k_bs_all, one per cluster of two CTAs: the
 // catch-up's integrator (bs2c_rounds: three warps, a coordinate each; rank 0
 // tries H, rank 1 H/2).  The chain of macro sub-steps of the hardest group sets
 // the launch's time, and a sub-step takes 16 FP64 instructions of a warp here
@@ -1322,73 +1316,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(128) k_bs_spread2(De
   cl.sync();
 }
 
-// Four groups of LO..HI bodies per warp, 8 lanes each (separate kernels keep
-// the common two-body case free of the larger cases' register pressure).  One
-// warp per block: consecutive blocks land on different SMs, so the groups
-// spread over all SMs' FP64 pipes instead of filling a few SMs' worth of
-// four-warp blocks.
-template <int LO, int HI>
-__global__ void __launch_bounds__(32) k_bs_pack(Dev d) {
-  const int W = *d.work_count;
-  const int lane = threadIdx.x & 31;
-  const int slot = lane >> 3;
-  const int base = slot * 8;
-  const unsigned gmask = 0xffu << base;
-  const int gslot = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 4 + slot;
-  const int nslots = (gridDim.x * blockDim.x >> 5) * 4;
-  for (int w = gslot; w < W; w += nslots) {
-    const int nb = d.work_off[w + 1] - d.work_off[w];
-    if (nb < LO || nb > HI) continue;
-    if (LO <= 1 && nb == 1) pack_group<(LO <= 1 ? 1 : LO)>(d, w, gmask, base, lane);
-    else if (LO <= 2 && HI >= 2 && nb == 2) pack_group<2>(d, w, gmask, base, lane);
-    else if (LO <= 3 && HI >= 3 && nb == 3) pack_group<(HI >= 3 ? 3 : 2)>(d, w, gmask, base, lane);
-    else if (HI >= 4 && nb == 4) pack_group<(HI >= 4 ? 4 : 2)>(d, w, gmask, base, lane);
-  }
-}
-
-template <int NB>
-__device__ void spread_group(const Dev& d, int slot, int lane) {
-  const int w = d.cont_item[slot];
-  const int o0 = d.work_off[w];
-  const SysDev& S = d.sys[d.work_sys[w]];
-  double mu[NB];
-  MemberK K[NB];
-  load_members<NB>(d, S, o0, mu, K);
-  GroupRun<NB> g;
-  const double* c = d.cont_state + (size_t)slot * kContDoubles;
-  g.rem = c[0];
-  g.H = c[1];
-  g.nsub = (int)c[2];
-#pragma unroll
-  for (int m = 0; m < NB; ++m)
-#pragma unroll
-    for (int q = 0; q < 6; ++q) g.Y[q][m] = c[3 + 6 * m + q];
-  const int r = bs_rounds<NB, 4>(0xffffffffu, 0, lane, S.mu0, mu, K, d.bs_tol, d.bs_max_sub,
-                                 1 << 30, g);
-  if (lane == 0) {
-    if (r < 0) atomicOr(d.status, ST_BS);
-    d.work_nsub[w] = g.nsub;
-  }
-  write_members<NB>(d, w, o0, lane, g);
-}
-
-// The continued groups of LO..HI bodies, one per warp, four step candidates
-// x eight rows.
-template <int LO, int HI>
-__global__ void __launch_bounds__(32) k_bs_spread(Dev d) {
-  const int C = min(*d.cont_count, d.cont_cap);
-  const int lane = threadIdx.x & 31;
-  for (int slot = blockIdx.x; slot < C; slot += gridDim.x) {
-    const int w = d.cont_item[slot];
-    const int nb = d.work_off[w + 1] - d.work_off[w];
-    if (nb < LO || nb > HI) continue;
-    if (LO <= 1 && nb == 1) spread_group<(LO <= 1 ? 1 : LO)>(d, slot, lane);
-    else if (LO <= 2 && HI >= 2 && nb == 2) spread_group<2>(d, slot, lane);
-    else if (LO <= 3 && HI >= 3 && nb == 3) spread_group<(HI >= 3 ? 3 : 2)>(d, slot, lane);
-    else if (HI >= 4 && nb == 4) spread_group<(HI >= 4 ? 4 : 2)>(d, slot, lane);
-  }
-}
-
 // A group of more than kLaneMaxNB bodies on one thread.
 __device__ __noinline__ void thread_group(const Dev& d, int w) {
   const int N = d.N;
@@ -1412,13 +1339,6 @@ __device__ __noinline__ void thread_group(const Dev& d, int w) {
     const int g = d.work_mem[o0 + m];
     for (int c = 0; c < 6; ++c) d.xv[(size_t)c * N + g] = Y[c][m];
   }
-}
-
-// One thread per work item with more than kLaneMaxNB bodies, grid-stride.
-__global__ void __launch_bounds__(32) k_bs(Dev d) {
-  const int W = *d.work_count;
-  for (int w = blockIdx.x * blockDim.x + threadIdx.x; w < W; w += gridDim.x * blockDim.x)
-    if (d.work_off[w + 1] - d.work_off[w] > kLaneMaxNB) thread_group(d, w);
 }
 
 // ----------------------------------------------- deferred planetesimals
@@ -1508,8 +1428,7 @@ struct CatchGroup {
   double Y[6][kLaneMaxNB];
 };
 
-// Three or four bodies: the lane integrator of k_bs_spread on one warp, run
-// to the end of the step.
+// Three or four bodies: bsn_rounds on one warp, run to the end of the step.
 template <int NB>
 __device__ __noinline__ int catch_bs(const Dev& d, const SysDev& S, const CatchGroup& G, int t,
                                      int lane, double* s6) {
@@ -1524,8 +1443,7 @@ __device__ __noinline__ int catch_bs(const Dev& d, const SysDev& S, const CatchG
   g.rem = G.rem;
   g.H = G.H;
   g.nsub = G.nsub;
-  const int r = bs_rounds<NB, 4>(0xffffffffu, 0, lane, S.mu0, mu, K, d.bs_tol, d.bs_max_sub,
-                                 1 << 30, g);
+  const int r = bsn_rounds<NB>(lane, S.mu0, mu, K, d.bs_tol, d.bs_max_sub, 1 << 30, g);
 #pragma unroll
   for (int q = 0; q < 6; ++q) s6[q] = g.Y[q][NB - 1];
   return r;
@@ -2200,11 +2118,8 @@ void launch_bs(const Dev& d, int nblocks, cudaStream_t st) {
     return;
   }
   cudaMemsetAsync(d.cont_count, 0, sizeof(int), st);
-  k_bs_pack2<<<4 * nblocks, 32, 0, st>>>(d);
-  k_bs_pack<3, 4><<<4 * nblocks, 32, 0, st>>>(d);
-  k_bs<<<nblocks, 32, 0, st>>>(d);
+  k_bs_all<<<4 * nblocks, 32, 0, st>>>(d);
   k_bs_spread2<<<nblocks & ~1, 128, 0, st>>>(d);   // whole cluster pairs
-  k_bs_spread<3, 4><<<nblocks / 4, 32, 0, st>>>(d);
 }
 
 void launch_catchup(const Dev& d, int nblocks, int mode, int bank_a, int bank_b, int bank_out,
@@ -2220,11 +2135,7 @@ void configure_bs() {
   const int c = cudaSharedmemCarveoutMaxShared;
   cudaFuncSetAttribute(k_groups, cudaFuncAttributePreferredSharedMemoryCarveout, c);
   cudaFuncSetAttribute(k_bs_all, cudaFuncAttributePreferredSharedMemoryCarveout, c);
-  cudaFuncSetAttribute(k_bs_pack2, cudaFuncAttributePreferredSharedMemoryCarveout, c);
-  cudaFuncSetAttribute(k_bs_pack<3, 4>, cudaFuncAttributePreferredSharedMemoryCarveout, c);
-  cudaFuncSetAttribute(k_bs, cudaFuncAttributePreferredSharedMemoryCarveout, c);
   cudaFuncSetAttribute(k_bs_spread2, cudaFuncAttributePreferredSharedMemoryCarveout, c);
-  cudaFuncSetAttribute(k_bs_spread<3, 4>, cudaFuncAttributePreferredSharedMemoryCarveout, c);
   cudaFuncSetAttribute(k_catchup, cudaFuncAttributePreferredSharedMemoryCarveout, c);
   cudaFuncSetAttribute(k_step_persist, cudaFuncAttributePreferredSharedMemoryCarveout, c);
 }
