@@ -20,8 +20,8 @@
 // accelerations, does not use it.
 //
 // Measured: k_jump_kick with 2,000 big bodies and 200,000 planetesimals 11.8 ->
-// 1.73 ms a launch (34 -> 233 G pairs/s), two steps of that disk 40.2 -> 9.9 ms;
-// 301 big bodies and 20,011 planetesimals 0.43 -> 0.068 ms a launch.  64 gas
+// 1.65 ms a launch (34 -> 245 G pairs/s); 301 big bodies and 20,011
+// planetesimals 0.43 -> 0.068 ms a launch.  64 gas
 // disks of 2 to 50 light bodies (2.4 million bodies; with the drag, see
 // mx_split_gas.cuh) 2.35 -> 0.45 ms a launch, three steps 12.0 -> 4.34 ms.
 //
@@ -227,7 +227,8 @@ struct SplitTerm {
   float xh, xl, yh, yl, zh, zl;
 };
 
-// A pair's mu d/s^3; returns false, f not set, for a pair inside near2.
+// A pair's mu d/s^3; returns false, f zero, for a pair inside near2 (without a
+// branch, so that the caller's pairs overlap).
 // 1/s^3 = y^3 (1 + 3e/2 + 15e^2/8) from the single-precision estimate y of
 // 1/s, e = 1 - s^2 y^2, as in pair_weight.
 __device__ __forceinline__ bool split_term(const SplitPos& t, const SplitBig& b, float near2,
@@ -237,7 +238,7 @@ __device__ __forceinline__ bool split_term(const SplitPos& t, const SplitBig& b,
   split_sub(t.y0, t.y1, t.y2, b.y0, b.y1, b.y2, hy, my);
   split_sub(t.z0, t.z1, t.z2, b.z0, b.z1, b.z2, hz, mz);
   const FF s2 = ff_norm2(hx, mx, hy, my, hz, mz);
-  if (s2.h < near2) return false;
+  const bool far = !(s2.h < near2);
   const float y = rsqrtf(s2.h);
   float y2, y2l, a, c;
   ff_rsqrt_residual(s2, y, y2, y2l, a, c);
@@ -247,19 +248,21 @@ __device__ __forceinline__ bool split_term(const SplitPos& t, const SplitBig& b,
   // w = mu y^3 (1 + k1 + k2) = wh + wl
   const float y3 = __fmul_rn(y2, y);
   const float y3l = __fmaf_rn(y2l, y, __fmaf_rn(y2, y, -y3));
-  const float wh = __fmul_rn(b.muh, y3);
+  float wh = __fmul_rn(b.muh, y3);
   float wl = __fmaf_rn(b.muh, y3, -wh);
   wl = __fmaf_rn(b.muh, y3l, wl);
   wl = __fmaf_rn(b.mul, y3, wl);
   wl = __fmaf_rn(wh, k2, wl);
   wl = __fmaf_rn(wh, k1, wl);
+  wh = far ? wh : 0.0f;
+  wl = far ? wl : 0.0f;
   f.xh = __fmul_rn(wh, hx);
   f.yh = __fmul_rn(wh, hy);
   f.zh = __fmul_rn(wh, hz);
   f.xl = __fmaf_rn(wl, hx, __fmaf_rn(wh, mx, __fmaf_rn(wh, hx, -f.xh)));
   f.yl = __fmaf_rn(wl, hy, __fmaf_rn(wh, my, __fmaf_rn(wh, hy, -f.yh)));
   f.zl = __fmaf_rn(wl, hz, __fmaf_rn(wh, mz, __fmaf_rn(wh, hz, -f.zh)));
-  return true;
+  return far;
 }
 
 __device__ __forceinline__ void split_sum(SplitAcc& acc, const SplitTerm& f) {
