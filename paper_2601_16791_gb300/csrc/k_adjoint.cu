@@ -15,7 +15,7 @@
 //
 // Parameter cotangents (per system): d/d sigma1, d/d gamma, d/d cd_scale.
 #include "mx_common.cuh"
-#include "mx_kepler.cuh"
+#include "mx_kepler_short.cuh"
 #include "mx_kernels.h"
 #include "mx_physics.cuh"
 
@@ -251,10 +251,10 @@ __device__ bool kepler_vjp(double mu, double h, int maxit, const double* x, cons
   const double r = fma(eta, G[1], fma(zeta, G[2], r0));
   const double ir = rcp_d(r);
   const double mG1 = mu * G[1], mG2 = mu * G[2];
-  // f - 1 and gd - 1, small on a short step: their roundings do not reach the
-  // cotangents' last places
+  // f - 1, gd - 1 and g = r0 G1 + eta G2 = h - mu G3, so that the last additions
+  // alone round at the cotangents' size
   const double f1 = -mG2 * ir0;
-  const double g = fma(r0, G[1], eta * G[2]);
+  const double g = fma(-mu, G[3], h);
   const double fd = -mG1 * (ir * ir0);
   const double gd1 = -mG2 * ir;
   double lf = 0, lg = 0, lfd = 0, lgd = 0;
@@ -263,8 +263,8 @@ __device__ bool kepler_vjp(double mu, double h, int maxit, const double* x, cons
     lg = fma(lx1[c], v[c], lg);
     lfd = fma(lv1[c], x[c], lfd);
     lgd = fma(lv1[c], v[c], lgd);
-    lx0[c] = fma(f1, lx1[c], fma(fd, lv1[c], lx1[c]));
-    lv0[c] = fma(gd1, lv1[c], fma(g, lx1[c], lv1[c]));
+    lx0[c] = lx1[c] + fma(f1, lx1[c], fd * lv1[c]);
+    lv0[c] = fma(g, lx1[c], fma(gd1, lv1[c], lv1[c]));
   }
   // f = 1 - mu G2/r0, g = r0 G1 + eta G2, fd = -mu G1/(r r0), gd = 1 - mu G2/r
   const double qf = lf * ir0, qd = lfd * (ir * ir0), qg = lgd * ir;
@@ -434,7 +434,8 @@ __global__ void __launch_bounds__(kThreads) k_adj_move_fwd(Dev d, Adj a, int sta
       x = a.x2[j]; y = a.x2[(size_t)N + j]; z = a.x2[2 * (size_t)N + j];
     }
     double u = a.v1[j], v = a.v1[(size_t)N + j], w = a.v1[2 * (size_t)N + j];
-    if (!kepler_drift(S.mu0, S.h, d.kepler_max_iter, x, y, z, u, v, w)) atomicOr(d.status, ST_KEPLER);
+    if (!kepler_drift_sel(S.split, S.mu0, S.h, d.kepler_max_iter, x, y, z, u, v, w))
+      atomicOr(d.status, ST_KEPLER);
     a.xv3[j] = x; a.xv3[(size_t)N + j] = y; a.xv3[2 * (size_t)N + j] = z;
     a.xv3[3 * (size_t)N + j] = u; a.xv3[4 * (size_t)N + j] = v; a.xv3[5 * (size_t)N + j] = w;
   } else {

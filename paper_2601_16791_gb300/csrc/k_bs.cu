@@ -26,7 +26,7 @@
 
 #include "mx_common.cuh"
 #include "mx_encounter.cuh"
-#include "mx_kepler.cuh"
+#include "mx_kepler_short.cuh"
 #include "mx_kernels.h"
 #include "mx_bs.cuh"
 #include "mx_bs2.cuh"
@@ -1553,7 +1553,7 @@ __device__ int catch_front(const Dev& d, const SysDev& S, int sys, int j, int t,
   double x = s6[0] + dj[0], y = s6[1] + dj[1], z = s6[2] + dj[2];
   double u = s6[3], v = s6[4], w = s6[5];
   const double a0[6] = {x, y, z, u, v, w};
-  if (!kepler_drift(S.mu0, S.h, d.kepler_max_iter, x, y, z, u, v, w) && wr && lane == 0)
+  if (!kepler_drift_sel(S.split, S.mu0, S.h, d.kepler_max_iter, x, y, z, u, v, w) && wr && lane == 0)
     atomicOr(d.status, ST_KEPLER);
   const double a1[6] = {x, y, z, u, v, w};
   float af[12];

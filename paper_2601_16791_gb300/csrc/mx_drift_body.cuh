@@ -2,7 +2,7 @@
 // (k_drift.cu), shared by its kernel and the persistent step kernel.
 #pragma once
 #include "mx_common.cuh"
-#include "mx_kepler.cuh"
+#include "mx_kepler_short.cuh"
 
 namespace mx {
 
@@ -55,7 +55,7 @@ __device__ __forceinline__ void jump_drift_tile(const Dev& d, double jump_frac, 
   d.xv0[3 * (size_t)N + j] = u;
   d.xv0[4 * (size_t)N + j] = v;
   d.xv0[5 * (size_t)N + j] = w;
-  if (!kepler_drift(S.mu0, S.h, d.kepler_max_iter, x, y, z, u, v, w))
+  if (!kepler_drift_sel(S.split, S.mu0, S.h, d.kepler_max_iter, x, y, z, u, v, w))
     atomicOr(d.status, ST_KEPLER);
   d.xv[j] = x;
   d.xv[(size_t)N + j] = y;
