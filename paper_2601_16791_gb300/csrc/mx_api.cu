@@ -198,7 +198,7 @@ struct mx_system {
   double* d_tmp = nullptr;        // 6 x N scratch for readout / set_state
   double* d_energy = nullptr;
   double* d_sink = nullptr;
-  unsigned* h_status = nullptr;   // pinned
+  unsigned* h_status = nullptr;   // pinned; the kernels' status word (d.status)
   int* h_count = nullptr;         // pinned
   std::vector<void*> allocs;
   cudaGraphExec_t g_head = nullptr, g_mid = nullptr, g_last = nullptr;
@@ -302,17 +302,14 @@ mx_status set_device(mx_system* s) {
   return MX_OK;
 }
 
+// Waits for the stream and reads the kernels' status word.  The word is pinned
+// host memory, which a kernel touches only to report a failure, so that a call
+// ends without a copy behind its last kernel.
 mx_status sync_status(mx_system* s) {
-  MX_CUDA(cudaMemcpyAsync(s->h_status, s->d.status, sizeof(unsigned), cudaMemcpyDeviceToHost, s->st));
   MX_CUDA(cudaStreamSynchronize(s->st));
   MX_CUDA(cudaGetLastError());
-  const unsigned st = *s->h_status;
-  if (st) {
-    MX_CUDA(cudaMemsetAsync(s->d.status, 0, sizeof(unsigned), s->st));
-    MX_CUDA(cudaStreamSynchronize(s->st));
-    return status_to_code(st);
-  }
-  return MX_OK;
+  const unsigned st = __atomic_exchange_n(s->h_status, 0u, __ATOMIC_ACQ_REL);
+  return st ? status_to_code(st) : MX_OK;
 }
 
 // The device work of one interior step, or the last step of a call
@@ -709,7 +706,6 @@ mx_status trial_ms(mx_system* s, double* ms) {
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   MX_CUDA(cudaMemcpyAsync(s->d.xv, s->d_tmp, bytes, cudaMemcpyDeviceToDevice, s->st));
-  MX_CUDA(cudaMemsetAsync(s->d.status, 0, sizeof(unsigned), s->st));
   MX_CUDA(cudaMemsetAsync(s->d.pair_count, 0, 2 * sizeof(int), s->st));
   // trials run at creation: the encounter log and the counters start empty
   MX_CUDA(cudaMemsetAsync(s->d.ever, 0, s->N, s->st));
@@ -719,6 +715,7 @@ mx_status trial_ms(mx_system* s, double* ms) {
   MX_CUDA(cudaMemsetAsync(s->d.kick_ctr, 0, 2 * sizeof(int), s->st));
   MX_CUDA(cudaMemsetAsync(s->d.gstep, 0, sizeof(long long), s->st));
   MX_CUDA(cudaStreamSynchronize(s->st));
+  *s->h_status = 0;
   *ms = t;
   return MX_OK;
 }
@@ -851,7 +848,7 @@ mx_status build(mx_system* s, const std::vector<const double*>& m_big,
     MX_TRY(dalloc(s, &d.d_state, (size_t)3 * d.dcap * mx::kRecDoubles));
     s->window = std::min(kDefaultWindow, hc / 2);
   }
-  MX_TRY(dalloc(s, &d.status, 1));
+  d.status = s->h_status;   // in host memory the device reaches (sync_status)
   MX_TRY(dalloc(s, &d.gbar, 8));
   MX_TRY(dalloc(s, &d.stat, N));
   MX_TRY(dalloc(s, &s->d_grow, NB));
@@ -887,7 +884,7 @@ mx_status build(mx_system* s, const std::vector<const double*>& m_big,
   MX_CUDA(cudaMemcpyAsync(s->d_sys, sys.data(), nsys * sizeof(mx::SysDev), cudaMemcpyHostToDevice, st));
   MX_CUDA(cudaMemcpyAsync(s->d_tiles, tiles.data(), tiles.size() * sizeof(mx::Tile),
                           cudaMemcpyHostToDevice, st));
-  MX_CUDA(cudaMemsetAsync(d.status, 0, sizeof(unsigned), st));
+  *s->h_status = 0;
   MX_CUDA(cudaMemsetAsync(d.gbar, 0, 8 * sizeof(unsigned), st));
   MX_CUDA(cudaMemsetAsync(d.pair_count, 0, 2 * sizeof(int), st));
   MX_CUDA(cudaMemsetAsync(d.flags, 0, N, st));
@@ -952,15 +949,13 @@ void destroy_impl(mx_system* s) {
   if (!s) return;
   cudaSetDevice(s->device);
   if (s->st) cudaStreamSynchronize(s->st);
+  if (s->side_st) cudaStreamSynchronize(s->side_st);
   drop_graphs(s);
   for (void* p : s->allocs) cudaFree(p);
   if (s->h_status) cudaFreeHost(s->h_status);
   if (s->h_count) cudaFreeHost(s->h_count);
   if (s->h_need) cudaFreeHost(s->h_need);
-  if (s->side_st) {
-    cudaStreamSynchronize(s->side_st);
-    cudaStreamDestroy(s->side_st);
-  }
+  if (s->side_st) cudaStreamDestroy(s->side_st);
   for (auto& sp : s->side_spans) {
     cudaEventDestroy(sp.a);
     cudaEventDestroy(sp.b);
