@@ -525,11 +525,16 @@ __global__ void __launch_bounds__(kThreads) k_adj_kick_vjp(Dev d, Adj a, const d
   const Tile t = d.tiles[blockIdx.x];
   const SysDev& S = d.sys[t.sys];
   const int N = d.N;
-  const bool act = threadIdx.x < t.count;
-  const int j = t.start + threadIdx.x;
+  // parts > 1: every thread group of a tile's size takes the same targets and
+  // its share of the big bodies (whole warps)
+  const int tile = blockDim.x / a.parts, part = threadIdx.x / tile;
+  const int tx = threadIdx.x - part * tile;
+  const bool act = tx < t.count;
+  const int j = t.start + tx;
   const int jl = j - S.off;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int nwarps = (blockDim.x + 31) >> 5;
+  const int lane = tx & 31, warp = tx >> 5;   // the warp among its part's
+  const int nwarps = (tile + 31) >> 5;
+  const int wmax = a.parts > 4 ? 16 : 32;     // bodies a batch: a chunk has one for every part
   const double* Pk = a.P + 9 * t.sys + 3 * pslot;
   const double th = 0.5 * S.h;
   double* rec = a.part + a.poff[blockIdx.x];
@@ -549,7 +554,7 @@ __global__ void __launch_bounds__(kThreads) k_adj_kick_vjp(Dev d, Adj a, const d
     gay += r.lin[(size_t)N + j];
     gaz += r.lin[2 * (size_t)N + j];
   }
-  if (act && r.lout) {
+  if (act && part == 0 && r.lout) {
     r.lout[j] = lax;
     r.lout[(size_t)N + j] = lay;
     r.lout[2 * (size_t)N + j] = laz;
@@ -561,9 +566,14 @@ __global__ void __launch_bounds__(kThreads) k_adj_kick_vjp(Dev d, Adj a, const d
     __syncthreads();
     stage_chunk(d, S, X, c0, cn, sx, sy, sz, sm, sc);
     __syncthreads();
-    for (int base = 0; base < cn;) {
+    int batch = 0;
+    for (int base = 0; base < cn; ++batch) {
       const int left = cn - base;
-      const int W = left >= 32 ? 32 : 1 << (31 - __clz(left));
+      const int W = left >= wmax ? wmax : 1 << (31 - __clz(left));
+      if (a.parts > 1 && (batch & (a.parts - 1)) != part) {
+        base += W;
+        continue;
+      }
       const int gl = lane & (W - 1);
       double bx = 0, by = 0, bz = 0;   // the running sum of the body this lane holds
       for (int r = 0; r < W; ++r) {
@@ -604,11 +614,24 @@ __global__ void __launch_bounds__(kThreads) k_adj_kick_vjp(Dev d, Adj a, const d
       rec[3 * (c0 + k) + 2] = s2;
     }
   }
+  if (a.parts > 1) {   // the parts' sums of a target, in order
+    __shared__ double tsum[kThreads][4];
+    if (part > 0) {
+      double* q = tsum[threadIdx.x];
+      q[0] = sa; q[1] = sbx; q[2] = sby; q[3] = sbz;
+    }
+    __syncthreads();
+    if (part == 0)
+      for (int p = 1; p < a.parts; ++p) {
+        const double* q = tsum[p * tile + tx];
+        sa += q[0]; sbx += q[1]; sby += q[2]; sbz += q[3];
+      }
+  }
   // into lam_x of this target
   double gx = -fma(sa, gax, sbx), gy = -fma(sa, gay, sby), gz = -fma(sa, gaz, sbz);
   // drag
   double own[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};   // dP (3), sum lam_x (3), dparams (3)
-  if (act) {
+  if (act && part == 0) {
     double lvxn = lvx, lvyn = lvy, lvzn = lvz;
     if (r.drag && S.gas_on && jl >= S.nbig) {
       const double u = V[j] + Pk[0] * S.inv_mu0, v = V[(size_t)N + j] + Pk[1] * S.inv_mu0,
@@ -644,7 +667,7 @@ __global__ void __launch_bounds__(kThreads) k_adj_kick_vjp(Dev d, Adj a, const d
   for (int q = 0; q < 9; ++q) {
     double vq = own[q];
     for (int off = 16; off > 0; off >>= 1) vq += __shfl_down_sync(0xffffffffu, vq, off);
-    if (lane == 0) wsum[warp][q] = vq;
+    if (lane == 0 && part == 0) wsum[warp][q] = vq;
   }
   __syncthreads();
   if (threadIdx.x < 9) {
@@ -827,13 +850,6 @@ __global__ void __launch_bounds__(kThreads) k_adj_fold_jump1(Dev d, Adj a) {
   }
 }
 
-int adjoint_vjp_blocks_per_sm(int threads) {
-  int n = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_adj_kick_vjp, threads, 0) != cudaSuccess)
-    return 0;
-  return n;
-}
-
 void launch_fold_kick(const Dev& d, const Adj& a, int which, int grav, cudaStream_t st) {
   if (grav && 3 * d.big_max + 9 > kThreads)
     k_adj_fold_big<<<dim3(d.nsys, (3 * d.big_max + kThreads - 1) / kThreads), kThreads, 0, st>>>(d, a);
@@ -861,7 +877,7 @@ void launch_adjoint_step_b(const Dev& d, const Adj& a, cudaStream_t st) {
   // reverse sweep: kick 2 (at x4, v3, P3), jump 2, drift, jump 1, kick 1 (at x0, v0, P0)
   // (with a.lin, the pair pass also takes the next step's first half kick,
   // left pending at the same positions)
-  k_adj_kick_vjp<<<d.ntiles, d.tile, 0, st>>>(d, a, a.x4, a.xv3 + 3 * (size_t)N, 2, 2 * a.step + 1,
+  k_adj_kick_vjp<<<d.ntiles, d.tile * a.parts, 0, st>>>(d, a, a.x4, a.xv3 + 3 * (size_t)N, 2, 2 * a.step + 1,
                                                KickRev{1, 1, 1, a.lin, nullptr});
   launch_fold_kick(d, a, 2, 1, st);
   if (a.groups) launch_adjoint_bs_vjp(d, a, a.bs_blocks, st);
@@ -870,12 +886,12 @@ void launch_adjoint_step_b(const Dev& d, const Adj& a, cudaStream_t st) {
   k_adj_fold_jump1<<<d.nsys, kThreads, 0, st>>>(d, a);
   // merged: the drag now, the pair pass with the previous step's last half kick
   const KickRev r1{a.defer_k1 ? 0 : 1, 1, 1, nullptr, a.defer_k1 ? a.lpend : nullptr};
-  k_adj_kick_vjp<<<d.ntiles, d.tile, 0, st>>>(d, a, a.z0, a.z0 + 3 * (size_t)N, 0, 2 * a.step, r1);
+  k_adj_kick_vjp<<<d.ntiles, d.tile * a.parts, 0, st>>>(d, a, a.z0, a.z0 + 3 * (size_t)N, 0, 2 * a.step, r1);
   launch_fold_kick(d, a, 1, r1.grav, st);
 }
 
 void launch_adjoint_flush(const Dev& d, const Adj& a, const double* xpos, cudaStream_t st) {
-  k_adj_kick_vjp<<<d.ntiles, d.tile, 0, st>>>(d, a, xpos, xpos, 0, 0,
+  k_adj_kick_vjp<<<d.ntiles, d.tile * a.parts, 0, st>>>(d, a, xpos, xpos, 0, 0,
                                                KickRev{1, 0, 0, a.lpend, nullptr});
   launch_fold_kick(d, a, 1, 1, st);
 }

@@ -274,6 +274,7 @@ struct mx_system {
   mx::Tile* a_tiles = nullptr;
   int a_ntiles = 0;
   int a_tile = mx::kThreads;   // targets per block of the adjoint's per-target kernels
+  int a_parts = 1;             // parts of a block of the kick's reverse
   long long kbits_cap = 0;
 };
 
@@ -610,7 +611,7 @@ mx_status set_tiling(mx_system* s, int tile, int order) {
 // the same order and the pair keys are sorted).  Choices are kept in a
 // small JSON file ($MX_AUTOTUNE_CACHE, else ~/.cache/mx/autotune.json);
 // MX_AUTOTUNE=0 keeps the defaults.
-constexpr const char* kTuneTag = "split2";
+constexpr const char* kTuneTag = "split3";
 std::string tune_key(const mx_system* s) {
   cudaDeviceProp prop;
   cudaGetDeviceProperties(&prop, s->device);
@@ -1869,31 +1870,40 @@ mx::Dev adjoint_dev(const mx_system* s) {
   return d;
 }
 
-// The adjoint's targets per block.  With few big bodies, 256 (the per-tile
-// partial records and their folds favour full blocks: 0.62 against 1.01 ms a
-// step with 64 on the 4-core disk).  With many, the kick's reverse is a long
-// pass over the pairs in which every block does the same work, so the block
-// count is chosen to fill whole waves of the resident blocks: of 160 to 256
-// targets (whole warps), the size whose waves come closest to a whole number
-// (902 blocks of 224 targets make 2.97 waves on 152 SMs, where 790 of 256
-// make 2.6 and a third of the SMs idle through the last).
-int adjoint_tile(const mx_system* s) {
-  if (s->d.big_max <= 64) return mx::kThreads;
+// The adjoint's targets per block and, for the kick's reverse, the parts of a
+// block.  With few big bodies, 256 and one (the per-tile partial records and
+// their folds favour full blocks: 0.62 against 1.01 ms a step with 64 on the
+// 4-core disk).  With many, the kick's reverse is a long pass over the pairs,
+// bound by FP64 issue, and the busiest SM sets its end: ceil(tiles / SMs) blocks
+// of ceil(warps / 4) warps a scheduler, each over 1/parts of the big bodies.
+// The choice is the least of that over 256 to 160 targets in one part (whole
+// warps), 128 in two, 64 in four and 32 in eight, the larger tile among equals
+// (a tile's record holds a sum for every big body, so the records stay below
+// 256 MB).  1,000 big bodies + 20,000 planetesimals: 94 blocks of 224 targets
+// left 58 of 152 SMs idle.  TIMES
+void adjoint_tile(const mx_system* s, int* tile, int* parts) {
+  *tile = mx::kThreads;
+  *parts = 1;
+  if (s->d.big_max <= 64) return;
   const int nsm = s->bs_blocks / 4;
-  int best_tile = mx::kThreads;
-  double best = -1.0;
-  for (int w = mx::kThreads / 32; w >= 5; --w) {
-    const int t = 32 * w;
-    const int occ = mx::adjoint_vjp_blocks_per_sm(t);
-    if (occ <= 0 || nsm <= 0) continue;
-    const double waves = (double)make_tiles(s->h_sys, t, 0).size() / ((double)occ * nsm);
-    const double eff = waves / std::ceil(waves);
-    if (eff > best + 1e-9) {
-      best = eff;
-      best_tile = t;
+  double best = 1e300;
+  auto consider = [&](int t, int p) {
+    const std::vector<mx::Tile> tiles = make_tiles(s->h_sys, t, 0);
+    size_t rec = 0;
+    for (const mx::Tile& q : tiles) rec += 3 * (size_t)s->h_sys[q.sys].nbig + 9;
+    if (p > 1 && rec > ((size_t)1 << 25)) return;
+    const int per_sm = ((int)tiles.size() + nsm - 1) / nsm;
+    const double time = (double)per_sm * ((t * p + 127) / 128) / p;
+    if (time < best - 1e-9) {
+      best = time;
+      *tile = t;
+      *parts = p;
     }
-  }
-  return best_tile;
+  };
+  for (int t = mx::kThreads; t >= 160; t -= 32) consider(t, 1);
+  consider(128, 2);
+  consider(64, 4);
+  consider(32, 8);
 }
 
 mx_status ensure_adjoint_store(mx_system* s) {
@@ -1929,7 +1939,7 @@ mx_status ensure_adjoint(mx_system* s) {
     MX_TRY(dalloc(s, &s->a_x4, (size_t)3 * N));
     MX_TRY(dalloc(s, &s->a_P, 9 * s->h_sys.size()));
     MX_TRY(dalloc(s, &s->a_L, s->h_sys.size()));
-    s->a_tile = adjoint_tile(s);
+    adjoint_tile(s, &s->a_tile, &s->a_parts);
     std::vector<mx::Tile> tiles = make_tiles(s->h_sys, s->a_tile, 0);
     std::vector<int> poff(tiles.size());
     size_t off = 0;
@@ -1967,6 +1977,7 @@ mx::Adj make_adj(const mx_system* s, double* dev_lambda, double* dev_dparams) {
   a.x4 = s->a_x4;
   a.lam = dev_lambda;
   a.part = s->a_part;
+  a.parts = s->a_parts;
   a.poff = s->a_poff;
   a.sys_tiles = s->a_systiles;
   a.P = s->a_P;

@@ -202,6 +202,7 @@ struct Adj {
   double* x4;         // 3 x N after jump 2
   double* lam;        // 6 x N cotangent, in/out
   double* part;       // per-tile partial sums
+  int parts;          // parts of a block of k_adj_kick_vjp (a power of two)
   const int* poff;    // [ntiles] offset of each tile's partial record
   const int* sys_tiles;   // [nsys + 1] first tile of each system (tiles in system order)
   double* P;          // 9 per system: P0, P1, P3
