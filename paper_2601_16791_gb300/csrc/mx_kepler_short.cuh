@@ -10,7 +10,7 @@
 // in FP32 first; one FP64 evaluation there gives the last correction d (about
 // 1e-7), and U1..U3 are carried to sigma + d by their Taylor steps.  The state
 // moves by the differences f - 1 = -m U2, g = h - h m U3, gd - 1 = -m U2/rho,
-// fd = -(m/h) U1/rho, rho = r/r0 = 1 + a U1 + c U2.  About 75 FP64
+// fd = -(m/h) U1/rho, rho = r/r0 = 1 + a U1 + c U2.  About 77 FP64
 // instructions.  Against 64-bit-mantissa arithmetic over 20,000 orbits (1 to 15
 // AU, h = 10 d): position 5.7e-17 rms (kepler_drift 5.7e-17), velocity 6.8e-17
 // (7.6e-17).  Measured: mx_kepler_drift of 200,000 bodies 74.5 -> 59.6 us a call;
@@ -23,8 +23,11 @@
 namespace mx {
 
 // Advances the state and returns true, or returns false with it untouched:
-// |b| above 0.04 (a step of about 0.2 rad of mean motion), |a| above 0.25, a
-// value off FP32's range or not finite, or a correction above 4e-6.
+// |b| above 0.12 (a step of about 0.35 rad of mean motion), |a| or |c| above 0.25,
+// a value off FP32's range or not finite, or a correction above 4e-6.  (A warp
+// with one such body runs both forms, so the range covers the whole disk of the
+// usual step, about a twentieth of the innermost orbit: with |b| to 0.04 an
+// embryo disk from 0.5 AU at h = 6 d took 83 us a launch against 68 before.)
 __device__ __forceinline__ bool kepler_drift_short(double mu, double h, double& x, double& y,
                                                    double& z, double& u, double& v, double& w) {
   const double r02 = fma(x, x, fma(y, y, z * z));
@@ -40,7 +43,7 @@ __device__ __forceinline__ bool kepler_drift_short(double mu, double h, double& 
   // r0 in 2^-40 .. 2^40 and m above 2^-80 (h = 0 goes the general way)
   const int hr = __double2hiint(r02) >> 20;
   if (!(hr > 1023 - 80 && hr < 1023 + 80 && __double2hiint(m) >= (1023 - 80) << 20 &&
-        abs_le(b, 0.04) && abs_le(a, 0.25) && abs_le(c, 0.25)))
+        abs_le(b, 0.12) && abs_le(a, 0.25) && abs_le(c, 0.25)))
     return false;
   const float af = ff_of(a).h, bf = ff_of(b).h, cf = ff_of(c).h;
   // FP32: the series inverted to third order, then two Halley corrections
@@ -58,17 +61,19 @@ __device__ __forceinline__ bool kepler_drift_short(double mu, double h, double& 
     s -= __fdividef(F * Fp, fmaf(Fp, Fp, -0.5f * F * Fpp));
   }
   // FP64 at sigma = s (24 bits, so s - 1 and s^2 are exact): the series with
-  // their tails from z^3 on in FP32 (1e-4 of the sum)
+  // their tails from z^4 on in FP32 (1e-8 of the sum)
   const double sd = bits_to_double(s);
   const double s2 = sd * sd;
   const double zd = b * s2;
   const float zf = ff_of(zd).h;
-  const double t2 = bits_to_double(fmaf(-zf, fmaf(-zf, 1.0f / 479001600.0f, 1.0f / 3628800.0f),
-                                        1.0f / 40320.0f));
-  const double t3 = bits_to_double(fmaf(-zf, fmaf(-zf, 1.0f / 6227020800.0f, 1.0f / 39916800.0f),
-                                        1.0f / 362880.0f));
-  const double c2 = fma(-zd, fma(-zd, fma(-zd, t2, 1.0 / 720.0), 1.0 / 24.0), 0.5);
-  const double c3 = fma(-zd, fma(-zd, fma(-zd, t3, 1.0 / 5040.0), 1.0 / 120.0), 1.0 / 6.0);
+  const double t2 = bits_to_double(fmaf(-zf, fmaf(-zf, 1.0f / 87178291200.0f, 1.0f / 479001600.0f),
+                                        1.0f / 3628800.0f));
+  const double t3 = bits_to_double(fmaf(-zf, fmaf(-zf, 1.0f / 1307674368000.0f, 1.0f / 6227020800.0f),
+                                        1.0f / 39916800.0f));
+  const double c2 =
+      fma(-zd, fma(-zd, fma(-zd, fma(-zd, t2, 1.0 / 40320.0), 1.0 / 720.0), 1.0 / 24.0), 0.5);
+  const double c3 =
+      fma(-zd, fma(-zd, fma(-zd, fma(-zd, t3, 1.0 / 362880.0), 1.0 / 5040.0), 1.0 / 120.0), 1.0 / 6.0);
   const double U2 = s2 * c2, U3 = (s2 * sd) * c3;
   const double U1 = fma(-b, U3, sd);
   const double F = fma(c, U3, fma(a, U2, bits_to_double(s - 1.0f)));

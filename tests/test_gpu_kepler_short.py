@@ -34,8 +34,8 @@ def gauss(xv, mu, h):
 
 
 @pytest.mark.parametrize("nh,emax,sign", [
-    (1e-6, 0.05, 1), (0.01, 0.3, -1), (0.1, 0.05, 1), (0.17, 0.3, 1), (0.1995, 0.001, 1),
-    (0.2005, 0.001, -1), (0.21, 0.1, 1), (0.02, 0.5, 1),
+    (1e-6, 0.05, 1), (0.01, 0.3, -1), (0.1, 0.05, 1), (0.17, 0.3, 1), (0.1995, 0.001, 1), (0.345, 0.001, 1),
+    (0.348, 0.001, -1), (0.3, 0.1, 1), (0.02, 0.5, 1),
 ])
 @pytest.mark.parametrize("scale", [1e-3, 1.0, 1e4])
 def test_short_drift(nh, emax, sign, scale):
