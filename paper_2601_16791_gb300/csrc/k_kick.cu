@@ -48,8 +48,9 @@ __global__ void __launch_bounds__(kThreads, 2) k_accel(Dev d, double* acc, int d
   const SysDev& S = d.sys[t.sys];
   const double* P = d.P + 3 * t.sys;
   const int N = d.N;
-  const bool valid = threadIdx.x < t.count;
-  const int j = t.start + threadIdx.x;
+  const int part = threadIdx.x / d.tile, tx = threadIdx.x - part * d.tile;
+  const bool valid = tx < t.count;
+  const int j = t.start + tx;
   const bool act = valid && !removed(d, j);   // a removed body gets zero
   const int jl = j - S.off;
   double x = 0, y = 0, z = 0, u = 0, v = 0, w = 0, rcj = 0.0;
@@ -65,8 +66,9 @@ __global__ void __launch_bounds__(kThreads, 2) k_accel(Dev d, double* acc, int d
   double ax = 0, ay = 0, az = 0;
   SplitAcc3 sum{};
   if (!drag_only)
-    gravity_split<TripleSum, true>(d, S, sb, act, jl, rcj, x, y, z, ax, ay, az, sum, nullptr);
-  if (!valid) return;
+    gravity_split<TripleSum, true>(d, S, sb, act, jl, rcj, x, y, z, ax, ay, az, sum, nullptr,
+                                   blockDim.x / d.tile, part, tx);
+  if (!valid || part > 0) return;
   const bool drag = act && S.gas_on && jl >= S.nbig;
   double a[3] = {0.0, 0.0, 0.0};
   if (drag) {
@@ -91,25 +93,31 @@ void launch_prep(const Dev& d, double jump_frac, int nkick, cudaStream_t st) {
   k_prep<<<d.nsys, kThreads, 0, st>>>(d, jump_frac, nkick);
 }
 
+static int kick_threads(const Dev& d) {
+  return d.split_mode == kSplitAny ? d.tile * d.kick_parts : d.tile;
+}
+
 void launch_jump_kick(const Dev& d, double jump_frac, double kick_frac, int nkick,
                       cudaStream_t st) {
   const size_t sm = kick_smem_bytes(d, false);
   const KickKernel k =
       nkick == 2 ? kick_kernel<2, false>(d.split_mode) : kick_kernel<1, false>(d.split_mode);
-  k<<<d.ntiles, d.tile, sm, st>>>(d, jump_frac, kick_frac);
+  k<<<d.ntiles, kick_threads(d), sm, st>>>(d, jump_frac, kick_frac);
 }
 
 // The interior steps' kick with its own prep (no k_prep launch before it):
 // jump 1/2, two half kicks; for forward runs without growth tracks or k
 // branches recorded or replayed.
 void launch_jump_kick_fused(const Dev& d, cudaStream_t st) {
-  kick_kernel<2, true>(d.split_mode)<<<d.ntiles, d.tile, kick_smem_bytes(d, true), st>>>(d, 0.5, 0.5);
+  kick_kernel<2, true>(d.split_mode)<<<d.ntiles, kick_threads(d), kick_smem_bytes(d, true), st>>>(
+      d, 0.5, 0.5);
 }
 
 void launch_accel(const Dev& d, double* acc, int drag_only, int acc_stride, int acc_base,
                   cudaStream_t st) {
-  const size_t sm = stage_bytes(d.big_max) + sizeof(SplitBig3) * (size_t)big_chunk(d.big_max);
-  k_accel<<<d.ntiles, d.tile, sm, st>>>(d, acc, drag_only, acc_stride, acc_base);
+  const size_t sm = stage_bytes(d.big_max) + sizeof(SplitBig3) * (size_t)big_chunk(d.big_max) +
+                    seg_bytes(d.tile, d.kick_parts);
+  k_accel<<<d.ntiles, d.tile * d.kick_parts, sm, st>>>(d, acc, drag_only, acc_stride, acc_base);
 }
 
 // The kernels of a step share one shared-memory carveout (the largest), so

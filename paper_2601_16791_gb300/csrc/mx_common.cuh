@@ -106,6 +106,7 @@ struct Dev {
   unsigned char* flags;               // N
   unsigned long long* keys;           // pair keys [pair_cap]
   unsigned long long* sort_tmp;       // [kSortTmp] scratch of launch_sort_keys
+  int kick_parts;                     // parts of a block of the kick and of k_accel (kick_parts)
   int bb_only;                        // 1: k_groups lists the groups of big bodies only
   int* pair_count;
   int* work_count;

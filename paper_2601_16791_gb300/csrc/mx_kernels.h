@@ -25,6 +25,18 @@ void launch_dfma(double* sink, int blocks, int iters, cudaStream_t st);
 
 // k_kick.cu
 void launch_prep(const Dev& d, double jump_frac, int nkick, cudaStream_t st);
+// Parts of a kick's block (a power of two): each part takes the block's targets
+// and a share of the big bodies.  As many as fit in 256 threads, up to 16 warps
+// an SM over the launch: with 301 big bodies + 20,011 planetesimals one part
+// leaves a scheduler a single warp, whose dependent FP32 chain fills less than
+// half of the issue slots (k_jump_kick 65 -> 48 us a launch in four parts); with
+// 200,000 planetesimals there are warps enough, and parts cost 3 to 10%.
+inline int kick_parts(int tile, int ntiles, int big_max, int nsm) {
+  int p = 1;
+  if (big_max > kDeferMaxBig)
+    while (2 * p * tile <= kThreads && (long long)ntiles * (tile / 32) * p < 16LL * nsm) p *= 2;
+  return p;
+}
 void launch_jump_kick(const Dev& d, double jump_frac, double kick_frac, int nkick, cudaStream_t st);
 void launch_jump_kick_fused(const Dev& d, cudaStream_t st);
 void launch_accel(const Dev& d, double* acc, int drag_only, int acc_stride, int acc_base,

@@ -74,7 +74,7 @@ __device__ __forceinline__ void gravity_all(const Dev& d, const SysDev& S, BigSm
 
 // Systems with at most kDeferMaxBig big bodies keep the pair sum in FP32 pairs
 // up to the velocity update (split_kicks), which the catch-up of deferred
-// planetesimals repeats; with more, it goes into FP64 every kSplitRun bodies.
+// planetesimals repeats; with more, it goes into FP64 every kSplitSeg bodies.
 __host__ __device__ __forceinline__ bool split_flushes(int nbig) { return nbig > kDeferMaxBig; }
 
 // Bytes of the FP64 staging (nine arrays of doubles), rounded up for the
@@ -98,20 +98,32 @@ __device__ __forceinline__ SplitBig split_big(double x, double y, double z, doub
   return b;
 }
 
+// The parts' sums of a chunk of big bodies, by segment and target.
+constexpr int kSplitSeg = 64;
+__host__ __device__ __forceinline__ size_t seg_bytes(int tile, int parts) {
+  return parts > 1 ? 3 * sizeof(double) * (size_t)tile * 4 : 0;   // a chunk has at most four
+}
+
 // Gravity on target j (local index jl, own changeover radius rcj) from all big
 // bodies of its system.  Far pairs are formed in FP32 pairs and summed (sign
 // reversed) in acc, which a system with many big bodies (split_flushes) empties
 // into (ax, ay, az) as it goes; pairs inside the changeover shell, and every
 // pair of a target off the positions' grid, go through the FP64 pair_acc into
 // (ax, ay, az).  Every thread of the block must call it.
+// A system with many big bodies is summed by segments of kSplitSeg, each from
+// zero, and the segments in order, so that the parts of a block can share them
+// (segment s goes to part s mod parts) with the same bits; part 0 (thread tx
+// of it) ends up with the sum.
 template <class Sum, bool MANY>
 __device__ __forceinline__ void gravity_split(const Dev& d, const SysDev& S, BigSmem& sb,
                                               bool act, int jl, double rcj, double x, double y,
                                               double z, double& ax, double& ay, double& az,
-                                              typename Sum::Acc& acc, const double* dj) {
+                                              typename Sum::Acc& acc, const double* dj, int parts,
+                                              int part, int tx) {
   __shared__ int s_hi;
   using Big = typename Sum::Big;
   Big* sp = reinterpret_cast<Big*>(reinterpret_cast<unsigned char*>(sb.x) + stage_bytes(d.big_max));
+  double* ss = reinterpret_cast<double*>(sp + big_chunk(d.big_max));   // seg_bytes
   const bool jbig = jl < S.nbig;
   const bool flush = MANY && (!std::is_same<Sum, PairSum>::value || split_flushes(S.nbig));
   const float near_own = jbig ? near2_of(rcj * rcj) : 0.0f;
@@ -142,58 +154,96 @@ __device__ __forceinline__ void gravity_split(const Dev& d, const SysDev& S, Big
       for (int k = threadIdx.x; k < cn; k += blockDim.x)
         sp[k] = Sum::make(split_big(sb.x[k], sb.y[k], sb.z[k], sb.mu[k], sb.rc2[k], kg), sb.mu[k]);
     __syncthreads();
-    if (!act) continue;
+    double lx = 0, ly = 0, lz = 0;   // a segment's sum, or without segments (ax, ay, az)
     auto pair64 = [&](int k) {
       if (jbig) {
         if (c0 + k == jl) return;
         const double rc = fmax(sb.rc[k], rcj);
         pair_acc(x - sb.x[k], y - sb.y[k], z - sb.z[k], sb.mu[k], rc * rc, 0.01 * (rc * rc),
-                 0.1 * rc, 1.0 / (0.9 * rc), ax, ay, az);
+                 0.1 * rc, 1.0 / (0.9 * rc), lx, ly, lz);
       } else {
         pair_acc(x - sb.x[k], y - sb.y[k], z - sb.z[k], sb.mu[k], sb.rc2[k], sb.rc2lo[k],
-                 sb.rc01[k], sb.i09rc[k], ax, ay, az);
+                 sb.rc01[k], sb.i09rc[k], lx, ly, lz);
       }
     };
-    if (!grid || !split_in_range(x, y, z, kg)) {
-#pragma unroll 1
-      for (int k = 0; k < cn; ++k) pair64(k);
-      continue;
+    if (!flush) {
+      if (!act || part > 0) continue;
+      lx = ax;
+      ly = ay;
+      lz = az;
     }
-    if (kt != kg) {
+    const bool far_ok = act && grid && split_in_range(x, y, z, kg);
+    if (far_ok && kt != kg) {
       kt = kg;
       split3(x, kg, t.x0, t.x1, t.x2);
       split3(y, kg, t.y0, t.y1, t.y2);
       split3(z, kg, t.z0, t.z1, t.z2);
     }
+    const int step = flush ? kSplitSeg : cn, run = flush ? kSplitSeg : kSplitRun;
 #pragma unroll 1
-    for (int k0 = 0; k0 < cn; k0 += kSplitRun) {
-      const int kn = min(cn, k0 + kSplitRun);
-      if constexpr (std::is_same<Sum, PairSum>::value && MANY) {
-        // two pairs at a time, the rare near ones after both: a branch behind
-        // each pair kept the scheduler to one dependent chain a warp.
-        // Measured: 1.77 -> 1.65 ms a launch (two half kicks), 2,000 big
-        // bodies + 200,000 planetesimals.
-        int k = k0;
+    for (int s0 = 0, seg = 0; s0 < cn; s0 += step, ++seg) {
+      if (flush && (seg & (parts - 1)) != part) continue;
+      const int sn = min(cn, s0 + step);
+      if (flush) lx = ly = lz = 0.0;
+      if (act && !far_ok) {
 #pragma unroll 1
-        for (; k + 1 < kn; k += 2) {
-          SplitTerm f0, f1;
-          const bool far0 = split_term(t, sp[k], fmaxf(sp[k].near2, near_own), f0);
-          const bool far1 = split_term(t, sp[k + 1], fmaxf(sp[k + 1].near2, near_own), f1);
-          split_sum(acc, f0);
-          split_sum(acc, f1);
-          if (!(far0 && far1)) {
-            if (!far0) pair64(k);
-            if (!far1) pair64(k + 1);
-          }
-        }
-        if (k < kn && !Sum::term(t, sp[k], fmaxf(sp[k].near2, near_own), acc)) pair64(k);
-      } else {
+        for (int k = s0; k < sn; ++k) pair64(k);
+      } else if (act) {
+#pragma unroll 1
+        for (int k0 = s0; k0 < sn; k0 += run) {
+          const int kn = min(sn, k0 + run);
+          if constexpr (std::is_same<Sum, PairSum>::value && MANY) {
+            // two pairs at a time, the rare near ones after both: a branch behind
+            // each pair kept the scheduler to one dependent chain a warp.
+            // Measured: 1.77 -> 1.65 ms a launch (two half kicks), 2,000 big
+            // bodies + 200,000 planetesimals.
+            int k = k0;
+#pragma unroll 1
+            for (; k + 1 < kn; k += 2) {
+              SplitTerm f0, f1;
+              const bool far0 = split_term(t, sp[k], fmaxf(sp[k].near2, near_own), f0);
+              const bool far1 = split_term(t, sp[k + 1], fmaxf(sp[k + 1].near2, near_own), f1);
+              split_sum(acc, f0);
+              split_sum(acc, f1);
+              if (!(far0 && far1)) {
+                if (!far0) pair64(k);
+                if (!far1) pair64(k + 1);
+              }
+            }
+            if (k < kn && !Sum::term(t, sp[k], fmaxf(sp[k].near2, near_own), acc)) pair64(k);
+          } else {
 #pragma unroll 2
-        for (int k = k0; k < kn; ++k)
-          if (!Sum::term(t, sp[k], fmaxf(Sum::near2(sp[k]), near_own), acc)) pair64(k);
+            for (int k = k0; k < kn; ++k)
+              if (!Sum::term(t, sp[k], fmaxf(Sum::near2(sp[k]), near_own), acc)) pair64(k);
+          }
+          if (flush) Sum::flush(acc, lx, ly, lz);
+          else Sum::renorm(acc);
+        }
       }
-      if (flush) Sum::flush(acc, ax, ay, az);
-      else Sum::renorm(acc);
+      if (!flush) {
+        ax = lx;
+        ay = ly;
+        az = lz;
+      } else if (parts == 1) {
+        ax += lx;
+        ay += ly;
+        az += lz;
+      } else {
+        double* q = ss + 3 * ((size_t)seg * d.tile + tx);
+        q[0] = lx;
+        q[1] = ly;
+        q[2] = lz;
+      }
+    }
+    if (flush && parts > 1) {
+      __syncthreads();
+      if (part == 0)
+        for (int seg = 0; seg * kSplitSeg < cn; ++seg) {
+          const double* q = ss + 3 * ((size_t)seg * d.tile + tx);
+          ax += q[0];
+          ay += q[1];
+          az += q[2];
+        }
     }
   }
 }
@@ -463,10 +513,13 @@ __device__ __forceinline__ void jump_kick_tile(const Dev& d, double jump_frac, d
     for (int c = 0; c < 3; ++c) hp[c] = Pv[c] * S.inv_mu0;
   }
   const double kick_h = kick_frac * S.h;
-  const int j = t.start + threadIdx.x;
+  const int parts = MODE == kSplitAny ? (int)(blockDim.x / d.tile) : 1;
+  const int part = MODE == kSplitAny ? (int)(threadIdx.x / d.tile) : 0;
+  const int tx = threadIdx.x - part * d.tile;
+  const int j = t.start + tx;
   // a deferred planetesimal is kicked by the window's catch-up instead; a
   // removed body is not kicked
-  const bool act = threadIdx.x < t.count && !(d.defer && d.lag[j]) && !removed(d, j);
+  const bool act = tx < t.count && !(d.defer && d.lag[j]) && !removed(d, j);
   const int jl = j - S.off;
   double x = 0, y = 0, z = 0, u = 0, v = 0, w = 0, rcj = 0.0;
   if (act) {
@@ -483,10 +536,10 @@ __device__ __forceinline__ void jump_kick_tile(const Dev& d, double jump_frac, d
   const bool split = MODE == kSplitFew || (MODE == kSplitAny && S.split);
   if (split)
     gravity_split<PairSum, MODE == kSplitAny>(d, S, sb, act, jl, rcj, x, y, z, ax, ay, az, acc,
-                                     FUSED ? dj : nullptr);
+                                              FUSED ? dj : nullptr, parts, part, tx);
   else
-    gravity_all(d, S, sb, act, jl, rcj, x, y, z, ax, ay, az, FUSED ? dj : nullptr);
-  if (!act) return;
+    gravity_all(d, S, sb, act && part == 0, jl, rcj, x, y, z, ax, ay, az, FUSED ? dj : nullptr);
+  if (!act || part > 0) return;
   const bool big = jl < S.nbig;
   if (__double_as_longlong(jump_frac) != 0 && !(FUSED && big)) {   // jump_frac is +0 or 1/2
     d.xv[j] = x;
@@ -569,6 +622,7 @@ __device__ __forceinline__ void jump_kick_tile(const Dev& d, double jump_frac, d
 __host__ __device__ __forceinline__ size_t kick_smem_bytes(const Dev& d, bool fused) {
   size_t n = stage_bytes(d.big_max);
   n += sizeof(SplitBig) * (size_t)big_chunk(d.big_max);
+  if (d.split_mode == kSplitAny) n += seg_bytes(d.tile, d.kick_parts);
   if (fused && d.big_max > 32) n = n < 3 * kThreads * sizeof(double) ? 3 * kThreads * sizeof(double) : n;
   return n;
 }

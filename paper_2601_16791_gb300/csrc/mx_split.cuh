@@ -38,7 +38,7 @@
 
 namespace mx {
 
-constexpr int kSplitRun = 32;     // big bodies summed in FP32 pairs between FP64 adds
+constexpr int kSplitRun = 32;     // big bodies summed in FP32 pairs before the low parts are put back below the high ones
 constexpr int kSplitMinK = -10;   // positions' grid: 2^k AU above the big bodies' coordinates,
 constexpr int kSplitMaxK = 10;    // else the pair sum stays FP64 (FP32 range of mu/s^3)
 
@@ -288,7 +288,7 @@ __device__ __forceinline__ void split_flush(SplitAcc& acc, double& ax, double& a
 // The same sum for mx_accel, which returns the acceleration itself: every
 // quantity carries a third FP32 part, so that a pair's relative error is 8e-20
 // (rms, against 80-bit arithmetic; FP64's is 1.3e-16) and what is left of the
-// sum's is its FP64 adds, one in kSplitRun.  About 340 FP32 instructions a pair
+// sum's is its FP64 adds, one in kSplitSeg.  About 340 FP32 instructions a pair
 // against pair_acc's 17 of 64 cycles.  Measured: k_accel with 2,000 big bodies
 // and 200,000 planetesimals 11.8 -> 4.57 ms (87% of the issue slots filled), and the
 // result's error against a 64-bit sum over all pairs 1.5e-15 -> 6.5e-16.
