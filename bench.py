@@ -263,11 +263,12 @@ def source_hash(names):
 
 
 KERNEL_SOURCES = {"k_jump_kick": ["k_kick.cu", "mx_kick_body.cuh", "mx_common.cuh", "mx_physics.cuh",
-                                  "mx_growth.cuh"],
-                  "k_jump_drift": ["k_drift.cu", "mx_drift_body.cuh", "mx_common.cuh", "mx_kepler.cuh"],
+                                  "mx_growth.cuh", "mx_split.cuh", "mx_split_gas.cuh"],
+                  "k_jump_drift": ["k_drift.cu", "mx_drift_body.cuh", "mx_common.cuh", "mx_kepler.cuh",
+                                   "mx_kepler_short.cuh"],
                   "k_detect": ["k_detect.cu", "mx_detect_body.cuh", "mx_common.cuh",
                                "mx_encounter.cuh"],
-                  "k_bs": ["k_bs.cu", "mx_bs.cuh", "mx_common.cuh", "mx_physics.cuh"],
+                  "k_bs": ["k_bs.cu", "mx_bs.cuh", "mx_bs2.cuh", "mx_common.cuh", "mx_physics.cuh"],
                   "k_catchup": ["k_bs.cu", "mx_bs.cuh", "mx_common.cuh", "mx_physics.cuh",
                                 "mx_kepler.cuh", "mx_encounter.cuh"]}
 

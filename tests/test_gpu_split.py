@@ -156,3 +156,23 @@ def test_split_keeps_what_fp32_cannot_hold():
         g.step(1)
     g.close()
     assert e.value.code == 7   # MX_ERR_NONFINITE
+
+
+@pytest.mark.parametrize("nbig,nsmall", [(65, 40), (128, 700), (257, 1023), (300, 3000)])
+def test_parts_of_a_block_change_no_bit(nbig, nsmall):
+    """Tiles of 64, 96 or 128 targets share the big bodies among four or two
+    parts of a block, tiles of 256 do not: the same accelerations and states."""
+    w = W.semiactive_2000big_200k(seed=3, nbig=nbig, nsmall=nsmall)
+    out = []
+    for tile in (256, 64, 96, 128):
+        g = mx.System(w)
+        mx.mx_set_tiling(g.h, tile, 0)
+        acc = torch.empty((3, w.n), dtype=torch.float64, device="cuda")
+        xv = torch.empty((6, w.n), dtype=torch.float64, device="cuda")
+        mx.mx_accel(g.h, acc)
+        mx.mx_step(g.h, 3)
+        mx.mx_get_state_device(g.h, xv)
+        out.append((acc.cpu(), xv.cpu()))
+        g.close()
+    for acc, xv in out[1:]:
+        assert torch.equal(acc, out[0][0]) and torch.equal(xv, out[0][1])
