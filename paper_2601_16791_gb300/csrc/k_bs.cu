@@ -1535,6 +1535,13 @@ __device__ __noinline__ void catch_bs_thread(const Dev& d, const SysDev& S, cons
   for (int q = 0; q < 6; ++q) out[q] = Y[q][nb - 1];
 }
 
+// The drift of a light system's body.  Out of line, as catch_kick_light is: the
+// catch-up of systems with cores, whose hardest chains set its time, then keeps
+// its registers (k_catchup spilled 508 bytes of loads with both inline).
+static __device__ __noinline__ bool catch_drift_light(double mu, double h, int maxit, double* q) {
+  return kepler_drift_sel(true, mu, h, maxit, q[0], q[1], q[2], q[3], q[4], q[5]);
+}
+
 // Jump 1, drift and the encounter test of step t.  No encounter: returns 0
 // with the drifted state in s6.  A group of up to four bodies: returns its
 // size with the group set up in G (pre-drift states, a fresh step).  Larger
@@ -1553,8 +1560,16 @@ __device__ int catch_front(const Dev& d, const SysDev& S, int sys, int j, int t,
   double x = s6[0] + dj[0], y = s6[1] + dj[1], z = s6[2] + dj[2];
   double u = s6[3], v = s6[4], w = s6[5];
   const double a0[6] = {x, y, z, u, v, w};
-  if (!kepler_drift_sel(S.split, S.mu0, S.h, d.kepler_max_iter, x, y, z, u, v, w) && wr && lane == 0)
-    atomicOr(d.status, ST_KEPLER);
+  bool drifted = false;
+  if (S.split) {   // kepler_drift_sel, the light systems' part out of line
+    double q[6] = {x, y, z, u, v, w};
+    drifted = catch_drift_light(S.mu0, S.h, d.kepler_max_iter, q);
+    x = q[0]; y = q[1]; z = q[2];
+    u = q[3]; v = q[4]; w = q[5];
+  } else {
+    drifted = kepler_drift(S.mu0, S.h, d.kepler_max_iter, x, y, z, u, v, w);
+  }
+  if (!drifted && wr && lane == 0) atomicOr(d.status, ST_KEPLER);
   const double a1[6] = {x, y, z, u, v, w};
   float af[12];
   for (int k = 0; k < 6; ++k) {
@@ -1669,6 +1684,88 @@ __device__ int catch_front(const Dev& d, const SysDev& S, int sys, int j, int t,
   return 0;
 }
 
+// The half kicks of a light system's body in FP32 pairs (split_kicks): nk of
+// kick_h each, on the velocity in q[3..5] at the position q[0..2].
+static __device__ __noinline__ void catch_kick_light(const Dev& d, const SysDev& S, int nk,
+                                                     double kick_h, double hp0, double hp1,
+                                                     double hp2, double rp, double kd,
+                                                     const double* BX, const double* hmu,
+                                                     const double* hrc, double* q) {
+  const int lane = threadIdx.x & 31;
+  const double x = q[0], y = q[1], z = q[2];
+  double u = q[3], v = q[4], w = q[5];
+  double ax = 0, ay = 0, az = 0;
+  // the pairs' terms on the lanes (lane l: big body c0 + l), then the sum in
+  // ascending order, as the kick's loop makes it (the same bits)
+  SplitAcc acc{};
+  int hi = 0;
+  for (int l = lane; l < S.nbig; l += 32)
+    hi = max(hi, max(abs_hi(BX[l]), max(abs_hi(BX[d.NB + l]), abs_hi(BX[2 * (size_t)d.NB + l]))));
+  const int kg = split_k(__reduce_max_sync(0xffffffffu, hi));
+  const bool far_ok = kg <= kSplitMaxK && split_in_range(x, y, z, kg);
+  SplitPos tp{};
+  if (far_ok) {
+    split3(x, kg, tp.x0, tp.x1, tp.x2);
+    split3(y, kg, tp.y0, tp.y1, tp.y2);
+    split3(z, kg, tp.z0, tp.z1, tp.z2);
+  }
+  for (int c0 = 0; c0 < S.nbig; c0 += 32) {
+    const int l = c0 + lane;
+    double f = 0.0, ex = 0.0, ey = 0.0, ez = 0.0;
+    SplitTerm ft{};
+    bool near = false;
+    if (l < S.nbig) {
+      const double rc = hrc[l];
+      const double bx = BX[l], by = BX[d.NB + l], bz = BX[2 * (size_t)d.NB + l];
+      const double mu = fmax(hmu[l], 0.0);
+      if (far_ok) {
+        const SplitBig b = split_big(bx, by, bz, mu, rc * rc, kg);
+        near = !split_term(tp, b, b.near2, ft);
+      } else {
+        near = true;
+      }
+      if (near) {
+        ex = x - bx;
+        ey = y - by;
+        ez = z - bz;
+        f = pair_weight(ex, ey, ez, mu, rc * rc, 0.01 * (rc * rc), 0.1 * rc,
+                        (rc > 0.0) ? 1.0 / (0.9 * rc) : 0.0);
+      }
+    }
+    const int cn = min(32, S.nbig - c0);
+    const unsigned nearm = __ballot_sync(0xffffffffu, near);
+    for (int k = 0; k < cn; ++k) {
+      if ((nearm >> k) & 1u) {
+        const double fk = __shfl_sync(0xffffffffu, f, k);
+        ax = fma(-fk, __shfl_sync(0xffffffffu, ex, k), ax);
+        ay = fma(-fk, __shfl_sync(0xffffffffu, ey, k), ay);
+        az = fma(-fk, __shfl_sync(0xffffffffu, ez, k), az);
+      } else {
+        SplitTerm fk;
+        fk.xh = __shfl_sync(0xffffffffu, ft.xh, k);
+        fk.xl = __shfl_sync(0xffffffffu, ft.xl, k);
+        fk.yh = __shfl_sync(0xffffffffu, ft.yh, k);
+        fk.yl = __shfl_sync(0xffffffffu, ft.yl, k);
+        fk.zh = __shfl_sync(0xffffffffu, ft.zh, k);
+        fk.zl = __shfl_sync(0xffffffffu, ft.zl, k);
+        split_sum(acc, fk);
+      }
+    }
+    if (far_ok) split_renorm(acc);
+  }
+  DragSplit dc{};
+  if (S.gas_on) {
+    dc = drag_split(S, x, y, hp0, hp1, hp2, rp, kd);
+    ax += dc.adg[0];
+    ay += dc.adg[1];
+  }
+  split_kicks(S, kick_h, nk, split_gravity(acc, ax, ay, az), S.gas_on != 0, dc, x, y, hp0, hp1, hp2,
+              rp, kd, u, v, w, [](int) { return -1; }, [](int, int) {});
+  q[3] = u;
+  q[4] = v;
+  q[5] = w;
+}
+
 // Jump 2 and the half kick(s) that end step t, or (head) the leading half
 // kick of a call, which has no jump and keeps the positions as they are.
 __device__ void catch_back(const Dev& d, const SysDev& S, int sys, int j, int t, bool lead,
@@ -1691,72 +1788,11 @@ __device__ void catch_back(const Dev& d, const SysDev& S, int sys, int j, int t,
   const double hp0 = P2[0] * S.inv_mu0, hp1 = P2[1] * S.inv_mu0, hp2 = P2[2] * S.inv_mu0;
   const double rp = S.gas_on ? d.rp_cm[j] : 0.0, kd = S.gas_on ? d.kdrag[j] : 0.0;
   if (S.split) {
-    // the pairs' terms on the lanes (lane l: big body c0 + l), then the sum in
-    // ascending order, as the kick's loop makes it (the same bits)
-    SplitAcc acc{};
-    int hi = 0;
-    for (int l = lane; l < S.nbig; l += 32)
-      hi = max(hi, max(abs_hi(BX[l]), max(abs_hi(BX[d.NB + l]), abs_hi(BX[2 * (size_t)d.NB + l]))));
-    const int kg = split_k(__reduce_max_sync(0xffffffffu, hi));
-    const bool far_ok = kg <= kSplitMaxK && split_in_range(x, y, z, kg);
-    SplitPos tp{};
-    if (far_ok) {
-      split3(x, kg, tp.x0, tp.x1, tp.x2);
-      split3(y, kg, tp.y0, tp.y1, tp.y2);
-      split3(z, kg, tp.z0, tp.z1, tp.z2);
-    }
-    for (int c0 = 0; c0 < S.nbig; c0 += 32) {
-      const int l = c0 + lane;
-      double f = 0.0, ex = 0.0, ey = 0.0, ez = 0.0;
-      SplitTerm ft{};
-      bool near = false;
-      if (l < S.nbig) {
-        const double rc = hrc[l];
-        const double bx = BX[l], by = BX[d.NB + l], bz = BX[2 * (size_t)d.NB + l];
-        const double mu = fmax(hmu[l], 0.0);
-        if (far_ok) {
-          const SplitBig b = split_big(bx, by, bz, mu, rc * rc, kg);
-          near = !split_term(tp, b, b.near2, ft);
-        } else {
-          near = true;
-        }
-        if (near) {
-          ex = x - bx;
-          ey = y - by;
-          ez = z - bz;
-          f = pair_weight(ex, ey, ez, mu, rc * rc, 0.01 * (rc * rc), 0.1 * rc,
-                          (rc > 0.0) ? 1.0 / (0.9 * rc) : 0.0);
-        }
-      }
-      const int cn = min(32, S.nbig - c0);
-      const unsigned nearm = __ballot_sync(0xffffffffu, near);
-      for (int k = 0; k < cn; ++k) {
-        if ((nearm >> k) & 1u) {
-          const double fk = __shfl_sync(0xffffffffu, f, k);
-          ax = fma(-fk, __shfl_sync(0xffffffffu, ex, k), ax);
-          ay = fma(-fk, __shfl_sync(0xffffffffu, ey, k), ay);
-          az = fma(-fk, __shfl_sync(0xffffffffu, ez, k), az);
-        } else {
-          SplitTerm fk;
-          fk.xh = __shfl_sync(0xffffffffu, ft.xh, k);
-          fk.xl = __shfl_sync(0xffffffffu, ft.xl, k);
-          fk.yh = __shfl_sync(0xffffffffu, ft.yh, k);
-          fk.yl = __shfl_sync(0xffffffffu, ft.yl, k);
-          fk.zh = __shfl_sync(0xffffffffu, ft.zh, k);
-          fk.zl = __shfl_sync(0xffffffffu, ft.zl, k);
-          split_sum(acc, fk);
-        }
-      }
-      if (far_ok) split_renorm(acc);
-    }
-    DragSplit dc{};
-    if (S.gas_on) {
-      dc = drag_split(S, x, y, hp0, hp1, hp2, rp, kd);
-      ax += dc.adg[0];
-      ay += dc.adg[1];
-    }
-    split_kicks(S, kick_h, nk, split_gravity(acc, ax, ay, az), S.gas_on != 0, dc, x, y, hp0, hp1, hp2,
-                rp, kd, u, v, w, [](int) { return -1; }, [](int, int) {});
+    double q[6] = {x, y, z, u, v, w};
+    catch_kick_light(d, S, nk, kick_h, hp0, hp1, hp2, rp, kd, BX, hmu, hrc, q);
+    u = q[3];
+    v = q[4];
+    w = q[5];
   } else {
     // the pairs' weights on the lanes (lane l: big body c0 + l), then the sum
     // in ascending order, as the kick's loop makes it (the same bits)
