@@ -207,6 +207,7 @@ struct mx_system {
   cudaEvent_t mk_step[7] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
   long long step = 0;
   bool stepped = false;           // a step-taking call was made
+  bool tiled = false;             // the caller chose the tiling (mx_set_tiling)
   int eject_every = 0;            // ejection test schedule (Sec. 3.5), 0: none
   bool removed_any = false;       // a test outside the schedule removed bodies
   bool grow_any = false;          // some system follows growth tracks (mx_set_growth)
@@ -709,7 +710,8 @@ mx_status trial_ms(mx_system* s, double* ms) {
   cudaEventDestroy(e1);
   MX_CUDA(cudaMemcpyAsync(s->d.xv, s->d_tmp, bytes, cudaMemcpyDeviceToDevice, s->st));
   MX_CUDA(cudaMemsetAsync(s->d.pair_count, 0, 2 * sizeof(int), s->st));
-  // trials run at creation: the encounter log and the counters start empty
+  // trials run before the first step (build, retune): the encounter log and the
+  // counters start empty; retune puts the step index back
   MX_CUDA(cudaMemsetAsync(s->d.ever, 0, s->N, s->st));
   MX_CUDA(cudaMemsetAsync(s->d.bb_count, 0, sizeof(unsigned long long), s->st));
   MX_CUDA(cudaMemsetAsync(s->d.defer_total, 0, sizeof(unsigned long long), s->st));
@@ -754,6 +756,23 @@ mx_status autotune(mx_system* s) {
   MX_TRY(set_tiling(s, bt, bo));
   tune_store(key, bt, bo);
   return MX_OK;
+}
+
+// The tiling chosen again when the kick's kernel changes (mx_set_growth), where
+// it is still the autotuner's to choose and its trials leave nothing behind:
+// before the first step, with no k branches recorded or replayed (the trials'
+// kicks would record theirs), without the persistent step (whose tiles are full
+// blocks).  The state is kept by trial_ms; the caller may have set it, and the
+// step index with it, which the trials count on from.
+mx_status retune(mx_system* s) {
+  if (s->stepped || s->tiled || s->d.kmode != 0 || s->persist) return MX_OK;
+  const int tile = s->tile, order = s->order;
+  const long long catchups = s->catchups;
+  const mx_status r = autotune(s);
+  s->catchups = catchups;
+  if (r != MX_OK) set_tiling(s, tile, order);
+  mx::launch_set_step(s->d, s->step, s->st);
+  return r;
 }
 
 // Builds the device side of a batch of systems (one system = batch of one).
@@ -1105,6 +1124,7 @@ mx_status mx_set_tiling(mx_system* s, int tile, int order) {
   if (!s || !valid_tile(tile) || !(order == 0 || order == 1))
     return fail(MX_ERR_ARG, "tile must be a multiple of 32 from 64 to 256 and order 0 or 1");
   MX_TRY(set_device(s));
+  s->tiled = true;
   return set_tiling(s, tile, order);
 }
 
@@ -1736,10 +1756,20 @@ mx_status mx_set_growth(mx_system* s, int sys, const mx_growth* g, double gap_c)
   MX_TRY(settle(s));
   mx::SysDev& S = s->h_sys[sys];
   if (any && S.split) {   // masses change from here on: the FP64 kick, and its tile
-    S.split = 0;
-    MX_CUDA(cudaMemcpyAsync(s->d_sys + sys, &S, sizeof(mx::SysDev), cudaMemcpyHostToDevice, s->st));
-    s->d.split_mode = split_mode(s->h_sys);
-    if (!s->stepped && !s->grow_any) MX_TRY(autotune(s));   // its trials start from a fresh system
+    auto set_split = [&](int on) -> mx_status {
+      S.split = on;
+      s->d.split_mode = split_mode(s->h_sys);
+      drop_graphs(s);
+      MX_CUDA(cudaMemcpyAsync(s->d_sys + sys, &S, sizeof(mx::SysDev), cudaMemcpyHostToDevice, s->st));
+      return MX_OK;
+    };
+    mx_status r = set_split(0);
+    if (r == MX_OK && !s->grow_any) r = retune(s);
+    if (r != MX_OK) {   // the system as it was, without the track
+      const std::string msg = g_last_error;
+      set_split(1);
+      return fail(r, msg);
+    }
   }
   if (nb > 0)
     MX_CUDA(cudaMemcpyAsync(s->d_grow + S.boff, gr.data(), nb * sizeof(mx::Growth),
