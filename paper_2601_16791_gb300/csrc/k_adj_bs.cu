@@ -177,7 +177,7 @@ __global__ void __launch_bounds__(32) k_adj_bs_fwd(Dev d, Adj a) {
     if (off + (unsigned long long)kAdjMaxSteps * stride > a.tape_cap) {
       if (lane == 0) {
         a.g_M[g] = -1;
-        atomicOr(d.status, ST_WORK_OVF);
+        report(d.status, ST_WORK_OVF);
       }
       continue;
     }
@@ -260,7 +260,7 @@ __global__ void __launch_bounds__(32) k_adj_bs_fwd(Dev d, Adj a) {
     }
     if (lane == 0) {
       if (!ok) {
-        atomicOr(d.status, M >= kAdjMaxSteps ? ST_TAPE : ST_BS);
+        report(d.status, M >= kAdjMaxSteps ? ST_TAPE : ST_BS);
         a.g_M[g] = -1;
       } else {
         a.g_M[g] = M;
@@ -302,7 +302,7 @@ __global__ void __launch_bounds__(128) k_adj_bs_fwd2(Dev d, Adj a) {
     if (off + (unsigned long long)kAdjMaxSteps * stride > a.tape_cap) {
       if (threadIdx.x == 0) {
         a.g_M[g] = -1;
-        atomicOr(d.status, ST_WORK_OVF);
+        report(d.status, ST_WORK_OVF);
       }
       continue;
     }
@@ -413,7 +413,7 @@ __global__ void __launch_bounds__(128) k_adj_bs_fwd2(Dev d, Adj a) {
     }
     if (c == 0 && lane == 0) {
       if (!ok) {
-        atomicOr(d.status, M >= kAdjMaxSteps ? ST_TAPE : ST_BS);
+        report(d.status, M >= kAdjMaxSteps ? ST_TAPE : ST_BS);
         a.g_M[g] = -1;
       } else {
         a.g_M[g] = M;
@@ -834,7 +834,7 @@ __global__ void __launch_bounds__(kThreads) k_adj_share_keys(Dev d, Adj a) {
     const int e0 = atomicAdd(a.scount, wf);
     for (int m = 0; m < wf; ++m) {
       if (e0 + m >= a.skeys_cap) {
-        atomicOr(d.status, ST_WORK_OVF);
+        report(d.status, ST_WORK_OVF);
         break;
       }
       a.skeys[e0 + m] = ((unsigned long long)d.work_mem[o + m] << 32) |

@@ -435,7 +435,7 @@ __global__ void __launch_bounds__(kThreads) k_adj_move_fwd(Dev d, Adj a, int sta
     }
     double u = a.v1[j], v = a.v1[(size_t)N + j], w = a.v1[2 * (size_t)N + j];
     if (!kepler_drift_sel(S.split, S.mu0, S.h, d.kepler_max_iter, x, y, z, u, v, w))
-      atomicOr(d.status, ST_KEPLER);
+      report(d.status, ST_KEPLER);
     a.xv3[j] = x; a.xv3[(size_t)N + j] = y; a.xv3[2 * (size_t)N + j] = z;
     a.xv3[3 * (size_t)N + j] = u; a.xv3[4 * (size_t)N + j] = v; a.xv3[5 * (size_t)N + j] = w;
   } else {
@@ -809,7 +809,7 @@ __global__ void __launch_bounds__(kThreads) k_adj_drift_vjp(Dev d, Adj a) {
       m1[c] = a.lam[(size_t)(3 + c) * N + j];
     }
     if (!kepler_vjp(S.mu0, S.h, d.kepler_max_iter, x, v, l1, m1, l0, m0))
-      atomicOr(d.status, ST_KEPLER);
+      report(d.status, ST_KEPLER);
     for (int c = 0; c < 3; ++c) {
       a.lam[(size_t)c * N + j] = l0[c];
       a.lam[(size_t)(3 + c) * N + j] = m0[c];

@@ -157,7 +157,7 @@ __device__ __forceinline__ void groups_block(const Dev& d) {
   __shared__ unsigned long long skeys[kGroupKeysSmem];
   const int count = *d.pair_count;
   if (count > d.pair_cap) {
-    if (threadIdx.x == 0) atomicOr(d.status, ST_PAIR_OVF);
+    if (threadIdx.x == 0) report(d.status, ST_PAIR_OVF);
     return;
   }
   const int n = count;
@@ -181,7 +181,7 @@ __device__ __forceinline__ void groups_block(const Dev& d) {
   __syncthreads();
   const int nbb = s_nbb;
   if (nbb > kMaxBigPairs) {
-    if (threadIdx.x == 0) atomicOr(d.status, ST_GROUP);
+    if (threadIdx.x == 0) report(d.status, ST_GROUP);
     return;
   }
   // ---- big groups: the connected components of the (few) big-big pairs.
@@ -298,7 +298,7 @@ __device__ __forceinline__ void groups_block(const Dev& d) {
   }
   __syncthreads();
   if (s_bad) {
-    if (threadIdx.x == 0) atomicOr(d.status, (unsigned)s_bad);
+    if (threadIdx.x == 0) report(d.status, (unsigned)s_bad);
     return;
   }
   // ---- test-particle groups: one per run of pairs with the same small body
@@ -339,7 +339,7 @@ __device__ __forceinline__ void groups_block(const Dev& d) {
   }
   if (threadIdx.x == 0) {
     if (s_bad) {
-      atomicOr(d.status, (unsigned)s_bad);
+      report(d.status, (unsigned)s_bad);
       *d.work_count = 0;
     } else {
       const int W = min(s_bw, d.work_cap);
@@ -732,7 +732,7 @@ __device__ __forceinline__ bool mail_wait_word(const ClusterMail& mb, volatile i
     int ok = 1;
     while (*w < v) {   // a shared-memory word: a poll costs tens of cycles
       if (++k > kMailSpin) {
-        atomicOr(mb.status, ST_BARRIER);
+        report(mb.status, ST_BARRIER);
         ok = 0;
         break;
       }
@@ -918,7 +918,7 @@ __device__ void pack_tail(const Dev& d, int w, unsigned gmask, int base, int lan
                           GroupRun<NB>& g, Finish&& finish_here) {
   if (r != 0) {
     if (lane == base) {
-      if (r < 0) atomicOr(d.status, ST_BS);
+      if (r < 0) report(d.status, ST_BS);
       d.work_nsub[w] = g.nsub;
     }
     write_members<NB>(d, w, o0, lane - base, g);
@@ -968,7 +968,7 @@ __device__ void pack_tail(const Dev& d, int w, unsigned gmask, int base, int lan
     const int r2 = finish_here(g);
     if (r2 == 2) return;   // the caller finishes the group itself
     if (lane == base) {
-      if (r2 < 0) atomicOr(d.status, ST_BS);
+      if (r2 < 0) report(d.status, ST_BS);
       d.work_nsub[w] = g.nsub;
     }
     write_members<NB>(d, w, o0, lane - base, g);
@@ -1253,7 +1253,7 @@ __device__ void pack_two_pair(const Dev& d, int a, int b, int lane) {
     gf.nsub = __shfl_sync(0xffffffffu, g.nsub, h);
     const int r2 = bs2_rounds<1>(0, lane, tf, d.bs_tol, d.bs_max_sub, 1 << 30, gf, nullptr, nullptr);
     if (lane == 0) {
-      if (r2 < 0) atomicOr(d.status, ST_BS);
+      if (r2 < 0) report(d.status, ST_BS);
       d.work_nsub[wf] = gf.nsub;
     }
     write_members<2>(d, wf, of, lane, gf);
@@ -1304,7 +1304,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(128) k_bs_spread2(De
       const int r = bs2c_rounds(wq, lane, t, d.bs_tol, d.bs_max_sub, 1 << 30, g, sm, nullptr, &mail);
       if (cta == 0 && wq == 0) {
         if (lane == 0) {
-          if (r < 0) atomicOr(d.status, ST_BS);
+          if (r < 0) report(d.status, ST_BS);
           d.work_nsub[w] = g.nsub;
         }
         write_members<2>(d, w, o0, lane, g);
@@ -1333,7 +1333,7 @@ __device__ __noinline__ void thread_group(const Dev& d, int w) {
     for (int c = 0; c < 6; ++c) Y[c][m] = d.xv0[(size_t)c * N + g];
   }
   int nsub = 0;
-  if (!bs_integrate(G, S.mu0, S.h, d.bs_tol, d.bs_max_sub, Y, &nsub)) atomicOr(d.status, ST_BS);
+  if (!bs_integrate(G, S.mu0, S.h, d.bs_tol, d.bs_max_sub, Y, &nsub)) report(d.status, ST_BS);
   d.work_nsub[w] = nsub;
   for (int m = d.work_wfrom[w]; m < nb; ++m) {
     const int g = d.work_mem[o0 + m];
@@ -1531,7 +1531,7 @@ __device__ __noinline__ void catch_bs_thread(const Dev& d, const SysDev& S, cons
     for (int q = 0; q < 6; ++q) Y[q][m] = big ? B0[(size_t)q * NBs + mem[m]] : a0[q];
   }
   int nsub = 0;
-  if (!bs_integrate(G, S.mu0, S.h, d.bs_tol, d.bs_max_sub, Y, &nsub)) atomicOr(d.status, ST_BS);
+  if (!bs_integrate(G, S.mu0, S.h, d.bs_tol, d.bs_max_sub, Y, &nsub)) report(d.status, ST_BS);
   for (int q = 0; q < 6; ++q) out[q] = Y[q][nb - 1];
 }
 
@@ -1569,7 +1569,7 @@ __device__ int catch_front(const Dev& d, const SysDev& S, int sys, int j, int t,
   } else {
     drifted = kepler_drift(S.mu0, S.h, d.kepler_max_iter, x, y, z, u, v, w);
   }
-  if (!drifted && wr && lane == 0) atomicOr(d.status, ST_KEPLER);
+  if (!drifted && wr && lane == 0) report(d.status, ST_KEPLER);
   const double a1[6] = {x, y, z, u, v, w};
   float af[12];
   for (int k = 0; k < 6; ++k) {
@@ -1660,7 +1660,7 @@ __device__ int catch_front(const Dev& d, const SysDev& S, int sys, int j, int t,
     }
   }
   if (bad) {   // the direct path skips the step's Bulirsch-Stoer and reports it
-    if (wr && lane == 0) atomicOr(d.status, ST_GROUP);
+    if (wr && lane == 0) report(d.status, ST_GROUP);
     return 0;
   }
   const int nb = cnt + 1;
@@ -1840,7 +1840,7 @@ __device__ void catch_back(const Dev& d, const SysDev& S, int sys, int j, int t,
   }
   if (!(finite_d(x) && finite_d(y) && finite_d(z) && finite_d(u) && finite_d(v) && finite_d(w)) &&
       lead)
-    atomicOr(d.status, ST_NONFINITE);
+    report(d.status, ST_NONFINITE);
   if (!head) {
     s6[0] = x;
     s6[1] = y;
@@ -1926,7 +1926,7 @@ __device__ void catch_record(const Dev& d, const CatchArgs& a, int bank, int idx
         carried = true;
         break;
       }
-      if (r < 0 && lead) atomicOr(d.status, ST_BS);
+      if (r < 0 && lead) report(d.status, ST_BS);
       G.nb = 0;
       catch_back(d, S, sys, j, t, lead, s6, B.ops);
       ejected = eject_after(t);
@@ -1973,7 +1973,7 @@ __device__ void catch_record(const Dev& d, const CatchArgs& a, int bank, int idx
   const int oi = s_slot;
   __syncthreads();
   if (!lead || oi >= d.dcap) {
-    if (lead && oi >= d.dcap) atomicOr(d.status, ST_WORK_OVF);
+    if (lead && oi >= d.dcap) report(d.status, ST_WORK_OVF);
     return;
   }
   int* O = rec_ints(d, ob, oi);
@@ -2062,7 +2062,7 @@ __device__ bool grid_sync(unsigned* bar, long long spin, unsigned* status) {
             break;
           }
           if (++k > spin) {
-            atomicOr(status, ST_BARRIER);
+            report(status, ST_BARRIER);
             atomicExch(bar + 2, 1u);
             ok = 0;
             break;

@@ -30,7 +30,7 @@ __global__ void __launch_bounds__(kThreads) k_drift_buf(double* xv, int n, doubl
   if (j >= n) return;
   double x = xv[j], y = xv[(size_t)n + j], z = xv[2 * (size_t)n + j];
   double u = xv[3 * (size_t)n + j], v = xv[4 * (size_t)n + j], w = xv[5 * (size_t)n + j];
-  if (!kepler_drift_sel(true, mu, h, maxit, x, y, z, u, v, w)) atomicOr(status, ST_KEPLER);
+  if (!kepler_drift_sel(true, mu, h, maxit, x, y, z, u, v, w)) report(status, ST_KEPLER);
   xv[j] = x;
   xv[(size_t)n + j] = y;
   xv[2 * (size_t)n + j] = z;

@@ -49,6 +49,13 @@ enum : unsigned {
   ST_WINDOW = 1u << 8
 };
 
+// A failure into the status word, which lies in host memory: in system scope,
+// since the host takes and clears the word (sync_status) while a catch-up may
+// still run on the side stream.
+__device__ __forceinline__ void report(unsigned* status, unsigned bits) {
+  atomicOr_system(status, bits);
+}
+
 // Constants of one system.
 struct SysDev {
   int off;        // global index of the system's first body

@@ -143,7 +143,7 @@ __device__ __forceinline__ void detect_tile(const Dev& d, const double* xv0, con
         d.ever[j] = 1;
       }
       if (nh == kMaxGroup) {   // a run split in two: only past the group limit
-        if (runs) atomicOr(d.status, ST_GROUP);
+        if (runs) report(d.status, ST_GROUP);
         nh = -1;               // marks the flush below as due
       } else {
         hits[nh++] = il;

@@ -56,7 +56,7 @@ __device__ __forceinline__ void jump_drift_tile(const Dev& d, double jump_frac, 
   d.xv0[4 * (size_t)N + j] = v;
   d.xv0[5 * (size_t)N + j] = w;
   if (!kepler_drift_sel(S.split, S.mu0, S.h, d.kepler_max_iter, x, y, z, u, v, w))
-    atomicOr(d.status, ST_KEPLER);
+    report(d.status, ST_KEPLER);
   d.xv[j] = x;
   d.xv[(size_t)N + j] = y;
   d.xv[2 * (size_t)N + j] = z;

@@ -612,7 +612,7 @@ __device__ __forceinline__ void jump_kick_tile(const Dev& d, double jump_frac, d
     d.xv[5 * (size_t)N + j] = w;
   }
   if (!(finite_d(x) && finite_d(y) && finite_d(z) && finite_d(u) && finite_d(v) && finite_d(w)))
-    atomicOr(d.status, ST_NONFINITE);
+    report(d.status, ST_NONFINITE);
 }
 
 // Dynamic shared memory of a kick: the big bodies' staging (and their FP32
