@@ -1759,8 +1759,8 @@ static __device__ __noinline__ void catch_kick_light(const Dev& d, const SysDev&
     ax += dc.adg[0];
     ay += dc.adg[1];
   }
-  split_kicks(S, kick_h, nk, split_gravity(acc, ax, ay, az), S.gas_on != 0, dc, x, y, hp0, hp1, hp2,
-              rp, kd, u, v, w, [](int) { return -1; }, [](int, int) {});
+  split_kicks(S, kick_h, nk, acc, ax, ay, az, S.gas_on != 0, dc, x, y, hp0, hp1, hp2, rp, kd, u, v,
+              w, [](int) { return -1; }, [](int, int) {});
   q[3] = u;
   q[4] = v;
   q[5] = w;

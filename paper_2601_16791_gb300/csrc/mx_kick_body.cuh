@@ -558,7 +558,6 @@ __device__ __forceinline__ void jump_kick_tile(const Dev& d, double jump_frac, d
       ax += dc.adg[0];   // disk gravity: fixed over the launch, like the big bodies'
       ay += dc.adg[1];
     }
-    const SplitGrav g = split_gravity(acc, ax, ay, az);
     auto word = [&](int kk) { return (size_t)(kbase + kk) * d.kwords + (j >> 5); };
     auto branch = [&](int kk) {
       return (d.kmode == 2 && kbase + kk < d.kcap) ? (int)((d.kbits[word(kk)] >> (j & 31)) & 1u) : -1;
@@ -566,8 +565,8 @@ __device__ __forceinline__ void jump_kick_tile(const Dev& d, double jump_frac, d
     auto keep = [&](int kk, int kb) {
       if (d.kmode == 1 && kb && kbase + kk < d.kcap) atomicOr(&d.kbits[word(kk)], 1u << (j & 31));
     };
-    split_kicks(S, kick_h, NKICK, g, drag, dc, x, y, hp0, hp1, hp2, rp, kd, u, v, w, branch,
-                keep);
+    split_kicks(S, kick_h, NKICK, acc, ax, ay, az, drag, dc, x, y, hp0, hp1, hp2, rp, kd, u, v, w,
+                branch, keep);
   } else {
     // the gas at the (fixed) position, shared by the launch's half kicks
     GasAt gq = drag ? gas_at(S, x, y) : GasAt{false, 0.0, 0.0, 0.0};

@@ -8,16 +8,18 @@
 // same pair in pairs of FP32 numbers (a value kept as hi + lo, 48 bits) takes
 // about 115 instructions.
 //
-// What the precision is: the state, the jump and the velocity update stay
-// FP64; only a far pair's acceleration mu d/s^3 is formed in FP32 pairs, with
-// a relative error of about 1.5e-14 (rms, against 80-bit arithmetic).  A half
-// kick adds (h/2) a to a velocity; outside the changeover shell (3 Hill radii)
-// that is at most a few 1e-4 of the velocity, so the split's share of
-// the new velocity's error is below 1e-17 of it, where the FP64 rounding of
-// the velocity itself is 1e-16.  A pair inside the shell, where the
-// acceleration is largest and K varies, goes through the FP64 pair_acc, and
-// so does a target outside the positions' grid below.  mx_accel, which returns
-// accelerations, does not use it.
+// What the precision is: the state, the jump, the impulse h a and its addition
+// to the velocity stay FP64.  In FP32 pairs are a far pair's acceleration
+// mu d/s^3, with a relative error of about 1.5e-14 (rms, against 80-bit
+// arithmetic; mu itself is held to 48 bits), and the sum of the far pairs, or
+// of kSplitSeg of them.  A half kick adds (h/2) a to a velocity; outside the
+// changeover shell (3 Hill radii) that is at most a few 1e-4 of the velocity,
+// so the split's share of the new velocity's error is below 1e-17 of it, where
+// the FP64 rounding of the velocity itself is 1e-16.  A pair inside the shell,
+// where the acceleration is largest and K varies, goes through the FP64
+// pair_acc and is added in FP64, and so is every pair of a target outside the
+// positions' grid below.  mx_accel, which returns accelerations, takes three
+// FP32 parts instead (below).
 //
 // Measured: k_jump_kick with 2,000 big bodies and 200,000 planetesimals 11.8 ->
 // 1.65 ms a launch (34 -> 245 G pairs/s); 301 big bodies and 20,011

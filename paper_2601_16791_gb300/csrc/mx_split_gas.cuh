@@ -4,14 +4,16 @@
 // masses are fixed: no gaps in the gas).
 //
 // What stays FP64: the state, the gas velocity at the body (g) and so the
-// relative velocity dv, which is a small difference of large velocities.
-// Formed in FP32 pairs (about 45 bits): rho_g, 1/c_s, |dv|, Re, Ma, C_D and
-// the impulse h (a_grav - coef dv), which then enters the velocity with one
-// FP64 rounding.  The drag changes a velocity by h/t_stop times dv, below
-// 1e-3 of it for an explicit kick to make sense, so 45 bits of it are finer
-// than the velocity's own last place.  mx_gas_drag and mx_accel, which return
-// the drag itself, keep FP64 (mx_physics.cuh), and so does a body whose Re, Ma
-// or |dv| leave the range FP32 holds with room (drag_coef_fp64).
+// relative velocity dv, which is a small difference of large velocities; the
+// pairs inside a changeover shell and the disk's gravity; the impulse h times
+// the sum of all accelerations, and its addition to the velocity.
+// Held in FP32 pairs (about 45 bits): the far pairs' sum (mx_split.cuh), rho_g,
+// 1/c_s, |dv|, Re, Ma, C_D and the drag coef dv.  45 bits are 2.8e-14 of the
+// drag, so its share of the velocity's error is 2.8e-14 h/t_stop |dv|: with
+// h/t_stop up to 2^-6 and |dv| up to a tenth of the velocity, 4e-17 of it,
+// below half a unit of its last place.  A body with a larger h/t_stop, or whose
+// Re, Ma or |dv| leaves the range FP32 holds with room, keeps the FP64 drag
+// (drag_fp64), as mx_gas_drag and mx_accel, which return the drag itself, do.
 #pragma once
 #include "mx_physics.cuh"
 #include "mx_split.cuh"
@@ -63,22 +65,22 @@ __device__ __forceinline__ DragSplit drag_split(const SysDev& S, double x, doubl
   return c;
 }
 
-// The FP64 coefficient of the same body (gas_at, drag_const, gas_drag_coef).
-static __device__ __noinline__ double drag_coef_fp64(const SysDev& S, double x, double y, double hp0,
-                                                     double hp1, double hp2, double rp_cm, double kd,
-                                                     double u, double v, double w, int kb_in,
-                                                     int* kb_out) {
+// The FP64 drag of the same body (gas_at, drag_const, gas_drag_coef): coef dv.
+static __device__ __noinline__ void drag_fp64(const SysDev& S, double x, double y, double hp0,
+                                              double hp1, double hp2, double rp_cm, double kd,
+                                              double u, double v, double w, double* a, int kb_in,
+                                              int* kb_out) {
   const GasAt q = gas_at(S, x, y);
-  double dvec[3];
-  return gas_drag_coef(S, drag_const(S, q, x, y, hp0, hp1, hp2, rp_cm, kd), u, v, w, dvec, kb_in,
-                       kb_out);
+  const double coef = gas_drag_coef(S, drag_const(S, q, x, y, hp0, hp1, hp2, rp_cm, kd), u, v, w, a,
+                                    kb_in, kb_out);
+  for (int c = 0; c < 3; ++c) a[c] *= coef;
 }
 
-// gas_drag_coef in pairs (Eqs. 3, 7): coef of -coef dv, dv written to d[3];
-// false where the values leave the range above (nothing else written).
-__device__ __forceinline__ bool drag_coef_split(const SysDev& S, const DragSplit& c, double u,
-                                                double v, double w, FF (&d)[3], FF& coef, int kb_in,
-                                                int* kb_out) {
+// gas_drag_coef in pairs (Eqs. 3, 7) for a half kick of h: coef of -coef dv, dv
+// written to d[3]; false where the values leave the range above.
+__device__ __forceinline__ bool drag_coef_split(const SysDev& S, const DragSplit& c, float h,
+                                                double u, double v, double w, FF (&d)[3], FF& coef,
+                                                int kb_in, int* kb_out) {
   d[0] = ff_of(u + c.offu);
   d[1] = ff_of(v + c.offv);
   d[2] = ff_of(w + c.offw);
@@ -104,62 +106,53 @@ __device__ __forceinline__ bool drag_coef_split(const SysDev& S, const DragSplit
     cd = ff_mul(ff_add(ff_mul(t2, den1), ff_mul(D, A)), r);
   }
   coef = ff_mul(ff_mul(cd, c.coef_k), dm);
-  return true;
+  return fabsf(h * coef.h) <= 0x1p-6f;
 }
 
-// u - h (acc + coef dv): acc the gravity with its sign reversed.
-__device__ __forceinline__ double kick_split(FF h, FF acc, FF coef, FF dv, double u) {
-  const FF p = ff_mul(h, ff_add(acc, ff_mul(coef, dv)));
-  return u - (bits_to_double(p.h) + bits_to_double(p.l));
-}
-__device__ __forceinline__ double kick_split(FF h, FF acc, double u) {
-  const FF p = ff_mul(h, acc);
-  return u - (bits_to_double(p.h) + bits_to_double(p.l));
+// u - h (t - a): t the accelerations held in pairs (sign reversed), a the FP64
+// ones.  The impulse is one FP64 product, added with one rounding.
+__device__ __forceinline__ double kick_split(double h, FF t, double a, double u) {
+  double s = bits_to_double(t.h) + bits_to_double(t.l);
+  if (__double_as_longlong(a) != 0) s -= a;   // zero for most bodies
+  return fma(-h, s, u);
 }
 
-// A body's gravity, sign reversed, from the far pairs' sum and the FP64 one
-// (pairs inside a changeover shell, disk gravity; zero for most bodies).
-struct SplitGrav {
-  FF x, y, z;
-};
-
-__device__ __forceinline__ SplitGrav split_gravity(const SplitAcc& acc, double ax, double ay,
-                                                   double az) {
-  SplitGrav g{{acc.xh, acc.xl}, {acc.yh, acc.yl}, {acc.zh, acc.zl}};
-  if (__double_as_longlong(ax) != 0 || __double_as_longlong(ay) != 0 || __double_as_longlong(az) != 0) {
-    g.x = ff_add(g.x, ff_neg(ff_of(ax)));
-    g.y = ff_add(g.y, ff_neg(ff_of(ay)));
-    g.z = ff_add(g.z, ff_neg(ff_of(az)));
-  }
-  return g;
-}
-
-// The half kicks of one body (nkick of h each) with the gravity g and, with drag, the gas at (x, y).  kick_branch(kk) gives the k
-// branch of Eq. 7 to take (-1: from Re), keep(kk, kb) receives the one taken.
+// The half kicks of one body (nkick of h each): the far pairs' sum acc (sign
+// reversed), the FP64 acceleration (ax, ay, az; pairs inside a changeover
+// shell, disk gravity) and, with drag, the gas at (x, y).  branch(kk) gives the
+// k branch of Eq. 7 to take (-1: from Re), keep(kk, kb) receives the one taken.
 template <class In, class Out>
-__device__ __forceinline__ void split_kicks(const SysDev& S, double kick_h, int nkick,
-                                            const SplitGrav& g, bool drag, const DragSplit& dc,
-                                            double x, double y, double hp0, double hp1, double hp2,
-                                            double rp, double kd, double& u, double& v, double& w,
+__device__ __forceinline__ void split_kicks(const SysDev& S, double h, int nkick,
+                                            const SplitAcc& acc, double ax, double ay, double az,
+                                            bool drag, const DragSplit& dc, double x, double y,
+                                            double hp0, double hp1, double hp2, double rp,
+                                            double kd, double& u, double& v, double& w,
                                             In&& branch, Out&& keep) {
-  const FF h = ff_of(kick_h);
+  const FF gx{acc.xh, acc.xl}, gy{acc.yh, acc.yl}, gz{acc.zh, acc.zl};
 #pragma unroll 1
   for (int kk = 0; kk < nkick; ++kk) {
-    FF d[3] = {}, coef{0.0f, 0.0f};
+    FF tx = gx, ty = gy, tz = gz;
+    double bx = ax, by = ay, bz = az;
     if (drag && dc.in_gas) {
       const int kin = branch(kk);
       int kout = 0;
-      if (!drag_coef_split(S, dc, u, v, w, d, coef, kin, &kout))
-        coef = ff_of(drag_coef_fp64(S, x, y, hp0, hp1, hp2, rp, kd, u, v, w, kin, &kout));
+      FF d[3], coef;
+      if (drag_coef_split(S, dc, ff_of(h).h, u, v, w, d, coef, kin, &kout)) {
+        tx = ff_add(tx, ff_mul(coef, d[0]));
+        ty = ff_add(ty, ff_mul(coef, d[1]));
+        tz = ff_add(tz, ff_mul(coef, d[2]));
+      } else {
+        double a[3];
+        drag_fp64(S, x, y, hp0, hp1, hp2, rp, kd, u, v, w, a, kin, &kout);
+        bx -= a[0];
+        by -= a[1];
+        bz -= a[2];
+      }
       keep(kk, kout);
-      u = kick_split(h, g.x, coef, d[0], u);
-      v = kick_split(h, g.y, coef, d[1], v);
-      w = kick_split(h, g.z, coef, d[2], w);
-    } else {
-      u = kick_split(h, g.x, u);
-      v = kick_split(h, g.y, v);
-      w = kick_split(h, g.z, w);
     }
+    u = kick_split(h, tx, bx, u);
+    v = kick_split(h, ty, by, v);
+    w = kick_split(h, tz, bz, w);
   }
 }
 
