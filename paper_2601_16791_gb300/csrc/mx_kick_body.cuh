@@ -94,7 +94,7 @@ __device__ __forceinline__ SplitBig split_big(double x, double y, double z, doub
   b.muh = m.h;
   b.mul = m.l;
   // a mass off FP32's range: no pair of it is a far one
-  b.near2 = split_mass(mu) ? near2_of(rc2) : __int_as_float(0x7f800000);
+  b.near2 = split_mass(mu) ? split_near2(rc2, kg) : __int_as_float(0x7f800000);
   return b;
 }
 

@@ -29,10 +29,14 @@
 //
 // Positions: each coordinate is cut on one grid for target and sources into
 // three FP32 parts, x = x0 + x1 + x2 with x0 a multiple of 2^(k-23), x1 of
-// 2^(k-47), |x| < 2^k, so that the differences of the parts are exact and a
-// separation keeps the bits of the FP64 positions however close the pair.
+// 2^(k-47) and x2 the rest, |x| < 2^k, so that the differences of the first two
+// parts are exact.  x2 and its difference round at 2^(k-73) and 2^(k-72): a
+// separation is off by at most 2^(k-71), and pairs closer than 2^(k-17) go
+// through FP64 (split_near2), so the others' separations keep 54 bits.
 // k comes from the positions of the chunk's big bodies (never from the tile),
-// so results do not depend on the tiling.
+// so results do not depend on the tiling.  A body 300 AU out (k = 10) sends the
+// pairs within 0.008 AU to FP64; the changeover shell of a lunar embryo at
+// 0.5 AU has 0.0035 AU.
 #pragma once
 #include <limits.h>
 #include "mx_common.cuh"
@@ -46,19 +50,20 @@ constexpr int kSplitMaxK = 10;    // else the pair sum stays FP64 (FP32 range of
 
 __device__ __forceinline__ float pow2f(int e) { return __int_as_float((e + 127) << 23); }
 
-// x = o[0] + o[1] + o[2] on the grid of 2^k (|x| < 2^k); bits of x below
-// 2^(k-62) are rounded off.  Integer instructions only.
+// x = o0 + o1 + o2 on the grid of 2^k (|x| < 2^k).  Integer instructions but
+// for the conversions.
 __device__ __forceinline__ void split3(double x, int k, float& o0, float& o1, float& o2) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
   const int e = (int)(b >> 52) & 0x7ff;
   const unsigned long long m = (b & 0xfffffffffffffull) | 0x10000000000000ull;
-  // x = m 2^(e-1075); v = x / 2^(k-62)
+  // |x| = m 2^(e-1075) = v 2^(k-62) + rem 2^(e-1075)
   const int sh = (k - 62) - (e - 1075);
   unsigned long long v;
   if (sh <= 0) v = m << min(-sh, 63);
   else if (sh < 54) v = (m + (1ull << (sh - 1))) >> sh;
   else v = 0;
-  const long long s = (b >> 63) ? -(long long)v : (long long)v;
+  const bool neg = (b >> 63) != 0;
+  const long long s = neg ? -(long long)v : (long long)v;
   const long long a = (s + (1ll << 38)) >> 39;           // multiples of 2^(k-23)
   const long long r = s - (a << 39);                     // |r| <= 2^38
   const long long c = (r + (1ll << 14)) >> 15;           // multiples of 2^(k-47)
@@ -66,6 +71,12 @@ __device__ __forceinline__ void split3(double x, int k, float& o0, float& o1, fl
   o0 = __int2float_rn((int)a) * pow2f(k - 23);
   o1 = __int2float_rn((int)c) * pow2f(k - 47);
   o2 = __int2float_rn(q) * pow2f(k - 62);
+  if (sh > 0 && e >= 885) {   // below 2^-138 AU nothing is left to keep
+    const long long rem = (long long)m - (long long)(sh < 54 ? v << sh : 0);
+    // in two factors: 2^(e-1075) itself may be below FP32's range
+    const float f = __ll2float_rn(neg ? -rem : rem) * 0x1p-64f * pow2f(max(e - 1075 + 64, -126));
+    o2 = __fadd_rn(o2, f);
+  }
 }
 
 // The grid's k for bodies whose largest coordinate has the high word `hi`
@@ -196,9 +207,15 @@ struct SplitAcc {
   float xh, xl, yh, yl, zh, zl;
 };
 
-// At least (1e-6 AU)^2: mu/s^3 and the reverse's mu/s^5 stay in FP32's range.
+// At least (1e-6 AU)^2: mu/s^3 stays in FP32's range.
 __device__ __forceinline__ float near2_of(double rc2) {
   return fmaxf(to_float_bits(rc2) * 1.0001f, 1e-12f);
+}
+
+// A source's near2 on the grid of 2^k: its shell, and the pairs whose
+// separation the grid does not hold to 54 bits (the positions, above).
+__device__ __forceinline__ float split_near2(double rc2, int k) {
+  return fmaxf(near2_of(rc2), pow2f(2 * (k - 17)));
 }
 
 // Whether the products of mu with powers of a far pair's 1/s keep their parts
@@ -289,7 +306,8 @@ __device__ __forceinline__ void split_flush(SplitAcc& acc, double& ax, double& a
 // ----------------------------------------------- a far pair in three FP32 parts
 // The same sum for mx_accel, which returns the acceleration itself: every
 // quantity carries a third FP32 part, so that a pair's relative error is 8e-20
-// (rms, against 80-bit arithmetic; FP64's is 1.3e-16) and what is left of the
+// (rms, against 80-bit arithmetic; FP64's is 1.3e-16) where the grid holds the
+// whole separation, 2^-54 of it by coordinate at the least; what is left of the
 // sum's is its FP64 adds, one in kSplitSeg.  About 340 FP32 instructions a pair
 // against pair_acc's 17 of 64 cycles.  Measured: k_accel with 2,000 big bodies
 // and 200,000 planetesimals 11.8 -> 4.57 ms (87% of the issue slots filled), and the

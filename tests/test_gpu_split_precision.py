@@ -138,3 +138,33 @@ def test_strong_drag_stays_fp64():
     assert (err / bound)[:, strong].max() <= 1.0, (err / bound)[:, strong].max()
     bound = bound + 2.8e-14 * imp
     assert (err / bound)[:, weak].max() <= 1.0, (err / bound)[:, weak].max()
+
+
+@pytest.mark.parametrize("far", [4.0, 40.0, 300.0, 480.0])
+def test_accel_with_a_distant_big_body(far):
+    """The distant body sets the grid of the positions; planetesimals just
+    outside the shells of the embryos near 0.5 AU are where it is coarsest.
+    Bound: the separation's 2^-54 by coordinate make 3.5 U of a pair, FP64's
+    own pair about 10 U (the close ones), two or three roundings of the sums:
+    12 U of the pairs' magnitudes."""
+    w = embryos(20, 600)
+    nb = w.nbig
+    xb = w.xv_helio[:, :nb]
+    r = np.linalg.norm(xb[:3], axis=0)
+    to = np.full(nb, 0.5)
+    to[-1] = far
+    xb[:3] *= to / r                    # the same orbits at other sizes
+    xb[3:] /= np.sqrt(to / r)
+    rng = np.random.default_rng(4)
+    p = orc.make_params(w.params)
+    _, _, rc = orc.init(p, nb, w.nsmall, w.m_big, w.xv_helio)
+    b = rng.integers(nb - 1, size=w.nsmall)
+    d = rng.normal(size=(3, w.nsmall))
+    w.xv_helio[:3, nb:] = xb[:3, b] + d / np.linalg.norm(d, axis=0) * rc[b] * rng.uniform(1.001, 1.5, w.nsmall)
+    start, acc, _, _ = half_kick(w)
+    x = start[:3]
+    err = np.sqrt(((acc - gravity(w, x)) ** 2).sum(0)).astype(np.float64)
+    s2 = ((x[:, :, None] - x[:, None, :nb]) ** 2).sum(0)
+    s2[s2 == 0] = np.inf
+    size = (W.G * w.m_big / s2).sum(1)
+    assert (err / size).max() <= 12 * U, (err / size).max() / U
