@@ -23,7 +23,8 @@ joins that of the previous step's last half kick, at the same positions.  The
 recomputation (mx_adjoint_recompute) keeps each step's pre-drift state, so the
 adjoint does not recompute the first half kick (mx_adjoint_step_predrift), and
 leaves out the encounter groups the adjoint skips: their bodies' states carry
-no derivative.
+no derivative.  The backward leaves the system in the run's own state at the end
+of its first segment, with every group integrated.
 
 Inputs: the initial heliocentric state (6 x N float64 CUDA tensor) and the
 gas parameters (sigma1 [g/cm^2], gamma, cd_scale) as a 3-vector.
@@ -92,6 +93,15 @@ class SemimajorLoss(torch.autograd.Function):
         w_eff = w * (1.0 - ever.to(torch.float64)) if mask_encounters else w
         # masked: the groups of big bodies only, and none when no big bodies met
         ctx.groups = (2 if nbb > 0 else 0) if mask_encounters else 1
+        # the run's state at the first segment's end, where the recomputation of
+        # the reverse sweep ends without the bodies of the groups it skips
+        ctx.after = None
+        if ctx.groups != 1 and ckpts:
+            if len(ckpts) == 1:
+                ctx.after = torch.empty((6, traj.n), dtype=torch.float64, device="cuda")
+                mx.mx_get_state_device(traj.h, ctx.after)
+            else:
+                ctx.after = ckpts[1][1]
         L, seed_f, seed_i = traj.loss(xv_helio0, w_eff)
         ctx.traj, ctx.nsteps, ctx.every, ctx.nbb = traj, nsteps, every, nbb
         ctx.ckpts = ckpts
@@ -125,6 +135,8 @@ class SemimajorLoss(torch.autograd.Function):
         grad0 = torch.empty((6, traj.n), dtype=torch.float64, device="cuda")
         mx.mx_adjoint_init(h, lam, grad0)
         mx.mx_adjoint_merge(h, False)
+        if ctx.after is not None:
+            mx.mx_set_state_device(h, ctx.after)
         grad0 += g * seed_i
         return grad0, dpar, None, None, None, None, None
 
