@@ -28,6 +28,7 @@ import hashlib
 import json
 import math
 import os
+import re
 import statistics
 import subprocess
 import sys
@@ -262,15 +263,21 @@ def source_hash(names):
     return h.hexdigest()[:16]
 
 
-KERNEL_SOURCES = {"k_jump_kick": ["k_kick.cu", "mx_kick_body.cuh", "mx_common.cuh", "mx_physics.cuh",
-                                  "mx_growth.cuh", "mx_split.cuh", "mx_split_gas.cuh"],
-                  "k_jump_drift": ["k_drift.cu", "mx_drift_body.cuh", "mx_common.cuh", "mx_kepler.cuh",
-                                   "mx_kepler_short.cuh"],
-                  "k_detect": ["k_detect.cu", "mx_detect_body.cuh", "mx_common.cuh",
-                               "mx_encounter.cuh"],
-                  "k_bs": ["k_bs.cu", "mx_bs.cuh", "mx_bs2.cuh", "mx_common.cuh", "mx_physics.cuh"],
-                  "k_catchup": ["k_bs.cu", "mx_bs.cuh", "mx_common.cuh", "mx_physics.cuh",
-                                "mx_kepler.cuh", "mx_encounter.cuh"]}
+def unit_sources(unit):
+    """A translation unit under csrc/ and every header there that it includes,
+    directly or through another."""
+    d = os.path.join(ROOT, "paper_2601_16791_gb300", "csrc")
+    out = [unit]
+    for f in out:
+        for m in re.findall(r'^\s*#include "([^"]+)"', open(os.path.join(d, f)).read(), re.M):
+            if m not in out and os.path.exists(os.path.join(d, m)):
+                out.append(m)
+    return [unit] + sorted(out[1:])
+
+
+KERNEL_SOURCES = {k: unit_sources(u) for k, u in
+                  (("k_jump_kick", "k_kick.cu"), ("k_jump_drift", "k_drift.cu"),
+                   ("k_detect", "k_detect.cu"), ("k_bs", "k_bs.cu"), ("k_catchup", "k_bs.cu"))}
 
 
 def dram_traffic(kname):
