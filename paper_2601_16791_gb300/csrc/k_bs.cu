@@ -1999,7 +1999,12 @@ __device__ void catch_record(const Dev& d, const CatchArgs& a, int bank, int idx
 // A cluster of two CTAs per deferred body, on two SMs: both replay the body
 // alike (only rank 0 writes), and in a two-body group's Bulirsch-Stoer rounds
 // rank 0 tries H and rank 1 tries H/2 (bs2c_rounds with a ClusterMail).
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(128) k_catchup(Dev d, CatchArgs a) {
+// Two blocks an SM by launch bounds: without them ptxas aims at three, with 168
+// registers and 408 bytes of spill loads in the chains that set the launch's
+// time, and the third block takes registers from the main stream's kernels
+// beside it.  4 cores + 100,000: 0.201 -> 0.191 ms a step over 400 steps, 0.227
+// -> 0.207 over 20 (220 registers, no spills).
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(128, 2) k_catchup(Dev d, CatchArgs a) {
   namespace cg = cooperative_groups;
   cg::cluster_group cl = cg::this_cluster();
   __shared__ int s_row[4], s_r;
