@@ -141,9 +141,9 @@ __device__ int run_members(const unsigned long long* keys, int p, int n, const i
 constexpr int kGroupKeysSmem = 2048;   // 16 KB of static shared memory
 
 // The encounter groups of the step from its pair keys, in one block of any
-// size (a multiple of 32, at most 1024): big groups by union-find over the
-// big-big pairs, then one test-particle group per run of keys with the same
-// planetesimal, in key order.
+// size (a multiple of 32, at most 1024): big groups as the components of the
+// big-big pairs, by spreading each one's smallest body, then one test-particle
+// group per run of keys with the same planetesimal, in key order.
 __device__ __forceinline__ void groups_block(const Dev& d) {
   __shared__ int nodes[2 * kMaxBigPairs];
   __shared__ int parent[2 * kMaxBigPairs];
@@ -167,7 +167,7 @@ __device__ __forceinline__ void groups_block(const Dev& d) {
   if (threadIdx.x == 0) {
     s_nbb = 0;
     s_bad = 0;
-    s_slot = d.defer ? *d.hstep : 0;   // read early, used by thread 0 below
+    s_slot = d.defer ? *d.hstep : 0;   // read early, used with the big groups' history
   }
   __syncthreads();
   for (int p = threadIdx.x; p < n; p += blockDim.x) {
@@ -186,8 +186,8 @@ __device__ __forceinline__ void groups_block(const Dev& d) {
   }
   // ---- big groups: the connected components of the (few) big-big pairs.
   // Every step on all threads, each counting over the shared lists (one thread
-  // with a union-find took most of 177 us for the 130 big-big pairs of 2,000
-  // big bodies + 200,000 planetesimals; now 50).  comp_nodes holds the
+  // with a union-find took most of the launch's 177 us for 2,000 big bodies +
+  // 200,000 planetesimals, about 30 big-big pairs among 5,700; now 47).  comp_nodes holds the
   // pairs' entries while the sorted list of distinct bodies is made.
   if (nbb == 0) {   // the common case of a few big bodies
     if (threadIdx.x == 0) s_nnodes = s_bw = s_bm = 0;
@@ -379,8 +379,8 @@ constexpr int kDeferRow = 3;
 // chain of FP64 instructions of one warp, 64 cycles each: about 50 to 65 a
 // force evaluation here, where every lane carried all bodies (150 to 290, all
 // 17 evaluations of a macro sub-step, four groups a warp).  Measured: four
-// steps of 301 big bodies + 20,011 planetesimals 1.157 -> 0.939 ms; twenty of 4
-// cores + 100,000, whose catch-up runs it too, 8.2 -> 7.4 ms.
+// steps of 301 big bodies + 20,011 planetesimals 1.157 -> 0.939 ms; no change
+// in twenty of 4 cores + 100,000, where groups of three are rare.
 // Returns 1 when the step is done, 0 when rounds ran out, -1 at the cap.
 template <int NB>
 __device__ int bsn_rounds(int lane, double mu0, const double* mu, const MemberK* K, double tol,
@@ -1535,9 +1535,8 @@ __device__ __noinline__ void catch_bs_thread(const Dev& d, const SysDev& S, cons
   for (int q = 0; q < 6; ++q) out[q] = Y[q][nb - 1];
 }
 
-// The drift of a light system's body.  Out of line, as catch_kick_light is: the
-// catch-up of systems with cores, whose hardest chains set its time, then keeps
-// its registers (k_catchup spilled 508 bytes of loads with both inline).
+// The drift of a light system's body, out of line as catch_kick_light is
+// (k_catchup spilled 508 bytes of loads with both inline).
 static __device__ __noinline__ bool catch_drift_light(double mu, double h, int maxit, double* q) {
   return kepler_drift_sel(true, mu, h, maxit, q[0], q[1], q[2], q[3], q[4], q[5]);
 }

@@ -3,10 +3,11 @@
 // min(d0, d1, d2min) <= rc^2, rc = max(rcrit_i, rcrit_j)).
 //
 // One thread per target body against the big bodies of its system, staged in
-// shared memory with FP64 endpoint states and FP32 copies.  A provably
-// conservative FP32 screen discards far pairs (mx_encounter.cuh); surviving
-// pairs are decided in FP64 with the closed-form minimum of the cubic Hermite
-// interpolant of the squared separation.
+// shared memory as FP32 copies of the endpoint states (with fewer than
+// kDetMinScreen of them, the FP64 states too).  Two provably conservative FP32
+// screens discard far pairs (mx_encounter.cuh; the first, by reach, from
+// kDetMinScreen big bodies on); surviving pairs are decided in FP64 with the
+// closed-form minimum of the cubic Hermite interpolant of the squared separation.
 // Each target keeps its flagged big bodies (ascending) and writes them as one
 // contiguous run, with one atomic per warp; runs of different targets come in
 // any order.  The step groups runs as they are; callers that want the pairs
@@ -33,9 +34,10 @@ __device__ __forceinline__ unsigned long long swapped(unsigned long long k) {
 
 // Ranks of up to kRankMax keys, all SMs together: a key's place is the number
 // of smaller ones (the keys are distinct pairs), counted by eight lanes.  The
-// n^2 compares of 5,500 keys (2,000 big bodies + 200,000 planetesimals) take
-// 39 us where one block's bitonic sort took 120; beyond kRankMax the sort's
-// n log^2 n wins (16,384 keys: 2.7e8 compares, about 40 us).
+// n^2 compares of 5,500 keys (2,000 big bodies + 200,000 planetesimals) and the
+// copy back take 44 + 6 us, where one block's bitonic sort takes 120; 1,000 keys
+// 13 + 3 against 14, 16,384 keys 189 + 11 against 250.  kRankMax is the size of
+// the scratch; the sort beyond it runs in global memory (16,385 keys: 960 us).
 constexpr int kRankMax = kSortTmp;
 __global__ void __launch_bounds__(256) k_rank_keys(const unsigned long long* keys, const int* count,
                                                    int cap, int swap_ij, unsigned long long* out) {

@@ -13,7 +13,7 @@
 // fd = -(m/h) U1/rho, rho = r/r0 = 1 + a U1 + c U2.  About 77 FP64
 // instructions.  Against 64-bit-mantissa arithmetic over 20,000 orbits (1 to 15
 // AU, h = 10 d): position 5.7e-17 rms (kepler_drift 5.7e-17), velocity 6.8e-17
-// (7.6e-17).  Measured: mx_kepler_drift of 200,000 bodies 74.5 -> 59.6 us a call;
+// (7.6e-17).  Measured: mx_kepler_drift of 200,000 bodies 75.4 -> 55.4 us a call;
 // k_jump_drift of 64 disks with 2.4 million bodies 481 -> 375 us a launch, three
 // steps of them 4.1 -> 3.7 ms.
 #pragma once

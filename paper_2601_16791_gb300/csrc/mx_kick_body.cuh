@@ -488,7 +488,7 @@ __device__ __forceinline__ FusedPrep fused_prep(const Dev& d, const SysDev& S, c
 // (measured on the gas disk and the semi-active disk).  `bid` is the tile,
 // `dsm` the block's dynamic shared memory (kick_smem_bytes).
 // MODE (kSplitNone, kSplitFew, kSplitAny): which of the two kicks the batch's
-// systems need, FP64 (kick_fp64) or FP32 pairs (kick_split_tile), and whether
+// systems need, FP64 (gravity_all) or FP32 pairs (gravity_split), and whether
 // some system may have more than kDeferMaxBig big bodies.
 template <int NKICK, bool FUSED, int MODE>
 __device__ __forceinline__ void jump_kick_tile(const Dev& d, double jump_frac, double kick_frac,

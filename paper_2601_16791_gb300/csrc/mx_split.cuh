@@ -22,10 +22,11 @@
 // FP32 parts instead (below).
 //
 // Measured: k_jump_kick with 2,000 big bodies and 200,000 planetesimals 11.8 ->
-// 1.65 ms a launch (34 -> 245 G pairs/s); 301 big bodies and 20,011
-// planetesimals 0.43 -> 0.068 ms a launch.  64 gas
-// disks of 2 to 50 light bodies (2.4 million bodies; with the drag, see
-// mx_split_gas.cuh) 2.35 -> 0.45 ms a launch, three steps 12.0 -> 4.34 ms.
+// 1.61 ms a launch (34 -> 251 G pairs/s, 84% of the issue slots filled); 301 big
+// bodies and 20,011 planetesimals 0.43 -> 0.05 ms a launch.  64 gas disks of 2
+// to 50 light bodies (2.4 million bodies; with the drag, see mx_split_gas.cuh)
+// 2.35 -> 0.41 ms a launch, three steps (with the drift's short form) 12.0 ->
+// 3.7 ms.
 //
 // Positions: each coordinate is cut on one grid for target and sources into
 // three FP32 parts, x = x0 + x1 + x2 with x0 a multiple of 2^(k-23), x1 of
@@ -310,8 +311,8 @@ __device__ __forceinline__ void split_flush(SplitAcc& acc, double& ax, double& a
 // whole separation, 2^-54 of it by coordinate at the least; what is left of the
 // sum's is its FP64 adds, one in kSplitSeg.  About 340 FP32 instructions a pair
 // against pair_acc's 17 of 64 cycles.  Measured: k_accel with 2,000 big bodies
-// and 200,000 planetesimals 11.8 -> 4.57 ms (87% of the issue slots filled), and the
-// result's error against a 64-bit sum over all pairs 1.5e-15 -> 6.5e-16.
+// and 200,000 planetesimals 11.8 -> 4.51 ms (86% of the issue slots filled), and the
+// result's error against a 64-bit sum over all pairs 1.6e-15 -> 5.7e-16.
 struct FT {
   float h, m, l;
 };
